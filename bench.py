@@ -15,8 +15,8 @@ Also reported on the same JSON line:
                 (pinned b copied in and x copied out every step)
   roofline      the dominant kernel (the fused CG operator kernel) timed with
                 CUDA events on libsem's stream: against HBM bandwidth when the
-                tuner picked the double-word operator (FP64 values evaluated
-                in FP32 pairs), against the FP64 pipe for the DFMA kernels
+                tuner picked the fixed-point operator (FP64 values evaluated
+                as 64-bit integers), against the FP64 pipe for the DFMA kernels
   mixed         the same solve by mixed-precision iterative refinement (FP32
                 inner CG, BF16 geometric factors, FP64 outer residual), with
                 its own HBM roofline, solves/s against FP64, and a 1e-10 leg
@@ -59,19 +59,19 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic.json")
 AX_SOURCES = [os.path.join(ROOT, "paper_2606_12650_gb300", "csrc", f)
               for f in ("sem_ax_kernel.cuh", "sem_ax_lines.cuh", "sem_ax.cu", "sem_ax_lines64.cu", "sem_device.cuh",
-                        "sem_internal.h", "sem_ax_dw.cuh", "sem_ax_dw.cu", "sem_dw.cuh")]
+                        "sem_internal.h", "sem_ax_fx.cuh", "sem_ax_fx.cu")]
 GOLDEN_SMALL = os.path.join(ROOT, "tests", "golden", "oracle_cg_E64_N7.npz")
 AX32_SOURCES = [os.path.join(ROOT, "paper_2606_12650_gb300", "csrc", f)
                 for f in ("sem_ax_kernel.cuh", "sem_ax_lines.cuh", "sem_ax32.cu", "sem_ax_lines32.cu", "sem_ax32p.cuh",
                           "sem_device.cuh", "sem_internal.h")]
-VARIANTS = {0: "columns", 1: "lines", 2: "persistent", 3: "lines_prefetch", 4: "lines_staged", 5: "lines_dw"}
+VARIANTS = {0: "columns", 1: "lines", 2: "persistent", 3: "lines_prefetch", 4: "lines_staged", 5: "lines_fx"}
 
 
 def kernel_label(variant, epb, N, t, gt):
     """Name of the CG-operator kernel the tuner chose."""
     q = N + 1
     if variant == 5:
-        return f"ax_dw_kernel<{q},CG> ({epb} elements/block, FP64 in double-word FP32 arithmetic)"
+        return f"ax_fx_kernel<{q},CG> ({epb} elements/block, FP64 in 64-bit fixed point)"
     if variant in (1, 3, 4):
         pf = {1: "", 3: ", G prefetched", 4: ", G staged"}[variant]
         return f"ax_lines_kernel<{q},{t},{gt},CG> ({epb} elements/block{pf})"
@@ -403,19 +403,19 @@ def run_ours(a):
     hbm, hbm_how = hbm_peak()
     gbs = bytes_alg / (ax_ms * 1e-3) / 1e9
     if v64 == 5:
-        # double-word arithmetic on the FP32 pipe: the FP64 pipe no longer
+        # 64-bit fixed-point arithmetic on the integer multiplier: the FP64 pipe no longer
         # bounds the kernel; HBM bandwidth is its roofline
         roofline = {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
                     "traffic": traffic, "kernel": kernel_label(v64, e64, N, "double", "double"),
                     "launch_ms": ax_ms, "alg_bytes_per_launch": bytes_alg,
                     "alg_bytes_note": "96 B per local node: r, p, x read; p, w, x written (x: the deferred "
-                                      "update); 6 geometric factors of 8 B (FP64, or their double-word FP32 "
-                                      "pairs, the same 48 B)",
+                                      "update); 6 geometric factors of 8 B (as 64-bit integers with one "
+                                      "scale per element)",
                     "peak_source": hbm_how,
                     "fp64_equiv_gflops": achieved, "fp64_pipe_peak_gflops": FP64_PEAK_GFLOPS,
                     "fp64_equiv_note": "the operator's direct-evaluation flops, 12(N+1)^4 + 15(N+1)^3 per "
                                        "element, per second: above the FP64 pipe's peak because the kernel "
-                                       "computes in FP32 pairs (~48-bit significands) on the FP32 pipe"}
+                                       "computes in 64-bit fixed point on the integer multiply-add pipe"}
     else:
         roofline = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_GFLOPS, "unit": "GFLOP/s",
                     "frac": achieved / FP64_PEAK_GFLOPS, "traffic": traffic,
@@ -536,7 +536,7 @@ def run_ours(a):
                 "warmup": a.warmup, "ms_per_step": t_max / a.steps, "higher_is_better": True,
                 "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
                 "dtype_note": ("FP64 vectors, recurrences and reductions; the operator kernel the tuner chose "
-                               + ("evaluates in double-word FP32 (~48-bit significands)" if v64 == 5
+                               + ("evaluates in 64-bit fixed point (one scale per element)" if v64 == 5
                                   else "evaluates in FP64")),
                 "config": config_of(a, world, iters_total // max(a.steps, 1)),
                 "autotune": tune, "paper_sweep": sweep_paper, "batched": batched, "serve": served,

@@ -2,7 +2,7 @@
 // instantiations (sem_ax_kernel.cuh) -- plain y = A_local x, the CG variant
 // with the fused p-update and <p, A p> reduction, the Jacobi-PCG variant --
 // and the dispatch to the variant the per-order tuner chose (the line kernel
-// lives in sem_ax_lines64.cu, its double-word form in sem_ax_dw.cu).
+// lives in sem_ax_lines64.cu, its fixed-point form in sem_ax_fx.cu).
 #include "sem_ax_kernel.cuh"
 
 namespace sem {
@@ -10,26 +10,26 @@ namespace sem {
 int prepare_ax(const Problem *Pb) { return prepare_ax_any<double, double>(Pb); }
 
 int prepare_f64_variant(Problem *P) {
-    return tune_get(kTuneF64, P->nq).variant == kAxLinesDW ? dw_prepare(P) : SEM_OK;
+    return tune_get(kTuneF64, P->nq).variant == kAxLinesFX ? fx_prepare(P) : SEM_OK;
 }
 
-// The double-word variant's factors: made on first use outside a capture
+// The fixed-point variant's factors: made on first use outside a capture
 // (solves prepare them before capturing their graphs).
-static int ensure_dw(const Problem *Pb) {
-    if (Pb->Gdw) return SEM_OK;
+static int ensure_fx(const Problem *Pb) {
+    if (Pb->Gfx) return SEM_OK;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    const int rc = cuda_check(cudaStreamIsCapturing(stream(), &cs), "ax dw: capture status");
+    const int rc = cuda_check(cudaStreamIsCapturing(stream(), &cs), "ax fx: capture status");
     if (rc != SEM_OK) return rc;
     if (cs != cudaStreamCaptureStatusNone)
-        return set_error(SEM_EARG, "ax dw: double-word factors must be prepared before a capture");
-    return dw_prepare(const_cast<Problem *>(Pb));
+        return set_error(SEM_EARG, "ax fx: integer factors must be prepared before a capture");
+    return fx_prepare(const_cast<Problem *>(Pb));
 }
 
 int launch_ax(const Problem *Pb, const double *x, double *y) {
     const TuneChoice c = tune_get(kTuneF64, Pb->nq);
-    if (c.variant == kAxLinesDW) {
-        const int rc = ensure_dw(Pb);
-        return rc != SEM_OK ? rc : launch_lines_dw(Pb, x, y, 0, c.epb);
+    if (c.variant == kAxLinesFX) {
+        const int rc = ensure_fx(Pb);
+        return rc != SEM_OK ? rc : launch_lines_fx(Pb, x, y, 0, c.epb);
     }
     if (c.variant == kAxLines) return launch_lines64(Pb, x, y, 0, c.epb);
     AxArgs<double, double> a = ax_args<double, double>(Pb, Pb->G, Pb->partials, Pb->st);
@@ -40,9 +40,9 @@ int launch_ax(const Problem *Pb, const double *x, double *y) {
 
 int launch_ax_cg(const Problem *Pb) {
     const TuneChoice c = tune_get(kTuneF64, Pb->nq);
-    if (c.variant == kAxLinesDW) {
-        const int rc = ensure_dw(Pb);
-        return rc != SEM_OK ? rc : launch_lines_dw(Pb, nullptr, nullptr, 1, c.epb);
+    if (c.variant == kAxLinesFX) {
+        const int rc = ensure_fx(Pb);
+        return rc != SEM_OK ? rc : launch_lines_fx(Pb, nullptr, nullptr, 1, c.epb);
     }
     if (c.variant == kAxLines) return launch_lines64(Pb, nullptr, nullptr, 1, c.epb);
     AxArgs<double, double> a = ax_args<double, double>(Pb, Pb->G, Pb->partials, Pb->st);
@@ -55,9 +55,9 @@ int launch_ax_cg(const Problem *Pb) {
 
 int launch_ax_pcg(const Problem *Pb) {
     const TuneChoice c = tune_get(kTuneF64, Pb->nq);
-    if (c.variant == kAxLinesDW) {
-        const int rc = ensure_dw(Pb);
-        return rc != SEM_OK ? rc : launch_lines_dw(Pb, nullptr, nullptr, 2, c.epb);
+    if (c.variant == kAxLinesFX) {
+        const int rc = ensure_fx(Pb);
+        return rc != SEM_OK ? rc : launch_lines_fx(Pb, nullptr, nullptr, 2, c.epb);
     }
     if (c.variant == kAxLines) return launch_lines64(Pb, nullptr, nullptr, 2, c.epb);
     AxArgs<double, double> a = ax_args<double, double>(Pb, Pb->G, Pb->partials, Pb->st);

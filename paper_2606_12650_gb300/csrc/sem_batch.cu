@@ -11,8 +11,8 @@
 // its own kernel, compiled for that order and body with the body inlined;
 // the vector kernel switches on N on the device.  The operator body and the
 // elements per pass follow the per-order tuner's table for the batch's
-// precision: the line body (sem_ax_lines.cuh), in double-word arithmetic for
-// FP64 batches where the table chose that variant (sem_ax_dw.cuh), or the
+// precision: the line body (sem_ax_lines.cuh), in fixed-point arithmetic for
+// FP64 batches where the table chose that variant (sem_ax_fx.cuh), or the
 // column body, passes of 256 / (N+1)^2 elements.  Items of problems whose
 // solve finished are dropped from the lists between rounds (the items of one
 // problem stay together and in order, so its reductions never change).
@@ -42,7 +42,7 @@
 #include <type_traits>
 #include <vector>
 
-#include "sem_ax_dw.cuh"
+#include "sem_ax_fx.cuh"
 #include "sem_box.cuh"
 #include "sem_device.cuh"
 #include "sem_internal.h"
@@ -58,7 +58,8 @@ struct BatchProb {
     BoxDims bd;                     // the box with its fast divisors
     int64_t E, nL;
     const double *G;
-    const float *Gdw;               // double-word factors (FP64 batches with the double-word body)
+    const int4 *Gfx;                // integer factors and their scales (FP64 batches with the
+    const int32_t *kgfx;            // fixed-point body)
     const __nv_bfloat16 *G16;
     const float *G32;
     double *x, *r, *p, *w;          // FP64 CG vectors / refinement x, r
@@ -82,7 +83,6 @@ struct BatchItem {
     int64_t first;  // first element (operator) or first local node (vector)
     int count;      // elements or nodes
     int group;      // operator items: elements per pass of the line body; 0 = column body
-    int dw;         // operator items of FP64 batches: the line body in double-word arithmetic
 };
 
 struct BatchQueue {
@@ -92,7 +92,7 @@ struct BatchQueue {
 enum BatchQ : int { kQAx = 0, kQVec = 1, kNumQ = 2 };
 
 // Operator bodies of a batch: every member of one order takes the same one.
-enum AxBody : int { kBodyColumns = 0, kBodyLines = 1, kBodyDW = 2, kBodyNone = -1 };
+enum AxBody : int { kBodyColumns = 0, kBodyLines = 1, kBodyFX = 2, kBodyNone = -1 };
 constexpr int kOrders = kMaxQ - 1;  // N+1 = 2 .. kMaxQ
 
 struct BatchCtl {
@@ -162,12 +162,12 @@ struct BEpb {
 };
 
 // Dynamic shared memory of one order's operator body: the column body's
-// slabs, or the line body's three regions (FP64-sized for the double-word
-// body, whose values are FP32 pairs).
+// slabs, or the line body's three regions, or the fixed-point body's.
 template <int NQ, typename T, int BODY>
 inline size_t batch_ax_smem() {
     return BODY == kBodyColumns ? AxShape<NQ, BEpb<NQ>::value, T>::SMEM
-                                : LineShape::smem(NQ, BEpb<NQ>::value, BODY == kBodyDW ? 8 : int(sizeof(T)));
+           : BODY == kBodyFX    ? 16 + fx_smem<NQ>(BEpb<NQ>::value)
+                                : LineShape::smem(NQ, BEpb<NQ>::value, int(sizeof(T)));
 }
 
 // Derivative matrices of every order in constant memory: D depends only on
@@ -178,7 +178,7 @@ __constant__ float c_D32[kMaxQ - 1][kMaxQ * kMaxQ];
 // even-odd coefficients of D ([0]) and D^T ([1]) for the line body
 __constant__ EoMat<double> c_E64[kMaxQ - 1][2];
 __constant__ EoMat<float> c_E32[kMaxQ - 1][2];
-__constant__ EoMatDW c_EDW[kMaxQ - 1][2];
+__constant__ EoMatFX c_EFX[kMaxQ - 1][2];
 
 template <typename T>
 __device__ __forceinline__ const EoMat<T> &const_eo(int nq, int which);
@@ -299,25 +299,20 @@ __device__ __forceinline__ bool batch_lines_item(const T *xin, T *yout, T *pv, c
     return true;
 }
 
-// The double-word line body (FP64 batches): same passes as batch_lines_item.
+// The fixed-point line body (FP64 batches): same passes as batch_lines_item.
 template <int NQ, bool CG>
-__device__ __forceinline__ bool batch_dw_item(const double *xin, double *yout, double *pv, const float *Gdw, double beta,
-                                           int64_t first, int count, int group, double *regA, uint64_t *bar,
-                                           uint32_t *phase, int32_t *status, double *pt) {
+__device__ __forceinline__ void batch_fx_item(const double *xin, double *yout, double *pv, const int4 *Gfx,
+                                              const int32_t *kg, double beta, int64_t first, int count, int group,
+                                              unsigned char *smem, double *pt) {
     double acc = 0.0;
     for (int g = 0; g < count; g += group) {
         double part = 0.0;
-        const bool ok = lines_group_dw<NQ, CG, false>(xin, yout, pv, Gdw, c_EDW[NQ - 2][0], c_EDW[NQ - 2][1], beta,
-                                                      0.0, nullptr, nullptr, first + g, min(group, count - g), group,
-                                                      regA, bar, *phase, status, &part);
-        *phase ^= 1u;
-        if (!ok) return false;
+        lines_group_fx<NQ, CG, false>(xin, yout, pv, Gfx, kg, c_EFX[NQ - 2][0], c_EFX[NQ - 2][1], beta, 0.0, nullptr,
+                                      nullptr, first + g, min(group, count - g), group, smem, &part);
         acc += part;
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
     }
     *pt = acc;
-    return true;
 }
 
 // mode: 0 = FP64 CG (p = r + beta p, w = A p), 1 = FP64 plain (w = A x),
@@ -330,7 +325,7 @@ __global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 4 ? 4 : 2)
     batch_ax_kernel(BatchProb *probs, const BatchItem *items, double *part, uint32_t *tickets, BatchCtl *ctl,
                     int32_t *status) {
     constexpr bool CG = MODE != 1;
-    static_assert(BODY != kBodyDW || std::is_same<T, double>::value, "the double-word body is FP64");
+    static_assert(BODY != kBodyFX || std::is_same<T, double>::value, "the fixed-point body is FP64");
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double red[32];
     __shared__ int s_item;
@@ -358,10 +353,10 @@ __global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 4 ? 4 : 2)
         else if (MODE == 1) { xin = reinterpret_cast<const T *>(P.x); yout = reinterpret_cast<T *>(P.w); pv = nullptr; }
         else { xin = reinterpret_cast<const T *>(P.r32); yout = reinterpret_cast<T *>(P.w32); pv = reinterpret_cast<T *>(P.p32); }
         T pt = T(0);
-        bool ok;
-        if constexpr (BODY == kBodyDW)
-            ok = batch_dw_item<NQ, CG>(xin, yout, pv, P.Gdw, beta, item.first, item.count, item.group, regA, bar,
-                                       &phase, status, &pt);
+        bool ok = true;
+        if constexpr (BODY == kBodyFX)
+            batch_fx_item<NQ, CG>(xin, yout, pv, P.Gfx, P.kgfx, beta, item.first, item.count, item.group, smem + 16,
+                                  &pt);
         else if constexpr (BODY == kBodyLines)
             ok = batch_lines_item<NQ, T, GT, CG>(xin, yout, pv, prob_G<GT>(P), beta, item.first, item.count,
                                                  item.group, regA, bar, &phase, status, &pt);
@@ -670,7 +665,7 @@ struct BaxLaunch {
 };
 
 // Dispatch on the order and body (prepare only, or launch for `count`
-// items).  The double-word body exists for FP64 CG batches only.
+// items).  The fixed-point body exists for FP64 CG batches only.
 template <typename T, typename GT, int MODE, int NQ>
 static int bax_order(Batch *B, int body, int count, bool launch, int *res) {
     int r = 0;
@@ -682,10 +677,10 @@ static int bax_order(Batch *B, int body, int count, bool launch, int *res) {
         case kBodyLines:
             return launch ? BaxLaunch<T, GT, MODE, NQ, kBodyLines>::launch(B, count)
                           : BaxLaunch<T, GT, MODE, NQ, kBodyLines>::resident(res);
-        case kBodyDW:
+        case kBodyFX:
             if constexpr (MODE == 0)
-                return launch ? BaxLaunch<T, GT, MODE, NQ, kBodyDW>::launch(B, count)
-                              : BaxLaunch<T, GT, MODE, NQ, kBodyDW>::resident(res);
+                return launch ? BaxLaunch<T, GT, MODE, NQ, kBodyFX>::launch(B, count)
+                              : BaxLaunch<T, GT, MODE, NQ, kBodyFX>::resident(res);
             [[fallthrough]];
         default: return set_error(SEM_EARG, "batch: no such operator body for this precision");
     }
@@ -857,7 +852,7 @@ static int batch_attrs(Batch *B) {
         }
         static EoMat<double> e64[kMaxQ - 1][2];
         static EoMat<float> e32[kMaxQ - 1][2];
-        static EoMatDW edw[kMaxQ - 1][2];
+        static EoMatFX efx[kMaxQ - 1][2];
         for (int N = 1; N <= kMaxQ - 1; ++N) {
             const int nq = N + 1;
             double Dt[kMaxQ * kMaxQ];
@@ -867,14 +862,13 @@ static int batch_attrs(Batch *B) {
             e64[N - 1][1] = eo_coefficients<double>(Dt, nq);
             e32[N - 1][0] = eo_coefficients<float>(h64[N - 1], nq);
             e32[N - 1][1] = eo_coefficients<float>(Dt, nq);
-            edw[N - 1][0] = eo_coefficients_dw(h64[N - 1], nq);
-            edw[N - 1][1] = eo_coefficients_dw(Dt, nq);
+            fx_coefficients(h64[N - 1], nq, &efx[N - 1][0], &efx[N - 1][1]);
         }
         int rc = cuda_check(cudaMemcpyToSymbol(c_D64, h64, sizeof h64), "batch: D table");
         if (rc == SEM_OK) rc = cuda_check(cudaMemcpyToSymbol(c_D32, h32, sizeof h32), "batch: D table");
         if (rc == SEM_OK) rc = cuda_check(cudaMemcpyToSymbol(c_E64, e64, sizeof e64), "batch: even-odd table");
         if (rc == SEM_OK) rc = cuda_check(cudaMemcpyToSymbol(c_E32, e32, sizeof e32), "batch: even-odd table");
-        if (rc == SEM_OK) rc = cuda_check(cudaMemcpyToSymbol(c_EDW, edw, sizeof edw), "batch: even-odd table");
+        if (rc == SEM_OK) rc = cuda_check(cudaMemcpyToSymbol(c_EFX, efx, sizeof efx), "batch: even-odd table");
         if (rc != SEM_OK) return rc;
         done = true;
     }
@@ -1075,22 +1069,23 @@ int batch_set(Batch *B, Problem **probs, const double *const *b, const uint8_t *
         // item holds several passes (~kAxItemNodes local nodes)
         const int full = kBatchThreads / (P->nq * P->nq);
         const TuneChoice c = tune_get(B->mode == 0 ? kTuneF64 : (B->mode == 1 ? kTuneF32G16 : kTuneF32G32), P->nq);
-        // the double-word variant: its line body in FP64 batches (factors
+        // the fixed-point variant: its line body in FP64 batches (factors
         // made here, before any capture); mixed batches (whose FP64 operator
         // runs only for the refinement residual) keep the FP64 line body
-        const bool dw = B->mode == 0 && c.variant == kAxLinesDW;
-        if (dw) {
-            rc = dw_prepare(P);
+        const bool fx = B->mode == 0 && c.variant == kAxLinesFX;
+        if (fx) {
+            rc = fx_prepare(P);
             if (rc != SEM_OK) break;
-            q.Gdw = P->Gdw;
+            q.Gfx = P->Gfx;
+            q.kgfx = P->kgfx;
         }
         const bool lines = c.variant == kAxLines || c.variant == kAxLinesPrefetch || c.variant == kAxLinesStaged ||
-                           c.variant == kAxLinesDW;
+                           c.variant == kAxLinesFX;
         const int group = full;
         const int np = P->nq * P->nq * P->nq;
         const int per_item = group * std::max(1, kAxItemNodes / (np * group));
         const int o = P->nq - 2;
-        const int body = dw ? kBodyDW : (lines ? kBodyLines : kBodyColumns);
+        const int body = fx ? kBodyFX : (lines ? kBodyLines : kBodyColumns);
         if (ord_body[o] != kBodyNone && ord_body[o] != body) {
             rc = set_error(SEM_EARG, "batch: members of one order with different operator bodies");
             break;
@@ -1099,8 +1094,7 @@ int batch_set(Batch *B, Problem **probs, const double *const *b, const uint8_t *
         std::vector<BatchItem> &oa = by_ord[o];
         q.ax_first = int(oa.size());   // within its order's items; placed below
         for (int64_t e = 0; e < P->E; e += per_item)
-            oa.push_back(BatchItem{k, P->nq, e, int(std::min<int64_t>(per_item, P->E - e)), lines ? group : 0,
-                                   dw ? 1 : 0});
+            oa.push_back(BatchItem{k, P->nq, e, int(std::min<int64_t>(per_item, P->E - e)), lines ? group : 0});
         q.ax_count = int(oa.size()) - q.ax_first;
         const int64_t chunk = std::max<int64_t>(P->nq, (kVecItemNodes / P->nq) * P->nq);
         std::vector<BatchItem> &ov = by_ord_v[o];

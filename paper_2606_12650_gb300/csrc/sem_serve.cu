@@ -80,13 +80,13 @@ double serve_now(const Server *S) {
 // Device bytes a request holds from admission until its result is fetched,
 // from the node count: FP64 geometry (48), mass (8), CG vectors (32),
 // right-hand side (8) and the retired result (8) per node, plus for FP64 the
-// double-word copy of the factors (48; counted whichever operator body the
-// tuner picked), for mixed precision BF16/FP32 factors (12 or 24) and FP32
+// integer copy of the factors (48, and a scale of 4 per element; counted
+// whichever operator body the tuner picked), for mixed precision BF16/FP32 factors (12 or 24) and FP32
 // inner vectors (16); and per problem its reduction partials, two CG states
 // and the vertex copy, plus 64 KB of allocation granularity.
 static size_t request_bytes(int mode, int nx, int ny, int nz, int64_t nL) {
     size_t per = 48 + 8 + 32 + 8 + 8;
-    if (mode == 0) per += 48;   // the double-word copy of G (FP64 batches' double-word body)
+    if (mode == 0) per += 48 + 1;   // the integer copy of G and its scales (FP64 batches' fixed-point body)
     if (mode == 1) per += 12 + 16;
     if (mode == 2) per += 24 + 16;
     const int64_t n_verts = int64_t(nx + 1) * (ny + 1) * (nz + 1);

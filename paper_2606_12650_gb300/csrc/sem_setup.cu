@@ -465,7 +465,7 @@ void problem_destroy(Problem *P) {
     if (P->dinv) dev_free(P->dinv);
     if (P->bad_dev) dev_free(P->bad_dev);
     mixed_release(P);
-    dw_release(P);
+    fx_release(P);
     if (P->partials) dev_free(reinterpret_cast<unsigned char *>(P->partials) - 16);
     double *dptrs[] = {P->verts, P->G, P->B, P->c, P->x, P->r, P->p, P->w};
     for (double *q : dptrs)

@@ -6,7 +6,7 @@
 // every order and the choice is made by timing: for one order and one
 // precision, each candidate -- the column kernel, the persistent kernel
 // (FP32), the line kernel at several element-per-block counts, and for FP64
-// the line kernel in double-word FP32 arithmetic -- runs
+// the line kernel in fixed-point arithmetic -- runs
 // the CG operator `reps` times on a real problem, and the fastest is kept.
 // The table can be saved to and loaded from a text file (one line per entry:
 // kind, N, variant, elements per block, microseconds), so a tuned table is
@@ -32,7 +32,7 @@ uint64_t g_epoch = 1;
 // nodes per problem (E = 129^3 at N = 1 down to 26^3 at N = 9; CG operator,
 // 10 launches per candidate), as {variant, elements per block} indexed by
 // N + 1 (entries 0 and 1 unused); the run-time tuner replaces entries for
-// the problems at hand.  FP64: the double-word line kernel at every order
+// the problems at hand.  FP64: the fixed-point line kernel at every order
 // (e.g. N = 3: 281 us against 1203 us for the DFMA line kernel; N = 7: 371
 // against 1579; N = 9: 576 against 2117).
 struct DefaultEntry {
@@ -40,7 +40,7 @@ struct DefaultEntry {
 };
 constexpr DefaultEntry kDefault[kTuneKinds][kMaxQ + 1] = {
     // FP64
-    {{0, 0}, {0, 0}, {5, 32}, {5, 14}, {5, 8}, {5, 5}, {5, 7}, {5, 5}, {5, 4}, {5, 3}, {5, 5}},
+    {{0, 0}, {0, 0}, {5, 32}, {5, 14}, {5, 8}, {5, 5}, {5, 3}, {5, 5}, {5, 1}, {5, 1}, {5, 1}},
     // FP32, FP32 factors
     {{2, 0}, {2, 0}, {2, 0}, {2, 0}, {2, 0}, {1, 10}, {1, 10}, {1, 5}, {1, 3}, {1, 3}, {1, 2}},
     // FP32, BF16 factors
@@ -70,20 +70,20 @@ bool choice_ok(int kind, int nq, const TuneChoice &c) {
         case kAxLinesPrefetch: return kind == kTuneF32G16 && lines_epb_ok(nq, c.epb, elem_bytes(kind));
         case kAxLinesStaged:
             return kind != kTuneF64 && lines_epb_ok(nq, c.epb, elem_bytes(kind), kind == kTuneF32G32 ? 24 : 12);
-        case kAxLinesDW: return kind == kTuneF64 && lines_epb_ok(nq, c.epb, sizeof(double));
+        case kAxLinesFX: return kind == kTuneF64 && lines_epb_ok(nq, c.epb, sizeof(double));
         default: return false;
     }
 }
 
 // The candidates for (kind, nq): the kind's column kernel, then the line
-// kernel with ~64 .. 512 threads per block (for FP64 also in double-word
+// kernel with ~64 .. 512 threads per block (for FP64 also in fixed-point
 // arithmetic; for FP32 with staged factors and, for BF16 factors, with the
 // factors prefetched).
 int candidates(int kind, int nq, TuneChoice *out, int cap) {
     int n = 0;
     out[n++] = {kind == kTuneF64 ? kAxColumns : kAxPersistent, 0, 0.0};
     const bool f64 = kind == kTuneF64;
-    const int variants[3] = {kAxLines, f64 ? kAxLinesDW : kAxLinesStaged, kAxLinesPrefetch};
+    const int variants[3] = {kAxLines, f64 ? kAxLinesFX : kAxLinesStaged, kAxLinesPrefetch};
     const int nv = f64 ? 2 : (kind == kTuneF32G32 ? 2 : 3);
     for (int v = 0; v < nv; ++v) {
         int prev = 0;
@@ -153,7 +153,7 @@ int tune_problem(Problem *P, int kind, int reps, double *cand, int cap, int *n_c
     if (reps < 1 || reps > 10000) return set_error(SEM_EARG, "autotune: reps must be in [1, 10000]");
     const int nq = P->nq;
     const int gprec = kind == kTuneF32G32 ? kGF32 : kGBF16;
-    int rc = kind != kTuneF64 ? mixed_prepare(P, gprec) : dw_prepare(P);
+    int rc = kind != kTuneF64 ? mixed_prepare(P, gprec) : fx_prepare(P);
     if (rc != SEM_OK) return rc;
     CgState *st = kind == kTuneF64 ? P->st : P->st_in;
     unsigned blocks = unsigned(std::min<int64_t>((P->nL + 255) / 256, int64_t(sm_count()) * 8));
@@ -211,7 +211,7 @@ int tune_save(const char *path) {
     FILE *f = fopen(path, "w");
     if (!f) return set_error(SEM_EARG, std::string("autotune_save: cannot write ") + path);
     fprintf(f, "# libsem operator table: kind(0 fp64, 1 fp32/fp32 G, 2 fp32/bf16 G) N variant(0 columns, "
-               "1 lines, 2 persistent, 3 lines with G prefetch, 4 lines with G staged, 5 lines in double-word FP32) "
+               "1 lines, 2 persistent, 3 lines with G prefetch, 4 lines with G staged, 5 lines in fixed point) "
                "elements_per_block us\n");
     for (int k = 0; k < kTuneKinds; ++k)
         for (int q = 2; q <= kMaxQ; ++q) {
