@@ -324,26 +324,158 @@ __device__ __forceinline__ void update_vec(T *__restrict__ x, T *__restrict__ r,
     if constexpr (PRE) acc_merge(*acc_rr, rr);
 }
 
-// Row-class mapping of update vectors to threads: a warp takes the same row
-// (j, k) of EG consecutive elements, LR = (N+1)/V lanes per row, so every
-// lane of a warp is in the same face class in s and t (the gather branches
-// of update_vec are warp-uniform).  Returns the first local node of the
-// lane's vector, or -1 for an idle lane.
-template <int NQ, int V>
-struct RowMap {
-    static constexpr int NQ2 = NQ * NQ, NP = NQ2 * NQ;
+// FP64 update by owner rows.  Only the first copy of a global node (i, j, k >=
+// 1 in its element) is summed and updated: r -= alpha (QQ^T w), and the result
+// is written to the node's other copies (the values are equal there, so they
+// are not read).  A warp takes the same row (j, k) of EG consecutive elements,
+// LR = (N+1)/V lanes per row; a row with j = N or k = N also takes the rows of
+// its copies in the elements above in s and t, and node i = N gets the sum of
+// its copies across the r face from the next lane (the next element's node
+// 0), or from memory for the warp's last element.
+//
+// Each combination of faces is compiled on its own (CY, CZ): GB300's FP64
+// pipe runs at 1/64 rate and an addition that is predicated off takes as long
+// as any other, so one body for all rows, with additions switched off by row
+// and lane, costs 6 FP64 operations per local node instead of 1.4.  E = 32^3,
+// N = 7: 133 us for every copy updating itself with the classes' additions in
+// one chain, 164 us for owner rows in one body, 78 us like this (HBM time of
+// the 22 B per node: 55 us); N = 8 187 -> 102 us, N = 9 102 -> 74 us.
+template <int NQ, typename T>
+struct OwnerRows {
+    static constexpr int V = UpdVec<NQ, T>::value;
+    static constexpr int N = NQ - 1, NQ2 = NQ * NQ, NP = NQ2 * NQ;
     static constexpr int LR = NQ / V;
     static constexpr int EG = 32 / LR;
-    static __device__ __forceinline__ int l0(int task, int lane, int E) {
-        const int eg = task / NQ2;
-        const int row = task - eg * NQ2;
-        const int g = lane / LR, v = lane - g * LR;
-        const int e = eg * EG + g;
-        if (g >= EG || e >= E) return -1;
-        return e * NP + row * NQ + v * V;
-    }
-    static __host__ __device__ int tasks(int E) { return (E + EG - 1) / EG * NQ2; }
+    static __host__ __device__ int64_t tasks(int64_t E) { return (E + EG - 1) / EG * (N * N); }
 };
+
+template <int NQ, int CY, int CZ, bool PRE, typename Acc>
+__device__ __forceinline__ void owner_rows(double *__restrict__ r, const double *__restrict__ w,
+                                           const double *__restrict__ dinv, int j, int k, int eg, int lane, int E,
+                                           const BoxDims &bd, double alpha, Acc &acc, Acc &acc_rr) {
+    using R = OwnerRows<NQ, double>;
+    constexpr int V = R::V, N = R::N, NP = R::NP, LR = R::LR, EG = R::EG, C = CY * CZ;
+    const int g = lane / LR, v = lane - g * LR;
+    const int e = eg * EG + g;
+    bool live = g < EG && e < E;
+    const unsigned ee = live ? unsigned(e) : 0u;
+    const unsigned t = divu(ee, bd.dx);
+    const int ex = int(ee - t * unsigned(bd.nx));
+    if (C > 1) {
+        const unsigned tz = divu(t, bd.dy);
+        const int ey = int(t - tz * unsigned(bd.ny));
+        if ((CY > 1 && ey == bd.ny - 1) || (CZ > 1 && int(tz) == bd.nz - 1)) live = false;   // on the cube boundary
+    }
+    const int oy = bd.nx * NP - N * NQ, oz = bd.nx * bd.ny * NP - N * R::NQ2, ox = NP - N;
+    const int l0 = int(ee) * NP + k * R::NQ2 + j * NQ + v * V;
+    const bool first = v == 0, last = v == LR - 1;
+    const bool hi = last && ex < bd.nx - 1;        // node N has a copy in element e + 1,
+    const bool here = g + 1 < EG && e + 1 < E;     // held by the next lane
+    double s[V], rv[V], dv[V], wv[C][V], xn[C];
+#pragma unroll
+    for (int q = 0; q < V; ++q) rv[q] = dv[q] = 0.0;
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        xn[c] = 0.0;
+#pragma unroll
+        for (int q = 0; q < V; ++q) wv[c][q] = 0.0;
+    }
+    auto offset = [&](int c) { return (CY > 1 && (c & 1) ? oy : 0) + (CZ > 1 && (CY > 1 ? c >> 1 : c) ? oz : 0); };
+    if (live) {
+        vload<double, V>(r + l0, rv);
+        if (PRE) vload_nc<double, V>(dinv + l0, dv);
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            vload_nc<double, V>(w + l0 + offset(c), wv[c]);
+            if (hi && !here) xn[c] = __ldg(w + l0 + offset(c) + V - 1 + ox);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+        s[q] = wv[0][q];
+#pragma unroll
+        for (int c = 1; c < C; ++c) s[q] += wv[c][q];
+    }
+    double up = xn[0];
+    if (C > 1 && hi && !here) {
+#pragma unroll
+        for (int c = 1; c < C; ++c) up += xn[c];
+    }
+    const double next = __shfl_down_sync(0xffffffffu, s[0], 1);
+    if (hi && here) up = next;
+    if (last) s[V - 1] += up;
+    // masked nodes (r faces of the cube) are left as they are
+    const bool mask_lo = first && ex == 0, mask_hi = last && !hi;
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+        const bool masked = (q == 0 && mask_lo) || (q == V - 1 && mask_hi);
+        rv[q] = fma(masked ? 0.0 : -alpha, s[q], rv[q]);
+        if (live && !masked && !(q == 0 && first)) {
+            if constexpr (PRE) {
+                acc_weighted_square(acc, dv[q], rv[q]);
+                acc_square(acc_rr, rv[q]);
+            } else {
+                acc_square(acc, rv[q]);
+            }
+        }
+    }
+    // node 0 has its first copy in element e - 1: the previous lane, or (first
+    // element of the warp) the previous warp, whose last lane writes it
+    const double prev = __shfl_up_sync(0xffffffffu, rv[V - 1], 1);
+    const bool skip = first && ex > 0 && g == 0;
+    if (first && ex > 0) rv[0] = prev;
+    if (live) {
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            double *q = r + l0 + offset(c);
+            if (skip) {
+#pragma unroll
+                for (int z = 1; z < V; ++z) q[z] = rv[z];
+            } else {
+                vstore<double, V>(q, rv);
+            }
+            if (hi && !here) q[V - 1 + ox] = rv[V - 1];
+        }
+    }
+}
+
+// One task: row (j, k) of element group eg, tasks numbered row fastest.
+template <int NQ, bool PRE, typename Acc>
+__device__ __forceinline__ void owner_task(double *r, const double *w, const double *dinv, int task, int lane, int E,
+                                           const BoxDims &bd, double alpha, Acc &acc, Acc &acc_rr) {
+    constexpr int N = NQ - 1;
+    const int eg = task / (N * N), row = task - eg * (N * N);
+    const int k = 1 + row / N, j = 1 + row - (k - 1) * N;
+    if (j < N && k < N)
+        owner_rows<NQ, 1, 1, PRE>(r, w, dinv, j, k, eg, lane, E, bd, alpha, acc, acc_rr);
+    else if (k < N)
+        owner_rows<NQ, 2, 1, PRE>(r, w, dinv, j, k, eg, lane, E, bd, alpha, acc, acc_rr);
+    else if (j < N)
+        owner_rows<NQ, 1, 2, PRE>(r, w, dinv, j, k, eg, lane, E, bd, alpha, acc, acc_rr);
+    else
+        owner_rows<NQ, 2, 2, PRE>(r, w, dinv, j, k, eg, lane, E, bd, alpha, acc, acc_rr);
+}
+
+// The tasks of warp `wid` of `nw`: a contiguous run, so that every warp gets
+// rows of every class (with a stride of nw, a multiple of N^2 gives a warp
+// the same row each time: 133 -> 106 us at N = 7 for the former kernel).
+template <int NQ, bool PRE, typename Acc>
+__device__ __forceinline__ void owner_tasks(double *r, const double *w, const double *dinv, int wid, int nw, int E,
+                                            const BoxDims &bd, double alpha, Acc &acc, Acc &acc_rr) {
+    const int ntask = int(OwnerRows<NQ, double>::tasks(E));
+    const int per = (ntask + nw - 1) / nw;
+    const int end = min(ntask, (wid + 1) * per);
+    for (int task = wid * per; task < end; ++task)
+        owner_task<NQ, PRE>(r, w, dinv, task, int(threadIdx.x & 31), E, bd, alpha, acc, acc_rr);
+}
+
+// Blocks of 256 threads (6 resident per SM) of an owner-row launch.
+constexpr int kOwnerBlocks = 6;
+template <int NQ>
+static unsigned owner_grid(const Problem *P) {
+    const int64_t blocks = (OwnerRows<NQ, double>::tasks(P->E) * 32 + 255) / 256;
+    return unsigned(std::min<int64_t>(blocks, int64_t(sm_count()) * kOwnerBlocks));
+}
 
 // b = mask(QQ^T f) on the box (copies summed in ascending local index).
 template <int NQ>
@@ -403,26 +535,17 @@ __global__ void __launch_bounds__(256, 5) cg_update_nodes_kernel(T *__restrict__
     }
 }
 
-// The same step with the row-class mapping (RowMap): used where the
-// arithmetic pipe, not HBM, bounds the update (FP64 on GB300).
-template <int NQ, typename T, typename Acc>
-__global__ void __launch_bounds__(256) cg_update_class_kernel(T *__restrict__ x, T *__restrict__ r,
-                                                              const T *__restrict__ p, const T *__restrict__ w,
-                                                              int nL, BoxDims bd, double *partials, CgState *st) {
+// The FP64 step by owner rows (x += alpha p is deferred to the next operator
+// kernel, which holds p anyway).
+template <int NQ>
+__global__ void __launch_bounds__(256, kOwnerBlocks)
+    cg_update_owner_kernel(double *__restrict__ r, const double *__restrict__ w, int E, BoxDims bd, double *partials,
+                           CgState *st) {
     __shared__ double scratch[256];
     if (st->done) return;
-    constexpr int V = UpdVec<NQ, T>::value;
-    using RM = RowMap<NQ, V>;
-    const T alpha = T(st->alpha);
-    const int E = nL / RM::NP;
-    const int ntask = RM::tasks(E);
-    const int lane = threadIdx.x & 31;
-    const int nwarps = int(gridDim.x * blockDim.x) >> 5;
-    Acc acc = acc_zero<Acc>();
-    for (int task = int(blockIdx.x * blockDim.x + threadIdx.x) >> 5; task < ntask; task += nwarps) {
-        const int l0 = RM::l0(task, lane, E);
-        if (l0 >= 0) update_vec<NQ, V, T, Acc, false, true>(x, r, p, w, l0, bd, alpha, acc);
-    }
+    DwAcc acc = acc_zero<DwAcc>(), unused = acc_zero<DwAcc>();
+    owner_tasks<NQ, false>(r, w, nullptr, int(blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                           int(gridDim.x * blockDim.x) >> 5, E, bd, st->alpha, acc, unused);
     // one warp's FP64 sum per block (13 instead of 40 warp-wide FP64 adds),
     // grid sum in groups
     const double bs = block_sum_wide(acc_value(acc), scratch);
@@ -432,12 +555,8 @@ __global__ void __launch_bounds__(256) cg_update_class_kernel(T *__restrict__ x,
     }
 }
 
-// Blocks of an update launch, grid-stride beyond.  Measured on GB300 at
-// E = 32^3, N = 7: the FP32 update is fastest with one resident wave
-// (inner CG iteration 216 -> 190 us); the FP64 update with 8 blocks per SM
-// (230 us; one wave of 5 per SM: 293 us; one vector per thread, 32768
-// blocks: 340 us -- each block's FP64 reduction costs more than the latency
-// it hides).
+// Blocks of an FP32 update launch, grid-stride beyond: one resident wave (E =
+// 32^3, N = 7: inner CG iteration 216 -> 190 us).
 template <typename K>
 static int64_t resident_blocks(K kern, int threads) {
     static int per_sm = 0;
@@ -454,13 +573,10 @@ template <int NQ, typename T, typename Acc>
 static int launch_update_rows_nq(const Problem *P, T *x, T *r, const T *p, const T *w, CgState *st) {
     constexpr int V = UpdVec<NQ, T>::value;
     if constexpr (sizeof(T) == 8) {
-        using RM = RowMap<NQ, V>;
-        int64_t blocks = (int64_t(RM::tasks(int(P->E))) * 32 + 255) / 256;
-        blocks = std::min<int64_t>(blocks, int64_t(sm_count()) * 8);
-        cg_update_class_kernel<NQ, T, Acc><<<unsigned(blocks), 256, 0, stream()>>>(
-            x, r, p, w, int(P->nL), box_dims(P->nx, P->ny, P->nz), P->partials, st);
+        cg_update_owner_kernel<NQ><<<owner_grid<NQ>(P), 256, 0, stream()>>>(
+            r, w, int(P->E), box_dims(P->nx, P->ny, P->nz), P->partials, st);
         count_launches(1);
-        return cuda_check(cudaGetLastError(), "cg_update_class_kernel");
+        return cuda_check(cudaGetLastError(), "cg_update_owner_kernel");
     }
     int64_t blocks = (P->nL / V + 255) / 256;
     blocks = std::min(blocks, resident_blocks(cg_update_nodes_kernel<NQ, T, Acc>, 256));

@@ -13,10 +13,10 @@
 //   1. the operator kernel in CG mode (the variant the tuner chose): the
 //      previous iteration's x += alpha p, then p = r + beta p; w = A_local p;
 //      <p, A p>; alpha
-//   2. cg_update_class_kernel (sem_box.cuh): every local node sums the copies
-//      of w of its global node in ascending local index (the direct-stiffness
-//      sum), then applies r -= alpha (QQ^T w) to itself; <r, r> is
-//      accumulated once per global node; the block that completes the grid
+//   2. cg_update_owner_kernel (sem_box.cuh): the first copy of every global
+//      node sums the copies of w (the direct-stiffness sum, in a fixed order),
+//      applies r -= alpha (QQ^T w) and writes the result to every copy; <r, r>
+//      is accumulated once per global node; the block that completes the grid
 //      sum forms rho, beta, the iteration count and the stop flag.
 // Moving x += alpha p into the next operator kernel (which has p in shared
 // memory anyway) takes 24 of the update's 48 bytes per node off HBM and one

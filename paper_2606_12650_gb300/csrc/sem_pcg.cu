@@ -118,28 +118,18 @@ __global__ void pcg_init_kernel(const double *__restrict__ b, const double *__re
     }
 }
 
+// The update by owner rows (sem_box.cuh), with both reductions accumulated in
+// double-word FP32 per thread (the recurrences stay FP64): GB300's FP64 pipe
+// runs at 1/64 rate.
 template <int NQ>
-__global__ void __launch_bounds__(256) pcg_update_kernel(double *__restrict__ x, double *__restrict__ r,
-                                                         const double *__restrict__ p,
-                                                         const double *__restrict__ w,
-                                                         const double *__restrict__ dinv, int nL, BoxDims bd,
-                                                         double *partials, CgState *st) {
+__global__ void __launch_bounds__(256, kOwnerBlocks)
+    pcg_update_kernel(double *__restrict__ r, const double *__restrict__ w, const double *__restrict__ dinv, int E,
+                      BoxDims bd, double *partials, CgState *st) {
     __shared__ double red[32];
     if (st->done) return;
-    constexpr int V = UpdVec<NQ, double>::value;
-    using RM = RowMap<NQ, V>;
-    const double alpha = st->alpha;
-    // both reductions accumulated in double-word FP32 per thread (the
-    // recurrences stay FP64): GB300's FP64 pipe runs at 1/64 rate
     DwAcc rz = acc_zero<DwAcc>(), rr = acc_zero<DwAcc>();
-    const int E = nL / RM::NP;
-    const int ntask = RM::tasks(E);
-    const int lane = threadIdx.x & 31;
-    const int nwarps = int(gridDim.x * blockDim.x) >> 5;
-    for (int task = int(blockIdx.x * blockDim.x + threadIdx.x) >> 5; task < ntask; task += nwarps) {
-        const int l0 = RM::l0(task, lane, E);
-        if (l0 >= 0) update_vec<NQ, V, double, DwAcc, true, true>(x, r, p, w, l0, bd, alpha, rz, dinv, &rr);
-    }
+    owner_tasks<NQ, true>(r, w, dinv, int(blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                          int(gridDim.x * blockDim.x) >> 5, E, bd, st->alpha, rz, rr);
     const double s0 = block_sum(acc_value(rz), red);
     const double s1 = block_sum(acc_value(rr), red);
     if (publish_partial2(s0, s1, partials, &st->ticket_up)) {
@@ -151,11 +141,8 @@ __global__ void __launch_bounds__(256) pcg_update_kernel(double *__restrict__ x,
 
 template <int NQ>
 static int launch_pcg_update_nq(const Problem *P) {
-    constexpr int V = UpdVec<NQ, double>::value;
-    int64_t blocks = (int64_t(RowMap<NQ, V>::tasks(int(P->E))) * 32 + 255) / 256;
-    blocks = std::min<int64_t>(blocks, int64_t(sm_count()) * 8);
-    pcg_update_kernel<NQ><<<unsigned(blocks), 256, 0, stream()>>>(P->x, P->r, P->p, P->w, P->dinv, int(P->nL),
-                                                                  box_dims(P->nx, P->ny, P->nz), P->partials, P->st);
+    pcg_update_kernel<NQ><<<owner_grid<NQ>(P), 256, 0, stream()>>>(P->r, P->w, P->dinv, int(P->E),
+                                                                   box_dims(P->nx, P->ny, P->nz), P->partials, P->st);
     count_launches(1);
     return cuda_check(cudaGetLastError(), "pcg_update_kernel");
 }
