@@ -433,6 +433,35 @@ __device__ __forceinline__ void lines_group_fx(const double *x, double *y, doubl
     }
 }
 
+// Block b of nb after lines_group_fx: the block's <p, A_local p>, and in the
+// last block alpha = rho / <p, A p>.
+template <int NQ>
+__device__ __forceinline__ void fx_publish(double part, unsigned char *smem, int epb, double *partials, CgState *st,
+                                           int b, int nb) {
+    double bs = part;
+    if (epb > 1) {
+        // the regions are free: every thread passed lines_group_fx's last barrier after its reads
+        double *sums = reinterpret_cast<double *>(smem + fx_words<NQ>(epb));
+        const int eb = threadIdx.x / (NQ * NQ);
+        if (int(threadIdx.x) == eb * NQ * NQ && eb < epb) sums[eb] = part;
+        __syncthreads();
+        bs = 0.0;
+        if (threadIdx.x < 32) {
+            for (int k = threadIdx.x; k < epb; k += 32) bs += sums[k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (o < epb) bs += __shfl_down_sync(0xffffffffu, bs, o);
+        }
+    }
+    if (publish_grouped(bs, partials, &st->ticket_ax, b, nb)) {
+        const double pap = finish_grouped(partials, &st->ticket_ax, nb);
+        if (threadIdx.x == 0) {
+            st->pap = pap;
+            st->alpha = st->rho / pap;
+        }
+    }
+}
+
 template <int NQ, bool CG, bool PRE>
 __global__ void __maxnreg__(FxRegs<NQ>::value) ax_fx_kernel(const __grid_constant__ AxFxArgs P) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -446,30 +475,7 @@ __global__ void __maxnreg__(FxRegs<NQ>::value) ax_fx_kernel(const __grid_constan
     double part = 0.0;
     lines_group_fx<NQ, CG, PRE>(A.x, A.y, A.p, P.G, P.kg, P.d, P.dt, beta, xalpha, CG ? A.xs : nullptr, A.dinv, e0, ne,
                                 P.epb, smem, &part);
-    if (CG) {
-        double bs = part;
-        if (P.epb > 1) {
-            // the regions are free: every thread passed lines_group_fx's last barrier after its reads
-            double *sums = reinterpret_cast<double *>(smem + fx_words<NQ>(P.epb));
-            const int eb = threadIdx.x / (NQ * NQ);
-            if (int(threadIdx.x) == eb * NQ * NQ && eb < P.epb) sums[eb] = part;
-            __syncthreads();
-            bs = 0.0;
-            if (threadIdx.x < 32) {
-                for (int k = threadIdx.x; k < P.epb; k += 32) bs += sums[k];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1)
-                    if (o < P.epb) bs += __shfl_down_sync(0xffffffffu, bs, o);
-            }
-        }
-        if (publish_grouped(bs, A.partials, &A.st->ticket_ax)) {
-            const double pap = finish_grouped(A.partials, &A.st->ticket_ax);
-            if (threadIdx.x == 0) {
-                A.st->pap = pap;
-                A.st->alpha = A.st->rho / pap;
-            }
-        }
-    }
+    if (CG) fx_publish<NQ>(part, smem, P.epb, A.partials, A.st, int(blockIdx.x), int(gridDim.x));
 }
 
 // Host: the even-odd halves of M (row-major nq x nq) times 2^k, rounded to

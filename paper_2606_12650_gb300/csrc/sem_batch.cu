@@ -3,17 +3,19 @@
 // problems (one per order present for the operator, one for the vector
 // update), replayed from a CUDA graph.
 //
-// Work lists.  Every problem is cut into operator items (~16384 local nodes:
+// Work lists.  Every problem is cut into operator items (item_nodes:
 // several passes of a 256-thread block) and vector items (row-aligned runs of
-// ~16384 local nodes).  A persistent kernel's CTAs take items from a global
+// item_nodes).  A persistent kernel's CTAs take items from a global
 // counter (dynamic load balance across problems of very different cost).
 // The operator list keeps each order's items together, and each order has
 // its own kernel, compiled for that order and body with the body inlined;
 // the vector kernel switches on N on the device.  The operator body and the
 // elements per pass follow the per-order tuner's table for the batch's
-// precision: the line body (sem_ax_lines.cuh), in fixed-point arithmetic for
-// FP64 batches where the table chose that variant (sem_ax_fx.cuh), or the
-// column body, passes of 256 / (N+1)^2 elements.  Items of problems whose
+// precision: the line body (sem_ax_lines.cuh) or the column body, passes of
+// 256 / (N+1)^2 elements.  FP64 batches whose table chose the fixed-point
+// variant (sem_ax_fx.cuh) take that kernel and the owner-row update
+// (sem_box.cuh) instead, one block per item as in a stand-alone solve, from
+// lists that a kernel writes on the device ("fixed-point orders" below).  Items of problems whose
 // solve finished are dropped from the lists between rounds (the items of one
 // problem stay together and in order, so its reductions never change).
 //
@@ -50,16 +52,17 @@
 namespace sem {
 
 constexpr int kBatchThreads = 256;
-constexpr int kVecItemNodes = 16384;
-constexpr int kAxItemNodes = 16384;  // local nodes per operator item (several passes of the block)
+// Local nodes per item of a problem of nL nodes: a 128th of it, at least 1024
+// and at most 16384 (several passes of the block share an item's queue ticket
+// and reduction, but a CTA works through an item alone).  A rule of the
+// problem only, so that its reductions do not depend on the batch.
+static int item_nodes(int64_t nL) { return int(std::min<int64_t>(16384, std::max<int64_t>(1024, nL / 128))); }
 
 struct BatchProb {
     int nq, nx, ny, nz;
     BoxDims bd;                     // the box with its fast divisors
     int64_t E, nL;
     const double *G;
-    const int4 *Gfx;                // integer factors and their scales (FP64 batches with the
-    const int32_t *kgfx;            // fixed-point body)
     const __nv_bfloat16 *G16;
     const float *G32;
     double *x, *r, *p, *w;          // FP64 CG vectors / refinement x, r
@@ -93,6 +96,91 @@ enum BatchQ : int { kQAx = 0, kQVec = 1, kNumQ = 2 };
 
 // Operator bodies of a batch: every member of one order takes the same one.
 enum AxBody : int { kBodyColumns = 0, kBodyLines = 1, kBodyFX = 2, kBodyNone = -1 };
+
+// ---- fixed-point orders (FP64 batches): one block per item, everything the
+// block needs in its item, so that it waits for one load before its own data.
+struct FxItem {                     // operator: ne elements from e0
+    const double *r;
+    double *w, *p, *x;
+    const int4 *G;
+    const int32_t *kg;
+    CgState *st;
+    double *partials;
+    int e0, ne;                     // ne = 0: beyond the list
+    int b, nb;                      // block b of the problem's nb
+};
+struct OwnerItem {                  // update: warps 8 b .. 8 b + 7 of the problem's 8 nb
+    double *r;
+    const double *w;
+    CgState *st;
+    double *partials;
+    BoxDims bd;
+    int E, b, nb;                   // nb = 0: beyond the list
+    int prob;
+};
+struct FxMember {                   // a member's ranges in its order's lists
+    FxItem op;                      // e0, ne, b unset
+    OwnerItem up;                   // b unset
+    FxItem *items;
+    OwnerItem *owners;
+    int first, epb;
+    int64_t E;
+    int up_first;
+};
+
+// Blocks of a problem's owner-row update: 1 to 8 rows per warp, more for
+// larger problems (a rule of the problem only).
+template <int NQ>
+static int owner_blocks(int64_t E) {
+    const int64_t tasks = OwnerRows<NQ, double>::tasks(E);
+    const int64_t per = std::min<int64_t>(8, std::max<int64_t>(1, tasks / 2048));
+    return int((tasks + 8 * per - 1) / (8 * per));
+}
+static int owner_blocks_of(const Problem *P) {
+    switch (P->nq) {
+#define SEM_OB(Q) case Q: return owner_blocks<Q>(P->E);
+        SEM_OB(2) SEM_OB(3) SEM_OB(4) SEM_OB(5) SEM_OB(6) SEM_OB(7) SEM_OB(8) SEM_OB(9) SEM_OB(10)
+#undef SEM_OB
+        default: return 0;
+    }
+}
+
+// One block per member: writes its items and clears its group tickets (no
+// launch of the batch is in flight).
+__global__ void batch_fx_items_kernel(const FxMember *members) {
+    const FxMember M = members[blockIdx.x];
+    for (int b = threadIdx.x; b < M.op.nb; b += blockDim.x) {
+        FxItem it = M.op;
+        it.b = b;
+        it.e0 = b * M.epb;
+        it.ne = int(min(int64_t(M.epb), M.E - it.e0));
+        M.items[M.first + b] = it;
+    }
+    for (int b = threadIdx.x; b < M.up.nb; b += blockDim.x) {
+        OwnerItem it = M.up;
+        it.b = b;
+        M.owners[M.up_first + b] = it;
+    }
+    uint32_t *gt = group_tickets(M.op.partials, partials_capacity(M.op.partials));
+    for (int g = threadIdx.x; g < (max(M.op.nb, M.up.nb) + kSumGroup - 1) / kSumGroup; g += blockDim.x) gt[g] = 0u;
+}
+
+struct FxBatchArgs {
+    const FxItem *items;
+    EoMatFX d, dt;
+    int epb;
+};
+
+template <int NQ>
+__global__ void __maxnreg__(FxRegs<NQ>::value) batch_fx_kernel(const __grid_constant__ FxBatchArgs P) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const FxItem it = P.items[blockIdx.x];
+    if (it.ne == 0 || it.st->done) return;
+    double part = 0.0;
+    lines_group_fx<NQ, true, false>(it.r, it.w, it.p, it.G, it.kg, P.d, P.dt, it.st->beta, it.st->alpha, it.x, nullptr,
+                                    it.e0, it.ne, P.epb, smem, &part);
+    fx_publish<NQ>(part, smem, P.epb, it.partials, it.st, it.b, it.nb);
+}
 constexpr int kOrders = kMaxQ - 1;  // N+1 = 2 .. kMaxQ
 
 struct BatchCtl {
@@ -139,15 +227,24 @@ struct Batch {
     BatchCtl *ctl_host = nullptr;
     unsigned seen_finished = 0;
     bool any_init = false;
+    // fixed-point orders: the two lists, their capacities, the blocks of a
+    // launch, and the elements per operator block
+    FxItem *d_fx[kOrders] = {};
+    OwnerItem *d_own[kOrders] = {};
+    int cap_fx[kOrders] = {}, cap_own[kOrders] = {};
+    int fx_grid[kOrders] = {}, own_grid[kOrders] = {}, fx_epb[kOrders] = {};
+    FxMember *d_members = nullptr;
+    int cap_members = 0;
     cudaGraphExec_t graph = nullptr;
     cudaStream_t graph_stream = nullptr;
     // the buffers the captured round reads and its grids; the graph stays
     // valid while the buffers stay in place and the grids stay the same
     // (membership changes only rewrite the lists' contents and counts)
-    const void *graph_bufs[7] = {};
+    const void *graph_bufs[7 + 2 * kOrders] = {};
     int graph_items[2] = {0, 0};    // power-of-two ceilings of the item counts at capture
     int ord_ranges[4 * kOrders];    // host copy of the device per-order ranges (operator, vector)
-    int graph_ord[2 * kOrders] = {};  // per order: the captured launches' grid ceilings and body (0: none)
+    int graph_fx[2 * kOrders] = {};   // the fixed-point orders' grids at capture
+    int graph_ord[3 * kOrders] = {};  // per order: the captured launches' grid ceilings and body (0: none)
     int64_t graph_launches = 0;     // kernel launches in one replay
     // side streams and events that fork the per-order operator launches into
     // parallel branches of the captured round (the tail of one order's launch
@@ -162,11 +259,10 @@ struct BEpb {
 };
 
 // Dynamic shared memory of one order's operator body: the column body's
-// slabs, or the line body's three regions, or the fixed-point body's.
+// slabs, or the line body's three regions.
 template <int NQ, typename T, int BODY>
 inline size_t batch_ax_smem() {
     return BODY == kBodyColumns ? AxShape<NQ, BEpb<NQ>::value, T>::SMEM
-           : BODY == kBodyFX    ? 16 + fx_smem<NQ>(BEpb<NQ>::value)
                                 : LineShape::smem(NQ, BEpb<NQ>::value, int(sizeof(T)));
 }
 
@@ -178,7 +274,6 @@ __constant__ float c_D32[kMaxQ - 1][kMaxQ * kMaxQ];
 // even-odd coefficients of D ([0]) and D^T ([1]) for the line body
 __constant__ EoMat<double> c_E64[kMaxQ - 1][2];
 __constant__ EoMat<float> c_E32[kMaxQ - 1][2];
-__constant__ EoMatFX c_EFX[kMaxQ - 1][2];
 
 template <typename T>
 __device__ __forceinline__ const EoMat<T> &const_eo(int nq, int which);
@@ -299,22 +394,6 @@ __device__ __forceinline__ bool batch_lines_item(const T *xin, T *yout, T *pv, c
     return true;
 }
 
-// The fixed-point line body (FP64 batches): same passes as batch_lines_item.
-template <int NQ, bool CG>
-__device__ __forceinline__ void batch_fx_item(const double *xin, double *yout, double *pv, const int4 *Gfx,
-                                              const int32_t *kg, double beta, int64_t first, int count, int group,
-                                              unsigned char *smem, double *pt) {
-    double acc = 0.0;
-    for (int g = 0; g < count; g += group) {
-        double part = 0.0;
-        lines_group_fx<NQ, CG, false>(xin, yout, pv, Gfx, kg, c_EFX[NQ - 2][0], c_EFX[NQ - 2][1], beta, 0.0, nullptr,
-                                      nullptr, first + g, min(group, count - g), group, smem, &part);
-        acc += part;
-        __syncthreads();
-    }
-    *pt = acc;
-}
-
 // mode: 0 = FP64 CG (p = r + beta p, w = A p), 1 = FP64 plain (w = A x),
 //       2 = FP32 inner CG on the FP32 vectors
 // One order's items (N+1 = NQ), one body.  FP32 items are HBM-bound: 4 CTAs
@@ -325,7 +404,6 @@ __global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 4 ? 4 : 2)
     batch_ax_kernel(BatchProb *probs, const BatchItem *items, double *part, uint32_t *tickets, BatchCtl *ctl,
                     int32_t *status) {
     constexpr bool CG = MODE != 1;
-    static_assert(BODY != kBodyFX || std::is_same<T, double>::value, "the fixed-point body is FP64");
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double red[32];
     __shared__ int s_item;
@@ -353,11 +431,8 @@ __global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 4 ? 4 : 2)
         else if (MODE == 1) { xin = reinterpret_cast<const T *>(P.x); yout = reinterpret_cast<T *>(P.w); pv = nullptr; }
         else { xin = reinterpret_cast<const T *>(P.r32); yout = reinterpret_cast<T *>(P.w32); pv = reinterpret_cast<T *>(P.p32); }
         T pt = T(0);
-        bool ok = true;
-        if constexpr (BODY == kBodyFX)
-            batch_fx_item<NQ, CG>(xin, yout, pv, P.Gfx, P.kgfx, beta, item.first, item.count, item.group, smem + 16,
-                                  &pt);
-        else if constexpr (BODY == kBodyLines)
+        bool ok;
+        if constexpr (BODY == kBodyLines)
             ok = batch_lines_item<NQ, T, GT, CG>(xin, yout, pv, prob_G<GT>(P), beta, item.first, item.count,
                                                  item.group, regA, bar, &phase, status, &pt);
         else
@@ -601,6 +676,26 @@ __global__ void __launch_bounds__(kBatchThreads, MODE == kVecUpdate32 ? kUpd32Bl
     leave_queue(q);
 }
 
+// The owner-row update of a fixed-point order.
+template <int NQ>
+__global__ void __launch_bounds__(256, kOwnerBlocks)
+    batch_owner_kernel(const OwnerItem *items, BatchProb *probs, BatchCtl *ctl, int32_t *finished_ids) {
+    __shared__ double scratch[256];
+    const OwnerItem it = items[blockIdx.x];
+    if (it.nb == 0 || it.st->done) return;
+    DwAcc acc = acc_zero<DwAcc>(), unused = acc_zero<DwAcc>();
+    owner_tasks<NQ, false>(it.r, it.w, nullptr, 8 * it.b + int(threadIdx.x >> 5), 8 * it.nb, it.E, it.bd, it.st->alpha,
+                           acc, unused);
+    const double bs = block_sum_wide(acc_value(acc), scratch);
+    if (publish_grouped(bs, it.partials, &it.st->ticket_up, it.b, it.nb)) {
+        const double rho_new = finish_grouped(it.partials, &it.st->ticket_up, it.nb);
+        if (threadIdx.x == 0) {
+            cg_close_iteration(it.st, rho_new);
+            if (it.st->done) finish_problem(probs[it.prob], it.prob, ctl, finished_ids);
+        }
+    }
+}
+
 // Per-problem flag updates between phases (one thread per problem).
 enum FlagOp : int { kFlagClearInit = 0, kFlagMarkRefine = 1, kFlagClearRefine = 2 };
 
@@ -665,7 +760,7 @@ struct BaxLaunch {
 };
 
 // Dispatch on the order and body (prepare only, or launch for `count`
-// items).  The fixed-point body exists for FP64 CG batches only.
+// items).
 template <typename T, typename GT, int MODE, int NQ>
 static int bax_order(Batch *B, int body, int count, bool launch, int *res) {
     int r = 0;
@@ -677,11 +772,6 @@ static int bax_order(Batch *B, int body, int count, bool launch, int *res) {
         case kBodyLines:
             return launch ? BaxLaunch<T, GT, MODE, NQ, kBodyLines>::launch(B, count)
                           : BaxLaunch<T, GT, MODE, NQ, kBodyLines>::resident(res);
-        case kBodyFX:
-            if constexpr (MODE == 0)
-                return launch ? BaxLaunch<T, GT, MODE, NQ, kBodyFX>::launch(B, count)
-                              : BaxLaunch<T, GT, MODE, NQ, kBodyFX>::resident(res);
-            [[fallthrough]];
         default: return set_error(SEM_EARG, "batch: no such operator body for this precision");
     }
 }
@@ -775,6 +865,46 @@ static int upd(Batch *B, int nq, int count, bool launch, int *res = nullptr) {
     }
 }
 
+// One fixed-point order's operator (up = false) or update launch.
+template <int NQ>
+static int fx_launch_nq(Batch *B, bool up, bool launch) {
+    const int o = NQ - 2;
+    if (up) {
+        if (!launch) return SEM_OK;
+        batch_owner_kernel<NQ><<<unsigned(B->own_grid[o]), 256, 0, stream()>>>(B->d_own[o], B->d_probs, B->ctl,
+                                                                              B->finished_ids);
+    } else {
+        const int epb = B->fx_epb[o];
+        static size_t sm_set = 0;
+        const size_t sm = fx_smem<NQ>(epb);
+        if (sm > sm_set) {   // before any capture (prepare_bax)
+            const int rc = cuda_check(cudaFuncSetAttribute(batch_fx_kernel<NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                           int(sm)), "batch: shared-memory attribute");
+            if (rc != SEM_OK) return rc;
+            sm_set = sm;
+        }
+        if (!launch) return SEM_OK;
+        FxBatchArgs A{};
+        A.items = B->d_fx[o];
+        A.epb = epb;
+        double xi[kMaxQ], w[kMaxQ], D[kMaxQ * kMaxQ];
+        gll_rule_and_derivative(NQ - 1, xi, w, D);
+        fx_coefficients(D, NQ, &A.d, &A.dt);
+        batch_fx_kernel<NQ><<<unsigned(B->fx_grid[o]), unsigned(line_threads(NQ, epb)), sm, stream()>>>(A);
+    }
+    count_launches(1);
+    return cuda_check(cudaGetLastError(), "batch: fixed-point launch");
+}
+
+static int fx_launch(Batch *B, int nq, bool up, bool launch) {
+    switch (nq) {
+#define SEM_FX(Q) case Q: return fx_launch_nq<Q>(B, up, launch);
+        SEM_FX(2) SEM_FX(3) SEM_FX(4) SEM_FX(5) SEM_FX(6) SEM_FX(7) SEM_FX(8) SEM_FX(9) SEM_FX(10)
+#undef SEM_FX
+        default: return set_error(SEM_EARG, "batch: unsupported order");
+    }
+}
+
 // Side streams and events of the parallel operator phase (made once, outside
 // any capture).
 static int make_side_streams(Batch *B) {
@@ -793,7 +923,9 @@ static int prepare_bax(Batch *B) {
         const int body = B->ord_body[o];
         if (body == kBodyNone) continue;
         int rc;
-        if (B->mode == 0) {
+        if (body == kBodyFX) {
+            rc = fx_launch(B, o + 2, false, false);
+        } else if (B->mode == 0) {
             rc = bax<double, double, 0>(B, o + 2, body, 0, false, &B->ord_res[o]);
             if (rc == SEM_OK) rc = upd<kVecUpdate64>(B, o + 2, 0, false, &B->ord_vres[o]);
         } else {
@@ -852,7 +984,6 @@ static int batch_attrs(Batch *B) {
         }
         static EoMat<double> e64[kMaxQ - 1][2];
         static EoMat<float> e32[kMaxQ - 1][2];
-        static EoMatFX efx[kMaxQ - 1][2];
         for (int N = 1; N <= kMaxQ - 1; ++N) {
             const int nq = N + 1;
             double Dt[kMaxQ * kMaxQ];
@@ -862,13 +993,11 @@ static int batch_attrs(Batch *B) {
             e64[N - 1][1] = eo_coefficients<double>(Dt, nq);
             e32[N - 1][0] = eo_coefficients<float>(h64[N - 1], nq);
             e32[N - 1][1] = eo_coefficients<float>(Dt, nq);
-            fx_coefficients(h64[N - 1], nq, &efx[N - 1][0], &efx[N - 1][1]);
         }
         int rc = cuda_check(cudaMemcpyToSymbol(c_D64, h64, sizeof h64), "batch: D table");
         if (rc == SEM_OK) rc = cuda_check(cudaMemcpyToSymbol(c_D32, h32, sizeof h32), "batch: D table");
         if (rc == SEM_OK) rc = cuda_check(cudaMemcpyToSymbol(c_E64, e64, sizeof e64), "batch: even-odd table");
         if (rc == SEM_OK) rc = cuda_check(cudaMemcpyToSymbol(c_E32, e32, sizeof e32), "batch: even-odd table");
-        if (rc == SEM_OK) rc = cuda_check(cudaMemcpyToSymbol(c_EFX, efx, sizeof efx), "batch: even-odd table");
         if (rc != SEM_OK) return rc;
         done = true;
     }
@@ -925,8 +1054,107 @@ static int upload_order_ranges(Batch *B, const int *ord_first) {
 static void order_signature(const Batch *B, int *out) {
     for (int o = 0; o < kOrders; ++o) {
         const bool on = B->ord_body[o] != kBodyNone;
+        out[2 * kOrders + o] = 0;
+        if (B->ord_body[o] == kBodyFX) {
+            out[o] = kBodyFX + 1;   // the grids: keep_or_drop_graph
+            out[kOrders + o] = 0;
+            out[2 * kOrders + o] = B->fx_epb[o];
+            continue;
+        }
         out[o] = on ? 4 * items_grid(B->ord_res[o], B->ord_count[o]) + B->ord_body[o] + 1 : 0;
         out[kOrders + o] = on ? items_grid(B->ord_vres[o], B->ord_vcount[o]) : 0;
+    }
+}
+
+static void graph_buffers(const Batch *B, const void **out) {
+    const void *bufs[7] = {B->d_probs, B->d_ax, B->d_vec, B->part, B->part_vec, B->tickets, B->finished_ids};
+    std::copy(bufs, bufs + 7, out);
+    for (int o = 0; o < kOrders; ++o) {
+        out[7 + o] = B->d_fx[o];
+        out[7 + kOrders + o] = B->d_own[o];
+    }
+}
+
+template <typename X>
+static int grow(X **buf, int *cap, int need);
+
+// The lists of the fixed-point orders, members in order, finished ones left
+// out, written on the device.  A member's items and their reduction tree
+// depend on the member only.
+static int build_fx_lists(Batch *B) {
+    const int n = int(B->probs.size());
+    std::vector<FxMember> ms;
+    int rc = SEM_OK;
+    for (int o = 0; o < kOrders && rc == SEM_OK; ++o) {
+        if (B->ord_body[o] != kBodyFX) continue;
+        const size_t m0 = ms.size();
+        int nf = 0, nu = 0;
+        for (int k = 0; k < n; ++k) {
+            const Problem *P = B->probs[k];
+            if (P->nq - 2 != o || B->gone[k]) continue;
+            FxMember M{};
+            M.op = FxItem{P->r, P->w, P->p, P->x, P->Gfx, P->kgfx, P->st, P->partials, 0, 0, 0,
+                          int((P->E + B->fx_epb[o] - 1) / B->fx_epb[o])};
+            M.up = OwnerItem{P->r, P->w, P->st, P->partials, box_dims(P->nx, P->ny, P->nz), int(P->E), 0,
+                             owner_blocks_of(P), k};
+            if (M.op.nb > P->partials_cap || M.up.nb > P->partials_cap)
+                return set_error(SEM_ERANGE, "batch: more blocks than reduction slots");
+            M.first = nf;
+            M.up_first = nu;
+            M.epb = B->fx_epb[o];
+            M.E = P->E;
+            nf += M.op.nb;
+            nu += M.up.nb;
+            ms.push_back(M);
+        }
+        B->fx_grid[o] = std::max(nf, 1);
+        B->own_grid[o] = std::max(nu, 1);
+        rc = grow(&B->d_fx[o], &B->cap_fx[o], B->fx_grid[o]);
+        if (rc == SEM_OK) rc = grow(&B->d_own[o], &B->cap_own[o], B->own_grid[o]);
+        for (size_t m = m0; m < ms.size(); ++m) {
+            ms[m].items = B->d_fx[o];
+            ms[m].owners = B->d_own[o];
+        }
+        // a captured round may have more blocks than there are items now: theirs are empty
+        if (rc == SEM_OK)
+            rc = cuda_check(cudaMemsetAsync(B->d_fx[o], 0, sizeof(FxItem) * size_t(B->cap_fx[o]), stream()), "batch");
+        if (rc == SEM_OK)
+            rc = cuda_check(cudaMemsetAsync(B->d_own[o], 0, sizeof(OwnerItem) * size_t(B->cap_own[o]), stream()), "batch");
+    }
+    if (rc != SEM_OK || ms.empty()) return rc;
+    rc = grow(&B->d_members, &B->cap_members, int(ms.size()));
+    if (rc == SEM_OK)
+        rc = cuda_check(cudaMemcpyAsync(B->d_members, ms.data(), sizeof(FxMember) * ms.size(), cudaMemcpyHostToDevice,
+                                        stream()), "batch: members");
+    if (rc != SEM_OK) return rc;
+    batch_fx_items_kernel<<<unsigned(ms.size()), 256, 0, stream()>>>(B->d_members);
+    count_launches(1);
+    rc = cuda_check(cudaGetLastError(), "batch_fx_items_kernel");
+    // the members come from pageable memory
+    return rc != SEM_OK ? rc : cuda_check(cudaStreamSynchronize(stream()), "batch: sync");
+}
+
+// Drops the captured round unless its buffers stayed in place and its
+// launches' grids still fit: equal ones, or, for the fixed-point orders, a
+// grid of at least the current blocks and at most twice as many (or 64 more:
+// the blocks beyond the lists find an empty item).
+static void keep_or_drop_graph(Batch *B) {
+    const void *bufs[7 + 2 * kOrders];
+    graph_buffers(B, bufs);
+    int ord_now[3 * kOrders];
+    order_signature(B, ord_now);
+    bool fits = true;
+    for (int o = 0; o < kOrders; ++o) {
+        if (B->ord_body[o] != kBodyFX) continue;
+        for (int u = 0; u < 2; ++u) {
+            const int now = u ? B->own_grid[o] : B->fx_grid[o], had = B->graph_fx[2 * o + u];
+            if (now > had || had > std::max(2 * now, now + 64)) fits = false;
+        }
+    }
+    if (B->graph && !(fits && std::equal(ord_now, ord_now + 3 * kOrders, B->graph_ord) &&
+                      std::equal(bufs, bufs + 7 + 2 * kOrders, B->graph_bufs))) {
+        cudaGraphExecDestroy(B->graph);
+        B->graph = nullptr;
     }
 }
 
@@ -994,7 +1222,9 @@ static int compact(Batch *B) {
     if (rc == SEM_OK) {
         B->n_ax = counts[0];
         B->n_vec = counts[1];
+        rc = build_fx_lists(B);
     }
+    if (rc == SEM_OK) keep_or_drop_graph(B);
     return rc;
 }
 
@@ -1039,6 +1269,7 @@ int batch_set(Batch *B, Problem **probs, const double *const *b, const uint8_t *
     std::vector<BatchItem> by_ord_v[kOrders]; // vector items likewise
     int ord_body[kOrders];
     std::fill(ord_body, ord_body + kOrders, int(kBodyNone));
+    int fx_epb[kOrders] = {};
     bool any_init = false;
     for (int k = 0; k < n && rc == SEM_OK; ++k) {
         Problem *P = probs[k];
@@ -1066,7 +1297,7 @@ int batch_set(Batch *B, Problem **probs, const double *const *b, const uint8_t *
         // operator body from the tuner's table; a pass of the line body fills
         // the engine's fixed 256-thread CTA (the table's elements per block
         // size stand-alone blocks, whose count per SM varies with it); an
-        // item holds several passes (~kAxItemNodes local nodes)
+        // item holds several passes (item_nodes)
         const int full = kBatchThreads / (P->nq * P->nq);
         const TuneChoice c = tune_get(B->mode == 0 ? kTuneF64 : (B->mode == 1 ? kTuneF32G16 : kTuneF32G32), P->nq);
         // the fixed-point variant: its line body in FP64 batches (factors
@@ -1076,14 +1307,17 @@ int batch_set(Batch *B, Problem **probs, const double *const *b, const uint8_t *
         if (fx) {
             rc = fx_prepare(P);
             if (rc != SEM_OK) break;
-            q.Gfx = P->Gfx;
-            q.kgfx = P->kgfx;
+            if (fx_epb[P->nq - 2] && fx_epb[P->nq - 2] != c.epb) {
+                rc = set_error(SEM_EARG, "batch: members of one order with different operator bodies");
+                break;
+            }
+            fx_epb[P->nq - 2] = c.epb;
         }
         const bool lines = c.variant == kAxLines || c.variant == kAxLinesPrefetch || c.variant == kAxLinesStaged ||
                            c.variant == kAxLinesFX;
         const int group = full;
         const int np = P->nq * P->nq * P->nq;
-        const int per_item = group * std::max(1, kAxItemNodes / (np * group));
+        const int per_item = group * std::max(1, item_nodes(P->nL) / (np * group));
         const int o = P->nq - 2;
         const int body = fx ? kBodyFX : (lines ? kBodyLines : kBodyColumns);
         if (ord_body[o] != kBodyNone && ord_body[o] != body) {
@@ -1096,7 +1330,7 @@ int batch_set(Batch *B, Problem **probs, const double *const *b, const uint8_t *
         for (int64_t e = 0; e < P->E; e += per_item)
             oa.push_back(BatchItem{k, P->nq, e, int(std::min<int64_t>(per_item, P->E - e)), lines ? group : 0});
         q.ax_count = int(oa.size()) - q.ax_first;
-        const int64_t chunk = std::max<int64_t>(P->nq, (kVecItemNodes / P->nq) * P->nq);
+        const int64_t chunk = std::max<int64_t>(P->nq, (item_nodes(P->nL) / P->nq) * P->nq);
         std::vector<BatchItem> &ov = by_ord_v[o];
         q.vec_first = int(ov.size());  // within its order's items; placed below
         for (int64_t l = 0; l < P->nL; l += chunk)
@@ -1117,6 +1351,7 @@ int batch_set(Batch *B, Problem **probs, const double *const *b, const uint8_t *
         hp[k].vec_first += ord_first[kOrders + probs[k]->nq - 2];
     }
     std::copy(ord_body, ord_body + kOrders, B->ord_body);
+    std::copy(fx_epb, fx_epb + kOrders, B->fx_epb);
     for (int o = 0; o < kOrders; ++o) {
         B->ord_count[o] = int(by_ord[o].size());
         B->ord_vcount[o] = int(by_ord_v[o].size());
@@ -1176,16 +1411,10 @@ int batch_set(Batch *B, Problem **probs, const double *const *b, const uint8_t *
     if (rc == SEM_OK) rc = upload_order_ranges(B, ord_first);
     if (rc == SEM_OK) rc = cuda_check(cudaStreamSynchronize(stream()), "batch: sync");
     B->seen_finished = 0;
+    if (rc == SEM_OK) rc = build_fx_lists(B);
     // the captured round reads the lists and counts from device memory: it
-    // is captured again only if a buffer moved (grew)
-    const void *bufs[7] = {B->d_probs, B->d_ax, B->d_vec, B->part, B->part_vec, B->tickets, B->finished_ids};
-    int ord_now[2 * kOrders];
-    order_signature(B, ord_now);
-    const bool same_grids = std::equal(ord_now, ord_now + 2 * kOrders, B->graph_ord);
-    if (B->graph && !(same_grids && std::equal(bufs, bufs + 7, B->graph_bufs))) {
-        cudaGraphExecDestroy(B->graph);
-        B->graph = nullptr;
-    }
+    // is captured again only if a buffer moved (grew) or a grid changed
+    if (rc == SEM_OK) keep_or_drop_graph(B);
     return rc;
 }
 
@@ -1200,6 +1429,11 @@ void batch_destroy(Batch *B) {
     void *ptrs[] = {B->d_probs, B->d_ax, B->d_vec, B->part, B->part_vec, B->tickets, B->finished_ids, B->ctl};
     for (void *q : ptrs)
         if (q) dev_free(q);
+    for (int o = 0; o < kOrders; ++o) {
+        if (B->d_fx[o]) dev_free(B->d_fx[o]);
+        if (B->d_own[o]) dev_free(B->d_own[o]);
+    }
+    if (B->d_members) dev_free(B->d_members);
     if (B->ctl_host) cudaFreeHost(B->ctl_host);
     delete B;
 }
@@ -1231,7 +1465,10 @@ static int capture(Batch *B) {
         const int nq = o + 2, body = B->ord_body[o], na = B->ord_count[o], nv = B->ord_vcount[o];
         int r = SEM_OK;
         for (int k = 0; k < B->K && r == SEM_OK; ++k) {
-            if (B->mode == 0) {
+            if (body == kBodyFX) {
+                r = fx_launch(B, nq, false, true);
+                if (r == SEM_OK) r = fx_launch(B, nq, true, true);
+            } else if (B->mode == 0) {
                 r = bax<double, double, 0>(B, nq, body, na, true);
                 if (r == SEM_OK) r = upd<kVecUpdate64>(B, nq, nv, true);
             } else {
@@ -1250,11 +1487,14 @@ static int capture(Batch *B) {
     if (g) cudaGraphDestroy(g);
     if (rc == SEM_OK) {
         B->graph_stream = stream();
-        const void *bufs[7] = {B->d_probs, B->d_ax, B->d_vec, B->part, B->part_vec, B->tickets, B->finished_ids};
-        std::copy(bufs, bufs + 7, B->graph_bufs);
+        graph_buffers(B, B->graph_bufs);
         B->graph_items[0] = items_grid(1 << 30, B->n_ax);
         B->graph_items[1] = items_grid(1 << 30, B->n_vec);
         order_signature(B, B->graph_ord);
+        for (int o = 0; o < kOrders; ++o) {
+            B->graph_fx[2 * o] = B->fx_grid[o];
+            B->graph_fx[2 * o + 1] = B->own_grid[o];
+        }
     }
     return rc;
 }
@@ -1374,6 +1614,15 @@ int batch_results_of(Batch *B, const std::vector<int> &which, int64_t *iters, do
     return SEM_OK;
 }
 
+// A finished member's solution: the fixed-point orders defer x += alpha p to
+// the next operator launch, so the last one is applied here.
+int batch_emit_x(const Batch *B, int k, double *out) {
+    const Problem *P = B->probs[k];
+    if (B->ord_body[P->nq - 2] == kBodyFX) return launch_x_finish(P, out);
+    return cuda_check(cudaMemcpyAsync(out, P->x, sizeof(double) * P->nL, cudaMemcpyDeviceToDevice, stream()),
+                      "batch: copy x");
+}
+
 // Fixed batch: every problem starts now; rounds until all have finished.
 int batch_solve(Batch *B, const double *b_all, double *x_all, double tol, int maxit, int mode, double inner_tol,
                 int max_outer, int64_t *iters, double *res) {
@@ -1407,8 +1656,7 @@ int batch_solve(Batch *B, const double *b_all, double *x_all, double tol, int ma
     if (rc != SEM_OK) return rc;
     off = 0;
     for (int k = 0; k < n && rc == SEM_OK; ++k) {
-        rc = cuda_check(cudaMemcpyAsync(x_all + off, ps[k]->x, sizeof(double) * ps[k]->nL, cudaMemcpyDeviceToDevice,
-                                        stream()), "batch: copy x");
+        rc = batch_emit_x(B, k, x_all + off);
         off += ps[k]->nL;
     }
     if (rc != SEM_OK) return rc;

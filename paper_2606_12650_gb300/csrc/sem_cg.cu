@@ -167,15 +167,15 @@ int launch_cg_init(const Problem *P, const double *b, int maxit, double tol, dou
 // The last iteration's x += alpha p: the FP64 CG operator kernel applies an
 // iteration's x update at the start of the next iteration (it holds p there
 // anyway); the iteration that stopped the solve has no next one.
-__global__ void x_finish_kernel(double *__restrict__ x, const double *__restrict__ p, const CgState *st,
+__global__ void x_finish_kernel(const double *x, const double *__restrict__ p, double *out, const CgState *st,
                                 int64_t n) {
     const double alpha = st->alpha;
     for (int64_t l = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; l < n; l += int64_t(gridDim.x) * blockDim.x)
-        x[l] = fma(alpha, p[l], x[l]);
+        out[l] = fma(alpha, p[l], x[l]);
 }
 
-int launch_x_finish(const Problem *P) {
-    x_finish_kernel<<<stream_grid(P->nL), kThreads, 0, stream()>>>(P->x, P->p, P->st, P->nL);
+int launch_x_finish(const Problem *P, double *out) {
+    x_finish_kernel<<<stream_grid(P->nL), kThreads, 0, stream()>>>(P->x, P->p, out, P->st, P->nL);
     count_launches(1);
     return cuda_check(cudaGetLastError(), "x_finish_kernel");
 }
@@ -245,13 +245,10 @@ int cg_solve(Problem *P, const double *b, double *x, double tol, int maxit, doub
         if (*status_host() != 0) break;
         if (P->st_host->done) break;
     }
-    rc = launch_x_finish(P);
+    rc = launch_x_finish(P, x);
     if (rc == SEM_OK)
         rc = cuda_check(cudaMemcpyAsync(P->st_host, P->st, sizeof(CgState), cudaMemcpyDeviceToHost, stream()),
                         "cg: state read");
-    if (rc == SEM_OK && x != P->x)
-        rc = cuda_check(cudaMemcpyAsync(x, P->x, sizeof(double) * P->nL, cudaMemcpyDeviceToDevice, stream()),
-                        "cg: copy x");
     if (rc == SEM_OK) rc = cuda_check(cudaStreamSynchronize(stream()), "cg: sync");
     if (rc != SEM_OK) return rc;
     rc = poll_status();

@@ -212,12 +212,13 @@ __device__ __forceinline__ double finish_partials(const double *partials, int n,
 // then sums the group sums in order.  The FP64 additions of the grid sum are
 // spread over the groups' last blocks instead of all falling on one block at
 // the end of the launch (on GB300 FP64 runs at 1/64 of the FP32 rate).
-__device__ __forceinline__ bool publish_grouped(double v0, double *partials, uint32_t *ticket) {
+// Block b of nb (a launch's own blocks, or the blocks of one problem of a batch).
+__device__ __forceinline__ bool publish_grouped(double v0, double *partials, uint32_t *ticket, int b, int nb) {
     __shared__ int s_last;
     const int64_t cap = partials_capacity(partials);
     uint32_t *gt = group_tickets(partials, cap);
-    const int b = int(blockIdx.x), g = b / kSumGroup, g0 = g * kSumGroup;
-    const int gn = min(kSumGroup, int(gridDim.x) - g0);
+    const int g = b / kSumGroup, g0 = g * kSumGroup;
+    const int gn = min(kSumGroup, nb - g0);
     if (threadIdx.x == 0) {
         partials[b] = v0;
         __threadfence();
@@ -235,12 +236,16 @@ __device__ __forceinline__ bool publish_grouped(double v0, double *partials, uin
             partials[cap + g] = s;
             gt[g] = 0u;
             __threadfence();
-            const uint32_t ng = (gridDim.x + kSumGroup - 1) / kSumGroup;
+            const uint32_t ng = uint32_t(nb + kSumGroup - 1) / kSumGroup;
             s_last = atomicAdd(ticket, 1u) == ng - 1;
         }
     }
     __syncthreads();
     return s_last != 0;
+}
+
+__device__ __forceinline__ bool publish_grouped(double v0, double *partials, uint32_t *ticket) {
+    return publish_grouped(v0, partials, ticket, int(blockIdx.x), int(gridDim.x));
 }
 
 // Zero the group tickets (grid-stride): at the start of every solve, so that
@@ -255,11 +260,11 @@ __device__ __forceinline__ void reset_group_tickets(double *partials) {
 
 // In the block for which publish_grouped returned true: the sum of the group
 // sums in a fixed order (one warp), the grid ticket reset.  Result in thread 0.
-__device__ __forceinline__ double finish_grouped(const double *partials, uint32_t *ticket) {
+__device__ __forceinline__ double finish_grouped(const double *partials, uint32_t *ticket, int nb) {
     double s = 0.0;
     if (threadIdx.x < 32) {
         __threadfence();
-        const int ng = int((gridDim.x + kSumGroup - 1) / kSumGroup);
+        const int ng = (nb + kSumGroup - 1) / kSumGroup;
         const int64_t cap = partials_capacity(partials);
         for (int q = threadIdx.x; q < ng; q += 32) s += __ldcg(partials + cap + q);
 #pragma unroll
@@ -267,6 +272,10 @@ __device__ __forceinline__ double finish_grouped(const double *partials, uint32_
         if (threadIdx.x == 0) *ticket = 0u;
     }
     return s;
+}
+
+__device__ __forceinline__ double finish_grouped(const double *partials, uint32_t *ticket) {
+    return finish_grouped(partials, ticket, int(gridDim.x));
 }
 
 // Block sum of FP32 values in FP32: fixed shuffle tree per warp, then the

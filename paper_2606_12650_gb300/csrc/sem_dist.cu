@@ -393,7 +393,7 @@ int dist_cg_solve(DistProblem *D, const double *b, double *x, double tol, int ma
         if (hist) hist[k] = std::sqrt(rho);
         if (tol > 0.0 && std::sqrt(rho / rho0) <= tol) break;
     }
-    rc = launch_x_finish(P);   // x += alpha p of the last iteration
+    rc = launch_x_finish(P, P->x);   // x += alpha p of the last iteration
     if (rc == SEM_OK && x != P->x)
         rc = cuda_check(cudaMemcpyAsync(x, P->x, sizeof(double) * size_t(P->nL), cudaMemcpyDeviceToDevice, stream()),
                         "dist: copy x");

@@ -241,7 +241,7 @@ int launch_dot(const Problem *P, const double *u, const double *v);  // -> st->d
 int launch_sub(const Problem *P, const double *a, const double *b, double *out);  // out = a - b
 int launch_cg_init(const Problem *P, const double *b, int maxit, double tol, double *hist);
 int launch_cg_update(const Problem *P);
-int launch_x_finish(const Problem *P);       // x += alpha p of the last iteration (deferred update)
+int launch_x_finish(const Problem *P, double *out);   // out = x + alpha p of the last iteration (deferred update)
 int cg_solve(Problem *P, const double *b, double *x, double tol, int maxit, double *hist,
              int64_t *iters, double *rel_res);
 int launch_ax_pcg(const Problem *P);         // p = dinv r + beta p; w = A_local p; <p,w>
@@ -258,6 +258,7 @@ int batch_round_launch(Batch *B);                       // the round's launches,
 int batch_round_finish(Batch *B, std::vector<int> *done);   // wait, finished problems
 int batch_results(Batch *B, int64_t *iters, double *res);
 int batch_results_of(Batch *B, const std::vector<int> &which, int64_t *iters, double *res);
+int batch_emit_x(const Batch *B, int k, double *out);   // a finished member's solution
 int batch_create(Problem **probs, int n, Batch **out);
 void batch_destroy(Batch *B);
 int64_t batch_total_nodes(const Batch *B);

@@ -216,13 +216,10 @@ int pcg_solve(Problem *P, const double *b, double *x, double tol, int maxit, dou
         if (rc != SEM_OK) return rc;
         if (*status_host() != 0 || P->st_host->done) break;
     }
-    rc = launch_x_finish(P);   // the last iteration's deferred x += alpha p
+    rc = launch_x_finish(P, x);   // the last iteration's deferred x += alpha p
     if (rc == SEM_OK)
         rc = cuda_check(cudaMemcpyAsync(P->st_host, P->st, sizeof(CgState), cudaMemcpyDeviceToHost, stream()),
                         "pcg: state read");
-    if (rc == SEM_OK && x != P->x)
-        rc = cuda_check(cudaMemcpyAsync(x, P->x, sizeof(double) * P->nL, cudaMemcpyDeviceToDevice, stream()),
-                        "pcg: copy x");
     if (rc == SEM_OK) rc = cuda_check(cudaStreamSynchronize(stream()), "pcg: sync");
     if (rc == SEM_OK) rc = poll_status();
     if (rc != SEM_OK) return rc;

@@ -275,8 +275,7 @@ static int retire(Server *S, const std::vector<int> &done) {
         ServeReq *q = S->active[k];
         q->x_dev = static_cast<double *>(dev_alloc(sizeof(double) * q->nL));
         if (!q->x_dev) return SEM_ENOMEM;
-        rc = cuda_check(cudaMemcpyAsync(q->x_dev, q->P->x, sizeof(double) * q->nL, cudaMemcpyDeviceToDevice,
-                                        stream()), "serve: result");
+        rc = batch_emit_x(S->B, k, q->x_dev);
         if (rc != SEM_OK) return rc;
         q->iters = its[j];
         q->res = res[j];
