@@ -415,8 +415,7 @@ int run_ax(ArgReader &R, bool assembled) {
     if (R.err) return R.err;
     if (x == y) return R.fail(SEM_EARG, "x and y must not alias");
     int rc = launch_ax(P, x, y);
-    if (rc == SEM_OK && assembled) rc = launch_gs(P, y);
-    if (rc == SEM_OK && assembled) rc = launch_mask(P, y);
+    if (rc == SEM_OK && assembled) rc = launch_gs_mask(P, y);
     return rc;
 }
 
@@ -506,8 +505,7 @@ int run_rhs(ArgReader &R, bool sin_source) {
     double *b = static_cast<double *>(R.arr(2, vb, "b"));
     if (R.err) return R.err;
     int rc = launch_scale(P, P->B, f, b);
-    if (rc == SEM_OK) rc = launch_gs(P, b);
-    if (rc == SEM_OK) rc = launch_mask(P, b);
+    if (rc == SEM_OK) rc = launch_gs_mask(P, b);
     return rc;
 }
 
@@ -1040,8 +1038,7 @@ int run_true_res(ArgReader &R) {
     double *w = P->w, *r = P->r;
     if (x == w || x == r || b == w || b == r) return R.fail(SEM_EARG, "arguments alias work vectors");
     int rc = launch_ax(P, x, w);
-    if (rc == SEM_OK) rc = launch_gs(P, w);
-    if (rc == SEM_OK) rc = launch_mask(P, w);
+    if (rc == SEM_OK) rc = launch_gs_mask(P, w);
     if (rc == SEM_OK) rc = launch_sub(P, b, w, r);
     double rr = 0.0, bb = 0.0;
     for (int pass = 0; pass < 2 && rc == SEM_OK; ++pass) {

@@ -3,7 +3,7 @@
 //
 // Gather-scatter (the paper's "gs" kernel, Section V-B: an outer loop over
 // global ids split across blocks and threads, and order-enforced inner loops
-// over the copies).  Each thread owns one global id that has two or more
+// over the copies).  Each thread owns one global node that has two or more
 // copies; it adds the copies in ascending local index and writes the sum back
 // to each.  There are no floating-point atomics, so the result does not
 // depend on scheduling and matches an ascending sequential sum bit for bit.
@@ -48,14 +48,139 @@ static unsigned grid_for(int64_t n, int threads) {
 }
 
 // ---------------------------------------------------------------- gs / mask
-__global__ void gs_kernel(double *__restrict__ u, const int32_t *__restrict__ ptr,
-                          const int32_t *__restrict__ idx, int64_t nseg) {
-    const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (t >= nseg) return;
-    const int32_t b0 = ptr[t], b1 = ptr[t + 1];
-    double s = u[idx[b0]];
-    for (int32_t q = b0 + 1; q < b1; ++q) s += u[idx[q]];
-    for (int32_t q = b0; q < b1; ++q) u[idx[q]] = s;
+// u = QQ^T u, or mask(QQ^T u), in place.  A global node's first copy (no
+// neighbour across a low face) adds its copies -- per direction its own
+// element and, across a high face, the next one -- in ascending local index
+// and writes the sum to each: every value is read and written by that one
+// thread.  The copies follow from the box structure, so no index lists are
+// read.  One thread per node on an element's high faces, in the order all
+// faces (1 addition), all edges (3), all corners (7): a warp runs the
+// additions of one class (predicated off they would cost as much on the
+// 1/64-rate FP64 pipe: 200 us at E = 32^3, N = 7 with one thread per node and
+// all seven, 66 us from index lists plus 4 us for the mask's).  MASK: nodes of
+// the cube's high faces are zeroed by their own thread, those of its low faces
+// by the last NQ^2 (ny nz + nx nz + nx ny) threads.
+template <int M>
+__device__ __forceinline__ void sum_copies(double *u, const int (&o)[M]) {
+    constexpr int C = 1 << M;
+    double v[C];
+    int at[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        at[c] = 0;
+#pragma unroll
+        for (int d = 0; d < M; ++d)
+            if (c >> d & 1) at[c] += o[d];
+        v[c] = u[at[c]];
+    }
+    double s = v[0];
+#pragma unroll
+    for (int c = 1; c < C; ++c) s += v[c];
+#pragma unroll
+    for (int c = 0; c < C; ++c) u[at[c]] = s;
+}
+
+template <int NQ, bool MASK>
+__global__ void __launch_bounds__(256) gs_box_kernel(double *__restrict__ u, int64_t E, BoxDims bd, int64_t total) {
+    constexpr int N = NQ - 1, N2 = N * N, NQ2 = NQ * NQ, NP = NQ2 * NQ;
+    const int64_t t64 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (t64 >= total) return;
+    const unsigned nE = unsigned(E);
+    unsigned t = unsigned(t64), e;
+    int c[3], m;                       // (i, j, k), the number of them at N by class
+    if (t < nE * (3 * N2)) {           // faces
+        e = t / (3 * N2);
+        const int f = int(t - e * (3 * N2)), d = f / N2, r = f - d * N2, q = r / N, p = r - q * N;
+        c[0] = d == 0 ? N : p;
+        c[1] = d == 1 ? N : (d == 0 ? p : q);
+        c[2] = d == 2 ? N : q;
+        m = 1;
+    } else if ((t -= nE * (3 * N2)) < nE * (3 * N)) {   // edges
+        e = t / (3 * N);
+        const int f = int(t - e * (3 * N)), d = f / N, p = f - d * N;
+        c[0] = d == 0 ? p : N;
+        c[1] = d == 1 ? p : N;
+        c[2] = d == 2 ? p : N;
+        m = 2;
+    } else if ((t -= nE * (3 * N)) < nE) {              // corners
+        e = t;
+        c[0] = c[1] = c[2] = N;
+        m = 3;
+    } else {                                            // MASK: the cube's low faces
+        t -= nE;
+        const unsigned yz = unsigned(bd.ny * bd.nz) * NQ2, xz = unsigned(bd.nx * bd.nz) * NQ2;
+        const int d = t < yz ? 0 : (t < yz + xz ? 1 : 2);
+        if (d) t -= d == 1 ? yz : yz + xz;
+        const unsigned g = t / NQ2;
+        const int r = int(t - g * NQ2), q = r / NQ, p = r - q * NQ;
+        const unsigned n0 = unsigned(d == 0 ? bd.ny : bd.nx);
+        const unsigned h = g / n0, a = g - h * n0;
+        e = d == 0 ? a * unsigned(bd.nx) + h * unsigned(bd.nx * bd.ny)
+                   : (d == 1 ? a + h * unsigned(bd.nx * bd.ny) : a + h * unsigned(bd.nx));
+        const int i = d == 0 ? 0 : p, j = d == 1 ? 0 : (d == 0 ? p : q), k = d == 2 ? 0 : q;
+        u[int64_t(e) * NP + k * NQ2 + j * NQ + i] = 0.0;
+        return;
+    }
+    const unsigned g = divu(e, bd.dx);
+    const int ex = int(e - g * unsigned(bd.nx));
+    const unsigned tz = divu(g, bd.dy);
+    const int ey = int(g - tz * unsigned(bd.ny)), ez = int(tz);
+    const int pos[3] = {ex, ey, ez}, top[3] = {bd.nx - 1, bd.ny - 1, bd.nz - 1};
+    const int off[3] = {NP - N, bd.nx * NP - N * NQ, bd.nx * bd.ny * NP - N * NQ2};
+    double *v = u + int64_t(e) * NP + c[2] * NQ2 + c[1] * NQ + c[0];
+    int o[3], n = 0;                   // offsets across the high faces with a neighbour, r first
+    bool low = false, edge = false;    // a copy below; on a low face of the cube
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        if (c[d] == 0) (pos[d] > 0 ? low : edge) = true;
+        if (c[d] == N && pos[d] < top[d]) {
+            o[2] = n == 2 ? off[d] : 0;
+            if (n == 1) o[1] = off[d];
+            if (n == 0) o[0] = off[d];
+            ++n;
+        }
+    }
+    if (MASK) {
+        if (n < m) {                   // on a high face of the cube
+            *v = 0.0;
+            return;
+        }
+        if (edge) return;
+    }
+    if (low || n == 0) return;
+    if (n == 1) sum_copies<1>(v, {o[0]});
+    else if (n == 2) sum_copies<2>(v, {o[0], o[1]});
+    else sum_copies<3>(v, {o[0], o[1], o[2]});
+}
+
+template <int NQ>
+static int launch_gs_nq(const Problem *P, double *u, bool mask) {
+    const BoxDims bd = box_dims(P->nx, P->ny, P->nz);
+    constexpr int N = NQ - 1;
+    const int64_t nx = P->nx, ny = P->ny, nz = P->nz;
+    int64_t total = P->E * (3 * N * N + 3 * N + 1);
+    if (mask) total += NQ * NQ * (ny * nz + nx * nz + nx * ny);
+    if (mask)
+        gs_box_kernel<NQ, true><<<grid_for(total, kThreads), kThreads, 0, stream()>>>(u, P->E, bd, total);
+    else
+        gs_box_kernel<NQ, false><<<grid_for(total, kThreads), kThreads, 0, stream()>>>(u, P->E, bd, total);
+    count_launches(1);
+    return cuda_check(cudaGetLastError(), "gs_box_kernel");
+}
+
+static int launch_gs_any(const Problem *P, double *u, bool mask) {
+    switch (P->nq) {
+        case 2: return launch_gs_nq<2>(P, u, mask);
+        case 3: return launch_gs_nq<3>(P, u, mask);
+        case 4: return launch_gs_nq<4>(P, u, mask);
+        case 5: return launch_gs_nq<5>(P, u, mask);
+        case 6: return launch_gs_nq<6>(P, u, mask);
+        case 7: return launch_gs_nq<7>(P, u, mask);
+        case 8: return launch_gs_nq<8>(P, u, mask);
+        case 9: return launch_gs_nq<9>(P, u, mask);
+        case 10: return launch_gs_nq<10>(P, u, mask);
+        default: return set_error(SEM_EARG, "gs: unsupported order");
+    }
 }
 
 __global__ void mask_kernel(double *__restrict__ u, const int32_t *__restrict__ idx, int64_t n) {
@@ -63,12 +188,8 @@ __global__ void mask_kernel(double *__restrict__ u, const int32_t *__restrict__ 
     if (t < n) u[idx[t]] = 0.0;
 }
 
-int launch_gs(const Problem *P, double *u) {
-    if (P->n_sh == 0) return SEM_OK;
-    gs_kernel<<<grid_for(P->n_sh, kThreads), kThreads, 0, stream()>>>(u, P->sh_ptr, P->sh_idx, P->n_sh);
-    count_launches(1);
-    return cuda_check(cudaGetLastError(), "gs_kernel");
-}
+int launch_gs(const Problem *P, double *u) { return launch_gs_any(P, u, false); }
+int launch_gs_mask(const Problem *P, double *u) { return launch_gs_any(P, u, true); }
 
 int launch_mask(const Problem *P, double *u) {
     if (P->n_mask == 0) return SEM_OK;

@@ -237,6 +237,7 @@ int mixed_solve(Problem *P, const double *b, double *x, double tol, int max_oute
 void mixed_release(Problem *P);
 int launch_gs(const Problem *P, double *u);
 int launch_mask(const Problem *P, double *u);
+int launch_gs_mask(const Problem *P, double *u);   // mask(QQ^T u), one pass
 int launch_dot(const Problem *P, const double *u, const double *v);  // -> st->dot_out
 int launch_sub(const Problem *P, const double *a, const double *b, double *out);  // out = a - b
 int launch_cg_init(const Problem *P, const double *b, int maxit, double tol, double *hist);

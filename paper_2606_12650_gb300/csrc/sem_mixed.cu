@@ -198,8 +198,7 @@ int mixed_solve(Problem *P, const double *b, double *x, double tol, int max_oute
         rc = cuda_check(cudaGetLastError(), "mixed_correct_kernel");
         // true residual in FP64: r = b - mask(QQ^T(A_local x))
         if (rc == SEM_OK) rc = launch_ax(P, P->x, P->w);
-        if (rc == SEM_OK) rc = launch_gs(P, P->w);
-        if (rc == SEM_OK) rc = launch_mask(P, P->w);
+        if (rc == SEM_OK) rc = launch_gs_mask(P, P->w);
         if (rc == SEM_OK) rc = launch_sub(P, b, P->w, P->r);
         if (rc == SEM_OK) rc = launch_dot(P, P->r, P->r);
         if (rc == SEM_OK) rc = read_state(P->st_host, P->st);

@@ -69,8 +69,7 @@ int jacobi_prepare(Problem *P) {
     local_diag_kernel<<<blocks, 256, 0, stream()>>>(a);
     count_launches(1);
     int rc = cuda_check(cudaGetLastError(), "local_diag_kernel");
-    if (rc == SEM_OK) rc = launch_gs(P, P->dinv);
-    if (rc == SEM_OK) rc = launch_mask(P, P->dinv);
+    if (rc == SEM_OK) rc = launch_gs_mask(P, P->dinv);
     if (rc == SEM_OK) {
         invert_kernel<<<blocks, 256, 0, stream()>>>(P->dinv, P->nL);
         count_launches(1);

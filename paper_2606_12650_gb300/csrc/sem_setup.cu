@@ -242,8 +242,7 @@ int launch_rhs_sin(const Problem *P, const double *verts, double *b) {
         count_launches(1);
         rc = cuda_check(cudaGetLastError(), "rhs_sin_kernel");
     }
-    if (rc == SEM_OK) rc = launch_gs(P, b);
-    if (rc == SEM_OK) rc = launch_mask(P, b);
+    if (rc == SEM_OK) rc = launch_gs_mask(P, b);
     cudaStreamSynchronize(stream());
     dev_free(X);
     return rc;
