@@ -98,9 +98,8 @@ static int launch_fx_nq(const Problem *Pb, const AxFxArgs &L) {
     }
     const int64_t blocks = (Pb->E + L.epb - 1) / L.epb;
     if (CG && blocks > Pb->partials_cap) return set_error(SEM_ERANGE, "ax fx: more blocks than reduction slots");
-    kern<<<unsigned(blocks), nt, sm, stream()>>>(L);
     count_launches(1);
-    return cuda_check(cudaGetLastError(), "ax_fx_kernel");
+    return cuda_check(launch_pdl(kern, unsigned(blocks), unsigned(nt), sm, L), "ax_fx_kernel");
 }
 
 template <bool CG, bool PRE>

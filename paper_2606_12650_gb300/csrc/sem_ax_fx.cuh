@@ -193,6 +193,14 @@ struct AxFxArgs {
     int epb;                    // elements per block
 };
 
+// Starts the factors of ne elements from e0, half of the traffic, towards L2
+// (before pdl_wait: no kernel of a solve writes them).
+template <int NQ>
+__device__ __forceinline__ void fx_prefetch(const int4 *G, int64_t e0, int ne) {
+    constexpr int NP = NQ * NQ * NQ;
+    if (threadIdx.x == 0) bulk_prefetch_l2(G + e0 * (3 * NP), uint32_t(ne) * uint32_t(3 * NP * sizeof(int4)));
+}
+
 // The integer factors of one node, from `q` (its element's first plane of
 // 16-byte pairs, at the node) with planes NP apart: lanes are consecutive
 // nodes, so each load of a warp is one contiguous run.
@@ -211,8 +219,7 @@ __device__ __forceinline__ void load_g6_fx(const int4 *q, int4 (&g)[3]) {
 //
 // Each thread loads and converts its own t line (coalesced: lanes are
 // consecutive nodes of a plane), so the vectors need no staging: 2 or 3 loads
-// per node are in flight per thread before the first barrier.  The factors,
-// half of the traffic, start towards L2 at once.
+// per node are in flight per thread before the first barrier.
 template <int NQ, bool CG, bool PRE>
 __device__ __forceinline__ void lines_group_fx(const double *x, double *y, double *p, const int4 *G,
                                                const int32_t *kg, const EoMatFX &cd, const EoMatFX &ct, double beta,
@@ -247,7 +254,6 @@ __device__ __forceinline__ void lines_group_fx(const double *x, double *y, doubl
     };
     auto word_of = [&]() { return WHOLE ? tid >> 5 : eb * MW + (tid >> 5) - (eb * NQ2 >> 5); };
     auto words = [&]() { return WHOLE ? MW : (((eb + 1) * NQ2 - 1) >> 5) - (eb * NQ2 >> 5) + 1; };
-    if (tid == 0) bulk_prefetch_l2(G + e0 * (3 * NP), uint32_t(ne) * uint32_t(3 * NP * sizeof(int4)));
 
     // ---- (0) the thread's t line, and the element's largest exponent
     double v[NQ];
@@ -259,13 +265,14 @@ __device__ __forceinline__ void lines_group_fx(const double *x, double *y, doubl
             double pv[NQ];
 #pragma unroll
             for (int k = 0; k < NQ; ++k) {
-                pv[k] = p[nb + k * NQ2];
-                v[k] = PRE ? dinv[nb + k * NQ2] * x[nb + k * NQ2] : x[nb + k * NQ2];
+                pv[k] = __ldcg(p + nb + k * NQ2);   // from L2, see vload_cg in sem_box.cuh
+                v[k] = __ldcg(x + nb + k * NQ2);
+                if (PRE) v[k] *= __ldg(dinv + nb + k * NQ2);
             }
             if (xs) {
                 double xv[NQ];
 #pragma unroll
-                for (int k = 0; k < NQ; ++k) xv[k] = xs[nb + k * NQ2];
+                for (int k = 0; k < NQ; ++k) xv[k] = __ldcg(xs + nb + k * NQ2);
 #pragma unroll
                 for (int k = 0; k < NQ; ++k) xs[nb + k * NQ2] = fma(xalpha, pv[k], xv[k]);
             }
@@ -276,7 +283,7 @@ __device__ __forceinline__ void lines_group_fx(const double *x, double *y, doubl
             }
         } else {
 #pragma unroll
-            for (int k = 0; k < NQ; ++k) v[k] = x[nb + k * NQ2];
+            for (int k = 0; k < NQ; ++k) v[k] = __ldcg(x + nb + k * NQ2);
         }
 #pragma unroll
         for (int k = 0; k < NQ; ++k) mx = max(mx, uint32_t(__double2hiint(v[k])) & 0x7fffffffu);
@@ -436,8 +443,8 @@ __device__ __forceinline__ void lines_group_fx(const double *x, double *y, doubl
 // Block b of nb after lines_group_fx: the block's <p, A_local p>, and in the
 // last block alpha = rho / <p, A p>.
 template <int NQ>
-__device__ __forceinline__ void fx_publish(double part, unsigned char *smem, int epb, double *partials, CgState *st,
-                                           int b, int nb) {
+__device__ __forceinline__ void fx_publish(double part, unsigned char *smem, int epb, double *partials, int64_t cap,
+                                           CgState *st, int b, int nb) {
     double bs = part;
     if (epb > 1) {
         // the regions are free: every thread passed lines_group_fx's last barrier after its reads
@@ -453,12 +460,10 @@ __device__ __forceinline__ void fx_publish(double part, unsigned char *smem, int
                 if (o < epb) bs += __shfl_down_sync(0xffffffffu, bs, o);
         }
     }
-    if (publish_grouped(bs, partials, &st->ticket_ax, b, nb)) {
-        const double pap = finish_grouped(partials, &st->ticket_ax, nb);
-        if (threadIdx.x == 0) {
-            st->pap = pap;
-            st->alpha = st->rho / pap;
-        }
+    double pap;
+    if (grid_sum(bs, partials, cap, &st->ticket_ax, b, nb, &pap) && threadIdx.x == 0) {
+        st->pap = pap;
+        st->alpha = st->rho / pap;
     }
 }
 
@@ -466,16 +471,19 @@ template <int NQ, bool CG, bool PRE>
 __global__ void __maxnreg__(FxRegs<NQ>::value) ax_fx_kernel(const __grid_constant__ AxFxArgs P) {
     extern __shared__ __align__(16) unsigned char smem[];
     const AxArgs<double, double> &A = P.a;
-    if (CG && A.st->done) return;  // solve finished: the rest of the graph is a no-op
     const int64_t e0 = int64_t(blockIdx.x) * P.epb;
     const int ne = int(min(int64_t(P.epb), A.E - e0));
+    if (!CG) fx_prefetch<NQ>(P.G, e0, ne);
+    pdl_wait();
+    if (CG && A.st->done) return;  // solve finished: the rest of the graph is a no-op
+    if (CG) fx_prefetch<NQ>(P.G, e0, ne);
     const double beta = CG ? A.st->beta : 0.0;
     // read before this launch's last block replaces it; only with a deferred x update
     const double xalpha = (CG && A.xs) ? A.st->alpha : 0.0;
     double part = 0.0;
     lines_group_fx<NQ, CG, PRE>(A.x, A.y, A.p, P.G, P.kg, P.d, P.dt, beta, xalpha, CG ? A.xs : nullptr, A.dinv, e0, ne,
                                 P.epb, smem, &part);
-    if (CG) fx_publish<NQ>(part, smem, P.epb, A.partials, A.st, int(blockIdx.x), int(gridDim.x));
+    if (CG) fx_publish<NQ>(part, smem, P.epb, A.partials, A.cap, A.st, int(blockIdx.x), int(gridDim.x));
 }
 
 // Host: the even-odd halves of M (row-major nq x nq) times 2^k, rounded to

@@ -51,6 +51,7 @@ struct AxArgs {
     T *xs;              // CG: solution, updated x += alpha p_old before p is replaced
                         // (the previous iteration's x update, deferred); nullptr: none
     int64_t E;
+    int64_t cap;        // slots of `partials`
     T D[kMaxQ * kMaxQ];
 };
 
@@ -254,12 +255,11 @@ ax_kernel(const AxArgs<T, GT> P) {
         // the column's partial is formed in T; the block and grid sums are FP64
         // (the grid sum over groups of blocks)
         const double bs = block_sum(double(part), red);
-        if (publish_grouped(bs, P.partials, &P.st->ticket_ax)) {
-            const double pap = finish_grouped(P.partials, &P.st->ticket_ax);
-            if (threadIdx.x == 0) {
-                P.st->pap = pap;
-                P.st->alpha = P.st->rho / pap;
-            }
+        double pap;
+        if (grid_sum(bs, P.partials, P.cap, &P.st->ticket_ax, int(blockIdx.x), int(gridDim.x), &pap) &&
+            threadIdx.x == 0) {
+            P.st->pap = pap;
+            P.st->alpha = P.st->rho / pap;
         }
     }
 }
@@ -341,6 +341,7 @@ static AxArgs<T, GT> ax_args(const Problem *Pb, const GT *G, double *partials, C
     a.E = Pb->E;
     a.status = status_word();
     a.partials = partials;
+    a.cap = Pb->partials_cap;
     a.st = st;
     for (int q = 0; q < Pb->nq * Pb->nq; ++q) a.D[q] = T(Pb->oc.D[q]);
     return a;

@@ -398,12 +398,11 @@ __global__ void __launch_bounds__(512) ax_lines_kernel(const AxLineArgs<T, GT> P
             bs = double(block_sum_f32(part, reinterpret_cast<float *>(regA)));
         else
             bs = block_sum_wide(double(part), reinterpret_cast<double *>(regA));
-        if (publish_grouped(bs, A.partials, &A.st->ticket_ax)) {
-            const double pap = finish_grouped(A.partials, &A.st->ticket_ax);
-            if (threadIdx.x == 0) {
-                A.st->pap = pap;
-                A.st->alpha = A.st->rho / pap;
-            }
+        double pap;
+        if (grid_sum(bs, A.partials, A.cap, &A.st->ticket_ax, int(blockIdx.x), int(gridDim.x), &pap) &&
+            threadIdx.x == 0) {
+            A.st->pap = pap;
+            A.st->alpha = A.st->rho / pap;
         }
     }
 }

@@ -108,6 +108,7 @@ struct FxItem {                     // operator: ne elements from e0
     double *partials;
     int e0, ne;                     // ne = 0: beyond the list
     int b, nb;                      // block b of the problem's nb
+    int64_t cap;                    // slots of `partials`
 };
 struct OwnerItem {                  // update: warps 8 b .. 8 b + 7 of the problem's 8 nb
     double *r;
@@ -117,6 +118,7 @@ struct OwnerItem {                  // update: warps 8 b .. 8 b + 7 of the probl
     BoxDims bd;
     int E, b, nb;                   // nb = 0: beyond the list
     int prob;
+    int64_t cap;
 };
 struct FxMember {                   // a member's ranges in its order's lists
     FxItem op;                      // e0, ne, b unset
@@ -174,12 +176,14 @@ struct FxBatchArgs {
 template <int NQ>
 __global__ void __maxnreg__(FxRegs<NQ>::value) batch_fx_kernel(const __grid_constant__ FxBatchArgs P) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const FxItem it = P.items[blockIdx.x];
+    const FxItem it = P.items[blockIdx.x];   // the lists do not change within a round
+    pdl_wait();
     if (it.ne == 0 || it.st->done) return;
+    fx_prefetch<NQ>(it.G, it.e0, it.ne);
     double part = 0.0;
     lines_group_fx<NQ, true, false>(it.r, it.w, it.p, it.G, it.kg, P.d, P.dt, it.st->beta, it.st->alpha, it.x, nullptr,
                                     it.e0, it.ne, P.epb, smem, &part);
-    fx_publish<NQ>(part, smem, P.epb, it.partials, it.st, it.b, it.nb);
+    fx_publish<NQ>(part, smem, P.epb, it.partials, it.cap, it.st, it.b, it.nb);
 }
 constexpr int kOrders = kMaxQ - 1;  // N+1 = 2 .. kMaxQ
 
@@ -682,17 +686,16 @@ __global__ void __launch_bounds__(256, kOwnerBlocks)
     batch_owner_kernel(const OwnerItem *items, BatchProb *probs, BatchCtl *ctl, int32_t *finished_ids) {
     __shared__ double scratch[256];
     const OwnerItem it = items[blockIdx.x];
+    pdl_wait();
     if (it.nb == 0 || it.st->done) return;
     DwAcc acc = acc_zero<DwAcc>(), unused = acc_zero<DwAcc>();
     owner_tasks<NQ, false>(it.r, it.w, nullptr, 8 * it.b + int(threadIdx.x >> 5), 8 * it.nb, it.E, it.bd, it.st->alpha,
                            acc, unused);
     const double bs = block_sum_wide(acc_value(acc), scratch);
-    if (publish_grouped(bs, it.partials, &it.st->ticket_up, it.b, it.nb)) {
-        const double rho_new = finish_grouped(it.partials, &it.st->ticket_up, it.nb);
-        if (threadIdx.x == 0) {
-            cg_close_iteration(it.st, rho_new);
-            if (it.st->done) finish_problem(probs[it.prob], it.prob, ctl, finished_ids);
-        }
+    double rho_new;
+    if (grid_sum(bs, it.partials, it.cap, &it.st->ticket_up, it.b, it.nb, &rho_new) && threadIdx.x == 0) {
+        cg_close_iteration(it.st, rho_new);
+        if (it.st->done) finish_problem(probs[it.prob], it.prob, ctl, finished_ids);
     }
 }
 
@@ -871,8 +874,10 @@ static int fx_launch_nq(Batch *B, bool up, bool launch) {
     const int o = NQ - 2;
     if (up) {
         if (!launch) return SEM_OK;
-        batch_owner_kernel<NQ><<<unsigned(B->own_grid[o]), 256, 0, stream()>>>(B->d_own[o], B->d_probs, B->ctl,
-                                                                              B->finished_ids);
+        count_launches(1);
+        return cuda_check(launch_pdl(batch_owner_kernel<NQ>, unsigned(B->own_grid[o]), 256, 0, B->d_own[o], B->d_probs,
+                                     B->ctl, B->finished_ids),
+                          "batch_owner_kernel");
     } else {
         const int epb = B->fx_epb[o];
         static size_t sm_set = 0;
@@ -890,10 +895,10 @@ static int fx_launch_nq(Batch *B, bool up, bool launch) {
         double xi[kMaxQ], w[kMaxQ], D[kMaxQ * kMaxQ];
         gll_rule_and_derivative(NQ - 1, xi, w, D);
         fx_coefficients(D, NQ, &A.d, &A.dt);
-        batch_fx_kernel<NQ><<<unsigned(B->fx_grid[o]), unsigned(line_threads(NQ, epb)), sm, stream()>>>(A);
+        count_launches(1);
+        return cuda_check(launch_pdl(batch_fx_kernel<NQ>, unsigned(B->fx_grid[o]), unsigned(line_threads(NQ, epb)), sm, A),
+                          "batch_fx_kernel");
     }
-    count_launches(1);
-    return cuda_check(cudaGetLastError(), "batch: fixed-point launch");
 }
 
 static int fx_launch(Batch *B, int nq, bool up, bool launch) {
@@ -1094,9 +1099,9 @@ static int build_fx_lists(Batch *B) {
             if (P->nq - 2 != o || B->gone[k]) continue;
             FxMember M{};
             M.op = FxItem{P->r, P->w, P->p, P->x, P->Gfx, P->kgfx, P->st, P->partials, 0, 0, 0,
-                          int((P->E + B->fx_epb[o] - 1) / B->fx_epb[o])};
+                          int((P->E + B->fx_epb[o] - 1) / B->fx_epb[o]), P->partials_cap};
             M.up = OwnerItem{P->r, P->w, P->st, P->partials, box_dims(P->nx, P->ny, P->nz), int(P->E), 0,
-                             owner_blocks_of(P), k};
+                             owner_blocks_of(P), k, P->partials_cap};
             if (M.op.nb > P->partials_cap || M.up.nb > P->partials_cap)
                 return set_error(SEM_ERANGE, "batch: more blocks than reduction slots");
             M.first = nf;

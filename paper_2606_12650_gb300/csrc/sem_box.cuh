@@ -142,6 +142,18 @@ __device__ __forceinline__ void vload_nc(const T *p, T (&v)[V]) {
     for (int c = 0; c < V; ++c) v[c] = a[c];
 }
 
+// From L2: values that the kernel before wrote.  With programmatic dependent
+// launch a block can be resident while that kernel still runs, so neither the
+// read-only path (__ldg) nor a pointer the compiler may read through it (const
+// __restrict__) is used for them.
+template <typename T, int V>
+__device__ __forceinline__ void vload_cg(const T *p, T (&v)[V]) {
+    const typename VecT<T, V>::type q = __ldcg(reinterpret_cast<const typename VecT<T, V>::type *>(p));
+    const T *a = reinterpret_cast<const T *>(&q);
+#pragma unroll
+    for (int c = 0; c < V; ++c) v[c] = a[c];
+}
+
 template <typename T, int V>
 __device__ __forceinline__ void vstore(T *p, const T (&v)[V]) {
     typename VecT<T, V>::type q;
@@ -350,8 +362,7 @@ struct OwnerRows {
 };
 
 template <int NQ, int CY, int CZ, bool PRE, typename Acc>
-__device__ __forceinline__ void owner_rows(double *__restrict__ r, const double *__restrict__ w,
-                                           const double *__restrict__ dinv, int j, int k, int eg, int lane, int E,
+__device__ __forceinline__ void owner_rows(double *r, const double *w, const double *__restrict__ dinv, int j, int k, int eg, int lane, int E,
                                            const BoxDims &bd, double alpha, Acc &acc, Acc &acc_rr) {
     using R = OwnerRows<NQ, double>;
     constexpr int V = R::V, N = R::N, NP = R::NP, LR = R::LR, EG = R::EG, C = CY * CZ;
@@ -382,12 +393,12 @@ __device__ __forceinline__ void owner_rows(double *__restrict__ r, const double 
     }
     auto offset = [&](int c) { return (CY > 1 && (c & 1) ? oy : 0) + (CZ > 1 && (CY > 1 ? c >> 1 : c) ? oz : 0); };
     if (live) {
-        vload<double, V>(r + l0, rv);
+        vload_cg<double, V>(r + l0, rv);
         if (PRE) vload_nc<double, V>(dinv + l0, dv);
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-            vload_nc<double, V>(w + l0 + offset(c), wv[c]);
-            if (hi && !here) xn[c] = __ldg(w + l0 + offset(c) + V - 1 + ox);
+            vload_cg<double, V>(w + l0 + offset(c), wv[c]);
+            if (hi && !here) xn[c] = __ldcg(w + l0 + offset(c) + V - 1 + ox);
         }
     }
 #pragma unroll
@@ -513,7 +524,8 @@ __global__ void assemble_box_kernel(const double *__restrict__ f, double *__rest
 template <int NQ, typename T, typename Acc>
 __global__ void __launch_bounds__(256, 5) cg_update_nodes_kernel(T *__restrict__ x, T *__restrict__ r,
                                                               const T *__restrict__ p, const T *__restrict__ w,
-                                                              int nL, BoxDims bd, double *partials, CgState *st) {
+                                                              int nL, BoxDims bd, double *partials, int64_t cap,
+                                                              CgState *st) {
     __shared__ double scratch[256];
     if (st->done) return;
     const T alpha = T(st->alpha);
@@ -529,19 +541,19 @@ __global__ void __launch_bounds__(256, 5) cg_update_nodes_kernel(T *__restrict__
         bs = double(block_sum_f32(acc, reinterpret_cast<float *>(scratch)));
     else
         bs = block_sum_wide(acc_value(acc), scratch);
-    if (publish_grouped(bs, partials, &st->ticket_up)) {
-        const double rho_new = finish_grouped(partials, &st->ticket_up);
-        if (threadIdx.x == 0) cg_close_iteration(st, rho_new);
-    }
+    double rho_new;
+    if (grid_sum(bs, partials, cap, &st->ticket_up, int(blockIdx.x), int(gridDim.x), &rho_new) && threadIdx.x == 0)
+        cg_close_iteration(st, rho_new);
 }
 
 // The FP64 step by owner rows (x += alpha p is deferred to the next operator
 // kernel, which holds p anyway).
 template <int NQ>
 __global__ void __launch_bounds__(256, kOwnerBlocks)
-    cg_update_owner_kernel(double *__restrict__ r, const double *__restrict__ w, int E, BoxDims bd, double *partials,
-                           CgState *st) {
+    cg_update_owner_kernel(double *r, const double *w, int E, BoxDims bd, double *partials,
+                           int64_t cap, CgState *st) {
     __shared__ double scratch[256];
+    pdl_wait();
     if (st->done) return;
     DwAcc acc = acc_zero<DwAcc>(), unused = acc_zero<DwAcc>();
     owner_tasks<NQ, false>(r, w, nullptr, int(blockIdx.x * blockDim.x + threadIdx.x) >> 5,
@@ -549,10 +561,9 @@ __global__ void __launch_bounds__(256, kOwnerBlocks)
     // one warp's FP64 sum per block (13 instead of 40 warp-wide FP64 adds),
     // grid sum in groups
     const double bs = block_sum_wide(acc_value(acc), scratch);
-    if (publish_grouped(bs, partials, &st->ticket_up)) {
-        const double rho_new = finish_grouped(partials, &st->ticket_up);
-        if (threadIdx.x == 0) cg_close_iteration(st, rho_new);
-    }
+    double rho_new;
+    if (grid_sum(bs, partials, cap, &st->ticket_up, int(blockIdx.x), int(gridDim.x), &rho_new) && threadIdx.x == 0)
+        cg_close_iteration(st, rho_new);
 }
 
 // Blocks of an FP32 update launch, grid-stride beyond: one resident wave (E =
@@ -573,15 +584,15 @@ template <int NQ, typename T, typename Acc>
 static int launch_update_rows_nq(const Problem *P, T *x, T *r, const T *p, const T *w, CgState *st) {
     constexpr int V = UpdVec<NQ, T>::value;
     if constexpr (sizeof(T) == 8) {
-        cg_update_owner_kernel<NQ><<<owner_grid<NQ>(P), 256, 0, stream()>>>(
-            r, w, int(P->E), box_dims(P->nx, P->ny, P->nz), P->partials, st);
         count_launches(1);
-        return cuda_check(cudaGetLastError(), "cg_update_owner_kernel");
+        return cuda_check(launch_pdl(cg_update_owner_kernel<NQ>, owner_grid<NQ>(P), 256, 0, r, w, int(P->E),
+                                     box_dims(P->nx, P->ny, P->nz), P->partials, P->partials_cap, st),
+                          "cg_update_owner_kernel");
     }
     int64_t blocks = (P->nL / V + 255) / 256;
     blocks = std::min(blocks, resident_blocks(cg_update_nodes_kernel<NQ, T, Acc>, 256));
     cg_update_nodes_kernel<NQ, T, Acc><<<unsigned(blocks), 256, 0, stream()>>>(
-        x, r, p, w, int(P->nL), box_dims(P->nx, P->ny, P->nz), P->partials, st);
+        x, r, p, w, int(P->nL), box_dims(P->nx, P->ny, P->nz), P->partials, P->partials_cap, st);
     count_launches(1);
     return cuda_check(cudaGetLastError(), "cg_update_nodes_kernel");
 }

@@ -23,9 +23,9 @@
 // FP64 operation off the update; x_finish_kernel applies the last one.
 // The dot products of the paper are tree reductions (Section VIII-B, the
 // unrolled reduction of Table "HIP-variable vs HIP-fixed"); here each block
-// reduces in a fixed order, the last block of each group of 32 blocks sums
-// the group's partials in index order and the last group sums the group sums
-// (publish_grouped), so results are reproducible run to run.  Scalars
+// reduces in a fixed order, the last block of each group of blocks sums the
+// group's partials in index order and the last group sums the group sums
+// (grid_sum), so results are reproducible run to run.  Scalars
 // never leave the device inside the loop: the host replays a CUDA graph of K
 // iterations and polls the stop flag once per replay.
 #include <cuda_runtime.h>
@@ -71,7 +71,7 @@ __device__ __forceinline__ void sum_copies(double *u, const int (&o)[M]) {
 #pragma unroll
         for (int d = 0; d < M; ++d)
             if (c >> d & 1) at[c] += o[d];
-        v[c] = u[at[c]];
+        v[c] = __ldcg(u + at[c]);
     }
     double s = v[0];
 #pragma unroll
@@ -81,9 +81,10 @@ __device__ __forceinline__ void sum_copies(double *u, const int (&o)[M]) {
 }
 
 template <int NQ, bool MASK>
-__global__ void __launch_bounds__(256) gs_box_kernel(double *__restrict__ u, int64_t E, BoxDims bd, int64_t total) {
+__global__ void __launch_bounds__(256) gs_box_kernel(double *u, int64_t E, BoxDims bd, int64_t total) {
     constexpr int N = NQ - 1, N2 = N * N, NQ2 = NQ * NQ, NP = NQ2 * NQ;
     const int64_t t64 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    pdl_wait();
     if (t64 >= total) return;
     const unsigned nE = unsigned(E);
     unsigned t = unsigned(t64), e;
@@ -160,12 +161,10 @@ static int launch_gs_nq(const Problem *P, double *u, bool mask) {
     const int64_t nx = P->nx, ny = P->ny, nz = P->nz;
     int64_t total = P->E * (3 * N * N + 3 * N + 1);
     if (mask) total += NQ * NQ * (ny * nz + nx * nz + nx * ny);
-    if (mask)
-        gs_box_kernel<NQ, true><<<grid_for(total, kThreads), kThreads, 0, stream()>>>(u, P->E, bd, total);
-    else
-        gs_box_kernel<NQ, false><<<grid_for(total, kThreads), kThreads, 0, stream()>>>(u, P->E, bd, total);
     count_launches(1);
-    return cuda_check(cudaGetLastError(), "gs_box_kernel");
+    return cuda_check(launch_pdl(mask ? gs_box_kernel<NQ, true> : gs_box_kernel<NQ, false>, grid_for(total, kThreads),
+                                 kThreads, 0, u, P->E, bd, total),
+                      "gs_box_kernel");
 }
 
 static int launch_gs_any(const Problem *P, double *u, bool mask) {

@@ -204,48 +204,75 @@ __device__ __forceinline__ double finish_partials(const double *partials, int n,
     return acc;
 }
 
-// Two-level grid sum for launches of many blocks.  Each block publishes into
-// its group of kSumGroup consecutive blocks; the group's last block to arrive
-// sums the group's partials in order (one warp, fixed shuffle tree), stores
-// the group sum, resets the group ticket and takes a ticket of the grid; the
-// last group returns true in all threads of its block, and finish_grouped
-// then sums the group sums in order.  The FP64 additions of the grid sum are
-// spread over the groups' last blocks instead of all falling on one block at
-// the end of the launch (on GB300 FP64 runs at 1/64 of the FP32 rate).
-// Block b of nb (a launch's own blocks, or the blocks of one problem of a batch).
-__device__ __forceinline__ bool publish_grouped(double v0, double *partials, uint32_t *ticket, int b, int nb) {
+// Sum of v[0..n) by one block in a fixed order (strided over as many warps as
+// give each lane four values, shuffle trees, then the warps' sums).  Result in
+// thread 0.
+__device__ __forceinline__ double block_sum_array(const double *v, int n) {
+    __shared__ double s_warp[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int nw = max(1, min(int(blockDim.x) >> 5, (n + 127) / 128));
+    double s = 0.0;
+    if (wid < nw) {
+        for (int q = threadIdx.x; q < n; q += 32 * nw) s += __ldcg(v + q);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) s_warp[wid] = s;
+    }
+    if (nw > 1) {
+        __syncthreads();
+        if (wid == 0) {
+            s = lane < nw ? s_warp[lane] : 0.0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        }
+        __syncthreads();
+    }
+    return s;
+}
+
+// Grid sum of the blocks' values v0 (thread 0) of block b of nb (a launch's
+// own blocks, or the blocks of one problem of a batch).  Returns true in all
+// threads of the block that completes it, with the sum in its thread 0.
+// partials: the problem's buffer of `cap` slots.  Up to kOneLevel blocks: the
+// last block to arrive sums all values.  More: the last block of each group
+// of kSumGroup consecutive blocks sums the group, the last group the groups'
+// sums, so that the FP64 additions (1/64 of the FP32 rate on GB300) are spread
+// over the launch.  Each level costs a store, a fence, a ticket and a load,
+// ~1.7 us at the end of a launch.
+constexpr int kOneLevel = 1024;
+__device__ __forceinline__ bool grid_sum(double v0, double *partials, int64_t cap, uint32_t *ticket, int b, int nb,
+                                         double *total) {
     __shared__ int s_last;
-    const int64_t cap = partials_capacity(partials);
-    uint32_t *gt = group_tickets(partials, cap);
-    const int g = b / kSumGroup, g0 = g * kSumGroup;
-    const int gn = min(kSumGroup, nb - g0);
+    const bool one = nb <= kOneLevel;
+    const int g = one ? 0 : b / kSumGroup, g0 = g * kSumGroup;
+    const int gn = one ? nb : min(kSumGroup, nb - g0);
+    uint32_t *gt = one ? ticket : group_tickets(partials, cap) + g;
     if (threadIdx.x == 0) {
         partials[b] = v0;
         __threadfence();
-        s_last = atomicAdd(gt + g, 1u) == uint32_t(gn - 1);
+        s_last = atomicAdd(gt, 1u) == uint32_t(gn - 1);
     }
     __syncthreads();
     if (!s_last) return false;
-    __syncthreads();  // every thread has read s_last before thread 0 rewrites it
-    if (threadIdx.x < 32) {
-        __threadfence();
-        double s = int(threadIdx.x) < gn ? __ldcg(partials + g0 + threadIdx.x) : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    __threadfence();
+    double s = block_sum_array(partials + g0, gn);
+    if (!one) {
+        const int ng = (nb + kSumGroup - 1) / kSumGroup;
+        __syncthreads();   // every thread has read s_last before thread 0 rewrites it
         if (threadIdx.x == 0) {
             partials[cap + g] = s;
-            gt[g] = 0u;
+            *gt = 0u;
             __threadfence();
-            const uint32_t ng = uint32_t(nb + kSumGroup - 1) / kSumGroup;
-            s_last = atomicAdd(ticket, 1u) == ng - 1;
+            s_last = atomicAdd(ticket, 1u) == uint32_t(ng - 1);
         }
+        __syncthreads();
+        if (!s_last) return false;
+        __threadfence();
+        s = block_sum_array(partials + cap, ng);
     }
-    __syncthreads();
-    return s_last != 0;
-}
-
-__device__ __forceinline__ bool publish_grouped(double v0, double *partials, uint32_t *ticket) {
-    return publish_grouped(v0, partials, ticket, int(blockIdx.x), int(gridDim.x));
+    if (threadIdx.x == 0) *ticket = 0u;
+    *total = s;
+    return true;
 }
 
 // Zero the group tickets (grid-stride): at the start of every solve, so that
@@ -258,25 +285,15 @@ __device__ __forceinline__ void reset_group_tickets(double *partials) {
         gt[i] = 0u;
 }
 
-// In the block for which publish_grouped returned true: the sum of the group
-// sums in a fixed order (one warp), the grid ticket reset.  Result in thread 0.
-__device__ __forceinline__ double finish_grouped(const double *partials, uint32_t *ticket, int nb) {
-    double s = 0.0;
-    if (threadIdx.x < 32) {
-        __threadfence();
-        const int ng = (nb + kSumGroup - 1) / kSumGroup;
-        const int64_t cap = partials_capacity(partials);
-        for (int q = threadIdx.x; q < ng; q += 32) s += __ldcg(partials + cap + q);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (threadIdx.x == 0) *ticket = 0u;
-    }
-    return s;
-}
-
-__device__ __forceinline__ double finish_grouped(const double *partials, uint32_t *ticket) {
-    return finish_grouped(partials, ticket, int(gridDim.x));
-}
+// Programmatic dependent launch: a kernel started by launch_pdl is set up while
+// the one before it in the stream still drains (E = 64, N = 7: a CG iteration
+// of two launches 21.5 -> 18.4 us, with the grid sums in one level).  pdl_wait
+// returns when that one has completed and its writes are visible; it comes
+// before any access to memory that an earlier kernel writes or reads.  No
+// kernel asks for an earlier start (griddepcontrol.launch_dependents): blocks
+// that only wait take slots from the last blocks that work (36.3 -> 36.6 ms
+// for 100 iterations at E = 32^3, 154.8 -> 159 ms for a batch).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Block sum of FP32 values in FP32: fixed shuffle tree per warp, then the
 // warp sums in order by warp 0.  scratch: >= 32 floats of shared memory that

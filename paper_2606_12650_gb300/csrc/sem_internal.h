@@ -15,8 +15,8 @@
 namespace sem {
 
 constexpr int kMaxQ = 10;          // N <= 9  ->  N+1 <= 10 points per direction
-// Grid sums of many blocks in two levels (publish_grouped): groups of
-// kSumGroup consecutive blocks.  A problem's partials buffer holds `cap`
+// Grid sums of many blocks in two levels (grid_sum): groups of kSumGroup
+// consecutive blocks.  A problem's partials buffer holds `cap`
 // block partials, then cap / kSumGroup group sums (doubles), then
 // cap / kSumGroup group tickets (uint32, zero between launches); cap is at
 // least kMinPartials and at least the problem's element count (the largest
@@ -207,6 +207,22 @@ int32_t *status_word();            // device status word (kernels write it)
 int32_t *status_host();            // pinned host copy (filled by poll_status / cg_solve)
 int poll_status();                 // sync, read and clear the status word -> SEM_OK/SEM_ETIMEDOUT
 void count_launches(int64_t n);
+// Launch on stream() with programmatic stream serialization: the kernel calls
+// pdl_wait (sem_device.cuh) before it touches what earlier kernels do.
+template <typename... K, typename... A>
+inline cudaError_t launch_pdl(void (*kern)(K...), unsigned grid, unsigned block, size_t smem, A... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream();
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, K(args)...);
+}
 int set_error(int code, const std::string &msg);
 int cuda_check(cudaError_t err, const char *what);
 

@@ -122,9 +122,10 @@ __global__ void pcg_init_kernel(const double *__restrict__ b, const double *__re
 // runs at 1/64 rate.
 template <int NQ>
 __global__ void __launch_bounds__(256, kOwnerBlocks)
-    pcg_update_kernel(double *__restrict__ r, const double *__restrict__ w, const double *__restrict__ dinv, int E,
+    pcg_update_kernel(double *r, const double *w, const double *__restrict__ dinv, int E,
                       BoxDims bd, double *partials, CgState *st) {
     __shared__ double red[32];
+    pdl_wait();
     if (st->done) return;
     DwAcc rz = acc_zero<DwAcc>(), rr = acc_zero<DwAcc>();
     owner_tasks<NQ, true>(r, w, dinv, int(blockIdx.x * blockDim.x + threadIdx.x) >> 5,
@@ -140,10 +141,10 @@ __global__ void __launch_bounds__(256, kOwnerBlocks)
 
 template <int NQ>
 static int launch_pcg_update_nq(const Problem *P) {
-    pcg_update_kernel<NQ><<<owner_grid<NQ>(P), 256, 0, stream()>>>(P->r, P->w, P->dinv, int(P->E),
-                                                                   box_dims(P->nx, P->ny, P->nz), P->partials, P->st);
     count_launches(1);
-    return cuda_check(cudaGetLastError(), "pcg_update_kernel");
+    return cuda_check(launch_pdl(pcg_update_kernel<NQ>, owner_grid<NQ>(P), 256, 0, P->r, P->w, P->dinv, int(P->E),
+                                 box_dims(P->nx, P->ny, P->nz), P->partials, P->st),
+                      "pcg_update_kernel");
 }
 
 static int launch_pcg_update(const Problem *P) {
