@@ -1,6 +1,6 @@
 // sem_ax32.cu -- the FP32 local Poisson operator for the inner solves of
-// mixed-precision iterative refinement (persistent, double-buffered kernel
-// of sem_ax32p.cuh): FP32 vectors and arithmetic, geometric factors stored in
+// mixed-precision iterative refinement: the choice of the kernel, and the
+// persistent, double-buffered one (sem_ax32p.cuh).  FP32 vectors and arithmetic, geometric factors stored in
 // FP32 (24 B/node) or BF16 (12 B/node) and widened exactly to FP32; the CG
 // variant's <p, A p> is reduced across threads and blocks in FP64.  Also the
 // one-time conversion of the FP64 geometric factors (round to nearest even).
@@ -129,8 +129,7 @@ int prepare_ax32(const Problem *Pb) {
 int launch_ax32(const Problem *Pb, const float *x, float *y, int gprec) {
     const TuneChoice c = tune_get(tune_kind_of_gprec(gprec), Pb->nq);
     if (c.variant == kAxLines || c.variant == kAxLinesPrefetch || c.variant == kAxLinesStaged)
-        return launch_lines32(Pb, x, y, gprec, false, c.epb,
-                              c.variant == kAxLinesPrefetch ? 1 : (c.variant == kAxLinesStaged ? 2 : 0));
+        return launch_lines32(Pb, x, y, gprec, false, c.epb, c.variant == kAxLinesStaged);
     if (gprec == kGF32) {
         AxArgs<float, float> a = ax_args<float, float>(Pb, static_cast<const float *>(Pb->G32), Pb->partials, Pb->st_in);
         a.x = x;
@@ -144,16 +143,21 @@ int launch_ax32(const Problem *Pb, const float *x, float *y, int gprec) {
     return launch_ax32p<__nv_bfloat16, false>(Pb, a);
 }
 
+int ax32_cg_launches(const Problem *Pb, int gprec) {
+    const int v = tune_get(tune_kind_of_gprec(gprec), Pb->nq).variant;
+    return v == kAxLines || v == kAxLinesPrefetch ? 2 : 1;
+}
+
 int launch_ax32_cg(const Problem *Pb, int gprec) {
     const TuneChoice c = tune_get(tune_kind_of_gprec(gprec), Pb->nq);
     if (c.variant == kAxLines || c.variant == kAxLinesPrefetch || c.variant == kAxLinesStaged)
-        return launch_lines32(Pb, nullptr, nullptr, gprec, true, c.epb,
-                              c.variant == kAxLinesPrefetch ? 1 : (c.variant == kAxLinesStaged ? 2 : 0));
+        return launch_lines32(Pb, nullptr, nullptr, gprec, true, c.epb, c.variant == kAxLinesStaged);
     if (gprec == kGF32) {
         AxArgs<float, float> a = ax_args<float, float>(Pb, static_cast<const float *>(Pb->G32), Pb->partials, Pb->st_in);
         a.x = Pb->r32;
         a.y = Pb->w32;
         a.p = Pb->p32;
+        a.xs = Pb->d32;   // d += alpha p of the previous iteration
         return launch_ax32p<float, true>(Pb, a);
     }
     AxArgs<float, __nv_bfloat16> a =
@@ -161,6 +165,7 @@ int launch_ax32_cg(const Problem *Pb, int gprec) {
     a.x = Pb->r32;
     a.y = Pb->w32;
     a.p = Pb->p32;
+    a.xs = Pb->d32;   // d += alpha p of the previous iteration
     return launch_ax32p<__nv_bfloat16, true>(Pb, a);
 }
 

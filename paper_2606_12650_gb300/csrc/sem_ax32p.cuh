@@ -12,7 +12,8 @@
 // with it (block barrier) and a proxy fence orders the threads' earlier
 // shared-memory writes before the engine's.
 //
-// CG mode: stage A holds r, stage B holds p; p = r + beta p is written back
+// CG mode: stage A holds r, stage B holds p; d += alpha p of the previous
+// iteration goes to global memory, p = r + beta p is written back
 // into B and to global memory; the r-direction products go into A (free once
 // p is formed).  Plain mode: A holds x; B takes the r-direction products.
 #pragma once
@@ -60,6 +61,9 @@ ax32p_kernel(const AxArgs<float, GT> P, int ngroups) {
     float *ws_buf = reinterpret_cast<float *>(stages + 2 * S::STAGE);
 
     if (CG && P.st->done) return;  // solve finished: the rest of the graph is a no-op
+
+    // read before this launch's last block replaces it
+    const float xalpha = CG ? float(P.st->alpha) : 0.f;
 
     const int tid = threadIdx.x;
     const int eb = tid / NQ2;
@@ -131,6 +135,7 @@ ax32p_kernel(const AxArgs<float, GT> P, int ngroups) {
                 for (int k = 0; k < NQ; ++k) {
                     const int q = eb * NP + k * NQ2 + ij;
                     const float pn = fmaf(beta, sb[q], sa[q]);
+                    P.xs[nb + k * NQ2 + ij] = fmaf(xalpha, sb[q], P.xs[nb + k * NQ2 + ij]);
                     sb[q] = pn;
                     xk[k] = pn;
                     P.p[nb + k * NQ2 + ij] = pn;

@@ -137,10 +137,9 @@ struct LinePad {
 };
 
 // Where phase 2 gets the geometric factors: loaded from global memory at use
-// (kGLoad), loaded into registers before the slab wait (kGRegs, BF16 only),
-// or copied into shared memory by the TMA engine with the slab (kGStaged,
-// FP32 arithmetic only: an element's FP64 factors would take 24 KB).
-enum LineG : int { kGLoad = 0, kGRegs = 1, kGStaged = 2 };
+// (kGLoad, FP64), or copied into shared memory by the TMA engine with the slab
+// (kGStaged, FP32: an element's FP64 factors would take 24 KB).
+enum LineG : int { kGLoad = 0, kGStaged = 1 };
 
 struct LineShape {
     // values per buffer for epb elements: the larger of the staged slab
@@ -173,19 +172,16 @@ struct LineShape {
 // first when xs is given; *part receives this thread's <p, A_local p> partial
 // (in T).  Returns false if the slab copy timed out (status set, copies
 // drained).
-// GM (LineG): kGRegs loads the element's BF16 factors into registers (3
-// words per node) before the slab wait, kGStaged has the TMA engine copy
-// them into shared memory after the three regions, with the slab; either
-// way their latency overlaps the slab copy instead of stalling phase 2.
+// GM (LineG): kGStaged has the TMA engine copy the factors into shared memory
+// after the three regions, with the slab, so that their latency overlaps the
+// slab copy instead of stalling phase 2.
 template <int NQ, typename T, typename GT, bool CG, bool PRE, int GM>
 __device__ __forceinline__ bool lines_group(const T *x, T *y, T *p, const GT *G, const EoMat<T> &cd,
                                             const EoMat<T> &ct, T beta, T xalpha, T *xs, const T *dinv, int64_t e0,
                                             int ne, int epb, T *regA, uint64_t *bar, uint32_t phase,
                                             int32_t *status, T *part) {
-    constexpr bool PF = GM == kGRegs;
     constexpr bool GS = GM == kGStaged;
-    static_assert(!PF || sizeof(GT) == 2, "G prefetch is for BF16 factors");
-    static_assert(!GS || sizeof(T) == 4, "G staging is for FP32 arithmetic");
+    static_assert(GS == (sizeof(T) == 4), "factors staged in FP32 arithmetic, loaded at use in FP64");
     constexpr int NQ2 = NQ * NQ, NP = NQ2 * NQ;
     constexpr int P1 = LinePad<NQ>::P1, P2 = LinePad<NQ>::P2, NPP = LinePad<NQ>::NPP;
     // N+1 = 8: the staged slab's rows and columns are read in a per-thread
@@ -221,10 +217,6 @@ __device__ __forceinline__ bool lines_group(const T *x, T *y, T *p, const GT *G,
         slab_issue(s1, src1, pl1, bar);
         if (CG) slab_issue(s2, src2, pl2, bar);
         if (GS) slab_issue(gdst, gsrc, plg, bar);
-        // FP32: the factors read from global memory in phase 2 start towards L2
-        // now (in FP64 a block computes so long that prefetched lines would be
-        // evicted before phase 2 reads them)
-        if (GM == kGLoad && sizeof(T) == 4) bulk_prefetch_l2(gsrc, uint32_t(ne) * NP * 6u * uint32_t(sizeof(GT)));
     }
     slab_edges(s1, src1, pl1, tid, nthreads);
     if (CG) slab_edges(s2, src2, pl2, tid, nthreads);
@@ -235,16 +227,6 @@ __device__ __forceinline__ bool lines_group(const T *x, T *y, T *p, const GT *G,
     const int a = ab % NQ, b = ab / NQ;
     const bool act = eb < ne;
     const int64_t nb = (e0 + eb) * NP;
-    unsigned gw[PF ? NQ : 1][3];
-    if (PF && act) {
-#pragma unroll
-        for (int k = 0; k < NQ; ++k) {
-            const unsigned *gq = reinterpret_cast<const unsigned *>(G + 6 * (nb + k * NQ2 + b * NQ + a));
-            gw[k][0] = __ldg(gq);
-            gw[k][1] = __ldg(gq + 1);
-            gw[k][2] = __ldg(gq + 2);
-        }
-    }
     const bool ok = mbar_wait_bounded(bar, phase, status);
     if (__syncthreads_or(!ok)) {
         mbar_wait_bounded(bar, phase, nullptr);  // let copies in flight land before leaving
@@ -321,11 +303,7 @@ __device__ __forceinline__ bool lines_group(const T *x, T *y, T *p, const GT *G,
             const int pq = k * P2 + tp;
             const T ur = SU[pq], us = SV[pq];
             T g[6];
-            if constexpr (PF) {
-                const float2 g01 = bf16x2_to_float2(gw[k][0]), g23 = bf16x2_to_float2(gw[k][1]),
-                             g45 = bf16x2_to_float2(gw[k][2]);
-                g[0] = g01.x; g[1] = g01.y; g[2] = g23.x; g[3] = g23.y; g[4] = g45.x; g[5] = g45.y;
-            } else if constexpr (GS) {
+            if constexpr (GS) {
                 load_g6_smem(reinterpret_cast<const GT *>(gdst) + 6 * (eb * NP + k * NQ2 + tq), g);
             } else {
                 load_g6(G, nb + k * NQ2 + tq, g);

@@ -12,10 +12,11 @@
 // the vector kernel switches on N on the device.  The operator body and the
 // elements per pass follow the per-order tuner's table for the batch's
 // precision: the line body (sem_ax_lines.cuh) or the column body, passes of
-// 256 / (N+1)^2 elements.  FP64 batches whose table chose the fixed-point
-// variant (sem_ax_fx.cuh) take that kernel and the owner-row update
-// (sem_box.cuh) instead, one block per item as in a stand-alone solve, from
-// lists that a kernel writes on the device ("fixed-point orders" below).  Items of problems whose
+// 256 / (N+1)^2 elements.  Orders whose table chose the fixed-point variant
+// (FP64, sem_ax_fx.cuh) or a line variant (FP32, sem_ax_f32.cuh) take that
+// kernel and the owner-row update (sem_box.cuh) instead, one block per item as
+// in a stand-alone solve, from lists that a kernel writes on the device ("block
+// orders" below).  Items of problems whose
 // solve finished are dropped from the lists between rounds (the items of one
 // problem stay together and in order, so its reductions never change).
 //
@@ -44,6 +45,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "sem_ax_f32.cuh"
 #include "sem_ax_fx.cuh"
 #include "sem_box.cuh"
 #include "sem_device.cuh"
@@ -75,6 +77,7 @@ struct BatchProb {
     int32_t refine;                 // mixed: inner solve ended, refine this round
     int32_t outer_done;             // mixed: true residual reached tol (or out of steps)
     int32_t finished;               // solve over; reported once in the finished list
+    int32_t deferred;               // mixed: the inner solve leaves its last step of d32 to be applied
     int32_t inner_total;            // mixed: inner iterations so far
     int32_t outer_steps;            // mixed: refinement steps so far
     double bb;                      // <b, b>
@@ -95,24 +98,32 @@ struct BatchQueue {
 enum BatchQ : int { kQAx = 0, kQVec = 1, kNumQ = 2 };
 
 // Operator bodies of a batch: every member of one order takes the same one.
-enum AxBody : int { kBodyColumns = 0, kBodyLines = 1, kBodyFX = 2, kBodyNone = -1 };
+enum AxBody : int { kBodyColumns = 0, kBodyLines = 1, kBodyBlocks = 2, kBodyNone = -1 };
 
-// ---- fixed-point orders (FP64 batches): one block per item, everything the
-// block needs in its item, so that it waits for one load before its own data.
-struct FxItem {                     // operator: ne elements from e0
-    const double *r;
-    double *w, *p, *x;
-    const int4 *G;
-    const int32_t *kg;
+// ---- block orders: one block per item, everything the block needs in its
+// item, so that it waits for one load before its own data.  Vectors are FP64
+// (fixed-point operator) or FP32 (inner CG).
+struct AxItem {                     // operator: ne elements from e0
+    const void *r;
+    void *w, *p, *x;                // x: the solution (FP64), the correction d (FP32)
+    const void *G;                  // int4 (fixed point), BF16 or FP32 factors
+    const int32_t *kg;              // fixed point: scale per element
     CgState *st;
     double *partials;
     int e0, ne;                     // ne = 0: beyond the list
     int b, nb;                      // block b of the problem's nb
     int64_t cap;                    // slots of `partials`
 };
+struct PapItem {                    // FP32: block b of the nb that add the problem's n parts of <p, A p>
+    CgState *st;
+    double *partials;
+    int64_t cap;
+    int n, b, nb;                   // nb = 0: beyond the list
+    int pad;
+};
 struct OwnerItem {                  // update: warps 8 b .. 8 b + 7 of the problem's 8 nb
-    double *r;
-    const double *w;
+    void *r;
+    const void *w;
     CgState *st;
     double *partials;
     BoxDims bd;
@@ -120,27 +131,30 @@ struct OwnerItem {                  // update: warps 8 b .. 8 b + 7 of the probl
     int prob;
     int64_t cap;
 };
-struct FxMember {                   // a member's ranges in its order's lists
-    FxItem op;                      // e0, ne, b unset
+struct BlockMember {                // a member's ranges in its order's lists
+    AxItem op;                      // e0, ne, b unset
+    PapItem pap;                    // b unset; nb = 0: none
     OwnerItem up;                   // b unset
-    FxItem *items;
+    AxItem *items;
+    PapItem *paps;
     OwnerItem *owners;
     int first, epb;
     int64_t E;
-    int up_first;
+    int pap_first, up_first;
 };
 
 // Blocks of a problem's owner-row update: 1 to 8 rows per warp, more for
 // larger problems (a rule of the problem only).
-template <int NQ>
+template <int NQ, typename T>
 static int owner_blocks(int64_t E) {
-    const int64_t tasks = OwnerRows<NQ, double>::tasks(E);
+    const int64_t tasks = OwnerRows<NQ, T>::tasks(E);
     const int64_t per = std::min<int64_t>(8, std::max<int64_t>(1, tasks / 2048));
     return int((tasks + 8 * per - 1) / (8 * per));
 }
+template <typename T>
 static int owner_blocks_of(const Problem *P) {
     switch (P->nq) {
-#define SEM_OB(Q) case Q: return owner_blocks<Q>(P->E);
+#define SEM_OB(Q) case Q: return owner_blocks<Q, T>(P->E);
         SEM_OB(2) SEM_OB(3) SEM_OB(4) SEM_OB(5) SEM_OB(6) SEM_OB(7) SEM_OB(8) SEM_OB(9) SEM_OB(10)
 #undef SEM_OB
         default: return 0;
@@ -149,14 +163,19 @@ static int owner_blocks_of(const Problem *P) {
 
 // One block per member: writes its items and clears its group tickets (no
 // launch of the batch is in flight).
-__global__ void batch_fx_items_kernel(const FxMember *members) {
-    const FxMember M = members[blockIdx.x];
+__global__ void batch_items_kernel(const BlockMember *members) {
+    const BlockMember M = members[blockIdx.x];
     for (int b = threadIdx.x; b < M.op.nb; b += blockDim.x) {
-        FxItem it = M.op;
+        AxItem it = M.op;
         it.b = b;
         it.e0 = b * M.epb;
         it.ne = int(min(int64_t(M.epb), M.E - it.e0));
         M.items[M.first + b] = it;
+    }
+    for (int b = threadIdx.x; b < M.pap.nb; b += blockDim.x) {
+        PapItem it = M.pap;
+        it.b = b;
+        M.paps[M.pap_first + b] = it;
     }
     for (int b = threadIdx.x; b < M.up.nb; b += blockDim.x) {
         OwnerItem it = M.up;
@@ -168,7 +187,7 @@ __global__ void batch_fx_items_kernel(const FxMember *members) {
 }
 
 struct FxBatchArgs {
-    const FxItem *items;
+    const AxItem *items;
     EoMatFX d, dt;
     int epb;
 };
@@ -176,14 +195,45 @@ struct FxBatchArgs {
 template <int NQ>
 __global__ void __maxnreg__(FxRegs<NQ>::value) batch_fx_kernel(const __grid_constant__ FxBatchArgs P) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const FxItem it = P.items[blockIdx.x];   // the lists do not change within a round
+    const AxItem it = P.items[blockIdx.x];   // the lists do not change within a round
     pdl_wait();
     if (it.ne == 0 || it.st->done) return;
-    fx_prefetch<NQ>(it.G, it.e0, it.ne);
+    const int4 *G = static_cast<const int4 *>(it.G);
+    fx_prefetch<NQ>(G, it.e0, it.ne);
     double part = 0.0;
-    lines_group_fx<NQ, true, false>(it.r, it.w, it.p, it.G, it.kg, P.d, P.dt, it.st->beta, it.st->alpha, it.x, nullptr,
-                                    it.e0, it.ne, P.epb, smem, &part);
+    lines_group_fx<NQ, true, false>(static_cast<const double *>(it.r), static_cast<double *>(it.w),
+                                    static_cast<double *>(it.p), G, it.kg, P.d, P.dt, it.st->beta, it.st->alpha,
+                                    static_cast<double *>(it.x), nullptr, it.e0, it.ne, P.epb, smem, &part);
     fx_publish<NQ>(part, smem, P.epb, it.partials, it.cap, it.st, it.b, it.nb);
+}
+
+struct F32BatchArgs {
+    const AxItem *items;
+    EoMat<float> d, dt;
+    int epb;
+};
+
+template <int NQ, typename GT>
+__global__ void __maxnreg__((F32Regs<NQ, GT>::value)) batch_f32_kernel(const __grid_constant__ F32BatchArgs P) {
+    extern __shared__ __align__(16) float smem32[];
+    const AxItem it = P.items[blockIdx.x];
+    pdl_wait();
+    if (it.ne == 0 || it.st->done) return;
+    const GT *G = static_cast<const GT *>(it.G);
+    f32_prefetch<NQ>(G, it.e0, it.ne);
+    const float part = lines_group_f32<NQ, GT, true>(static_cast<const float *>(it.r), static_cast<float *>(it.w),
+                                                     static_cast<float *>(it.p), static_cast<float *>(it.x), G, P.d,
+                                                     P.dt, float(it.st->beta), float(it.st->alpha), it.e0, it.ne, P.epb,
+                                                     smem32);
+    const float s = block_sum_f32(part, smem32);
+    if (threadIdx.x == 0) it.partials[it.b] = double(s);
+}
+
+__global__ void __launch_bounds__(kPapThreads) batch_pap_kernel(const PapItem *items) {
+    const PapItem it = items[blockIdx.x];
+    pdl_wait();
+    if (it.nb == 0 || it.st->done) return;
+    pap_sum(it.partials, it.cap, it.n, it.b, it.nb, it.st);
 }
 constexpr int kOrders = kMaxQ - 1;  // N+1 = 2 .. kMaxQ
 
@@ -201,6 +251,8 @@ struct BatchCtl {
     BatchQueue q_vec[kOrders];
 };
 
+constexpr int kGraphBufs = 7 + 3 * kOrders;
+
 struct Batch {
     int mode = 0;                   // 0 FP64 CG, 1 mixed (BF16 G), 2 mixed (FP32 G)
     int K = 16;                     // CG iterations per round
@@ -212,6 +264,7 @@ struct Batch {
     // member whose solve finished is left out of the device lists (`gone`)
     std::vector<BatchItem> ax_all, vec_all;
     std::vector<int> ax_first_all, ax_count_all, vec_first_all, vec_count_all;
+    TuneChoice ord_choice[kOrders] = {};   // per order: the table's entry when its members started
     int ord_body[kOrders];          // operator body per order (kBodyNone: no member of that order)
     int ord_count[kOrders];         // operator items per order in the device list now
     int ord_vcount[kOrders];        // vector items per order in the device list now
@@ -231,23 +284,25 @@ struct Batch {
     BatchCtl *ctl_host = nullptr;
     unsigned seen_finished = 0;
     bool any_init = false;
-    // fixed-point orders: the two lists, their capacities, the blocks of a
-    // launch, and the elements per operator block
-    FxItem *d_fx[kOrders] = {};
+    // block orders: the lists, their capacities, the blocks of a launch, and
+    // the elements per operator block
+    AxItem *d_op[kOrders] = {};
+    PapItem *d_pap[kOrders] = {};
     OwnerItem *d_own[kOrders] = {};
-    int cap_fx[kOrders] = {}, cap_own[kOrders] = {};
-    int fx_grid[kOrders] = {}, own_grid[kOrders] = {}, fx_epb[kOrders] = {};
-    FxMember *d_members = nullptr;
+    int cap_op[kOrders] = {}, cap_pap[kOrders] = {}, cap_own[kOrders] = {};
+    int blk_grid[kOrders][3] = {};   // operator, <p, A p> sums, update
+    int blk_epb[kOrders] = {};
+    BlockMember *d_members = nullptr;
     int cap_members = 0;
     cudaGraphExec_t graph = nullptr;
     cudaStream_t graph_stream = nullptr;
     // the buffers the captured round reads and its grids; the graph stays
     // valid while the buffers stay in place and the grids stay the same
     // (membership changes only rewrite the lists' contents and counts)
-    const void *graph_bufs[7 + 2 * kOrders] = {};
+    const void *graph_bufs[kGraphBufs] = {};
     int graph_items[2] = {0, 0};    // power-of-two ceilings of the item counts at capture
     int ord_ranges[4 * kOrders];    // host copy of the device per-order ranges (operator, vector)
-    int graph_fx[2 * kOrders] = {};   // the fixed-point orders' grids at capture
+    int graph_blk[kOrders][3] = {};   // the block orders' grids at capture
     int graph_ord[3 * kOrders] = {};  // per order: the captured launches' grid ceilings and body (0: none)
     int64_t graph_launches = 0;     // kernel launches in one replay
     // side streams and events that fork the per-order operator launches into
@@ -275,16 +330,8 @@ inline size_t batch_ax_smem() {
 // constant and the products read constant-bank operands directly.
 __constant__ double c_D64[kMaxQ - 1][kMaxQ * kMaxQ];
 __constant__ float c_D32[kMaxQ - 1][kMaxQ * kMaxQ];
-// even-odd coefficients of D ([0]) and D^T ([1]) for the line body
+// even-odd coefficients of D ([0]) and D^T ([1]) for the (FP64) line body
 __constant__ EoMat<double> c_E64[kMaxQ - 1][2];
-__constant__ EoMat<float> c_E32[kMaxQ - 1][2];
-
-template <typename T>
-__device__ __forceinline__ const EoMat<T> &const_eo(int nq, int which);
-template <>
-__device__ __forceinline__ const EoMat<double> &const_eo<double>(int nq, int which) { return c_E64[nq - 2][which]; }
-template <>
-__device__ __forceinline__ const EoMat<float> &const_eo<float>(int nq, int which) { return c_E32[nq - 2][which]; }
 
 template <int NQ, typename T>
 struct ConstD;
@@ -376,16 +423,15 @@ __device__ __forceinline__ bool batch_ax_item(const T *xin, T *yout, T *pv, cons
     return true;
 }
 
-template <int NQ, typename T, typename GT, bool CG>
-__device__ __forceinline__ bool batch_lines_item(const T *xin, T *yout, T *pv, const GT *G, T beta, int64_t first,
-                                              int count, int group, T *regA, uint64_t *bar, uint32_t *phase,
-                                              int32_t *status, T *pt) {
-    constexpr int GM = kGLoad;   // factors loaded at use: the register prefetch would not fit 4 CTAs per SM
-    T acc = T(0);
+template <int NQ, bool CG>
+__device__ __forceinline__ bool batch_lines_item(const double *xin, double *yout, double *pv, const double *G, double beta, int64_t first,
+                                              int count, int group, double *regA, uint64_t *bar, uint32_t *phase,
+                                              int32_t *status, double *pt) {
+    double acc = 0.0;
     for (int g = 0; g < count; g += group) {
-        T part = T(0);
-        const bool ok = lines_group<NQ, T, GT, CG, false, GM>(xin, yout, pv, G, const_eo<T>(NQ, 0),
-                                                              const_eo<T>(NQ, 1), beta, T(0), nullptr, nullptr,
+        double part = 0.0;
+        const bool ok = lines_group<NQ, double, double, CG, false, kGLoad>(xin, yout, pv, G, c_E64[NQ - 2][0],
+                                                              c_E64[NQ - 2][1], beta, 0.0, nullptr, nullptr,
                                                               first + g, min(group, count - g), group, regA, bar,
                                                               *phase, status, &part);
         *phase ^= 1u;
@@ -437,7 +483,7 @@ __global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 4 ? 4 : 2)
         T pt = T(0);
         bool ok;
         if constexpr (BODY == kBodyLines)
-            ok = batch_lines_item<NQ, T, GT, CG>(xin, yout, pv, prob_G<GT>(P), beta, item.first, item.count,
+            ok = batch_lines_item<NQ, CG>(xin, yout, pv, prob_G<GT>(P), beta, item.first, item.count,
                                                  item.group, regA, bar, &phase, status, &pt);
         else
             ok = batch_ax_item<NQ, T, GT, CG>(xin, yout, pv, prob_G<GT>(P), beta, item.first, item.count, regA, bar,
@@ -551,7 +597,7 @@ __device__ __noinline__ double vec_item_body(BatchProb &P, CgState *st, int64_t 
     } else if (MODE == kVecCorrect) {
         for (int v = tid; v < count; v += blockDim.x) {
             const int64_t l = first + v;
-            P.x[l] += double(P.d32[l]);
+            P.x[l] += double(P.deferred ? fmaf(float(P.st_in->alpha), P.p32[l], P.d32[l]) : P.d32[l]);
         }
     } else if (MODE == kVecResidual) {
         for (int v = tid; v < count; v += blockDim.x)
@@ -680,22 +726,23 @@ __global__ void __launch_bounds__(kBatchThreads, MODE == kVecUpdate32 ? kUpd32Bl
     leave_queue(q);
 }
 
-// The owner-row update of a fixed-point order.
-template <int NQ>
+// The owner-row update of a block order.
+template <int NQ, typename T>
 __global__ void __launch_bounds__(256, kOwnerBlocks)
     batch_owner_kernel(const OwnerItem *items, BatchProb *probs, BatchCtl *ctl, int32_t *finished_ids) {
+    using Acc = typename std::conditional<sizeof(T) == 8, DwAcc, float>::type;
     __shared__ double scratch[256];
     const OwnerItem it = items[blockIdx.x];
     pdl_wait();
     if (it.nb == 0 || it.st->done) return;
-    DwAcc acc = acc_zero<DwAcc>(), unused = acc_zero<DwAcc>();
-    owner_tasks<NQ, false>(it.r, it.w, nullptr, 8 * it.b + int(threadIdx.x >> 5), 8 * it.nb, it.E, it.bd, it.st->alpha,
-                           acc, unused);
-    const double bs = block_sum_wide(acc_value(acc), scratch);
+    Acc acc = acc_zero<Acc>(), unused = acc_zero<Acc>();
+    owner_tasks<NQ, false, T>(static_cast<T *>(it.r), static_cast<const T *>(it.w), nullptr,
+                              8 * it.b + int(threadIdx.x >> 5), 8 * it.nb, it.E, it.bd, T(it.st->alpha), acc, unused);
+    const double bs = owner_block_sum(acc, scratch);
     double rho_new;
     if (grid_sum(bs, it.partials, it.cap, &it.st->ticket_up, it.b, it.nb, &rho_new) && threadIdx.x == 0) {
         cg_close_iteration(it.st, rho_new);
-        if (it.st->done) finish_problem(probs[it.prob], it.prob, ctl, finished_ids);
+        if (sizeof(T) == 8 && it.st->done) finish_problem(probs[it.prob], it.prob, ctl, finished_ids);
     }
 }
 
@@ -773,8 +820,10 @@ static int bax_order(Batch *B, int body, int count, bool launch, int *res) {
             return launch ? BaxLaunch<T, GT, MODE, NQ, kBodyColumns>::launch(B, count)
                           : BaxLaunch<T, GT, MODE, NQ, kBodyColumns>::resident(res);
         case kBodyLines:
-            return launch ? BaxLaunch<T, GT, MODE, NQ, kBodyLines>::launch(B, count)
-                          : BaxLaunch<T, GT, MODE, NQ, kBodyLines>::resident(res);
+            if constexpr (sizeof(T) == 8)
+                return launch ? BaxLaunch<T, GT, MODE, NQ, kBodyLines>::launch(B, count)
+                              : BaxLaunch<T, GT, MODE, NQ, kBodyLines>::resident(res);
+            [[fallthrough]];
         default: return set_error(SEM_EARG, "batch: no such operator body for this precision");
     }
 }
@@ -824,11 +873,17 @@ static int launch_orders(Batch *B, bool parallel, F &&fn) {
     return rc;
 }
 
+// The persistent kernels' body for an order: its own, or (the refinement
+// residual of a block order) the line body.
+static int queue_body(const Batch *B, int o) {
+    return B->ord_body[o] == kBodyBlocks ? int(kBodyLines) : B->ord_body[o];
+}
+
 // The operator phase of one precision.
 template <typename T, typename GT, int MODE>
 static int launch_bax(Batch *B, bool parallel = false) {
     return launch_orders(B, parallel, [B](int o) {
-        return bax<T, GT, MODE>(B, o + 2, B->ord_body[o], B->ord_count[o], true);
+        return bax<T, GT, MODE>(B, o + 2, queue_body(B, o), B->ord_count[o], true);
     });
 }
 
@@ -868,44 +923,83 @@ static int upd(Batch *B, int nq, int count, bool launch, int *res = nullptr) {
     }
 }
 
-// One fixed-point order's operator (up = false) or update launch.
-template <int NQ>
-static int fx_launch_nq(Batch *B, bool up, bool launch) {
-    const int o = NQ - 2;
-    if (up) {
-        if (!launch) return SEM_OK;
-        count_launches(1);
-        return cuda_check(launch_pdl(batch_owner_kernel<NQ>, unsigned(B->own_grid[o]), 256, 0, B->d_own[o], B->d_probs,
-                                     B->ctl, B->finished_ids),
-                          "batch_owner_kernel");
-    } else {
-        const int epb = B->fx_epb[o];
-        static size_t sm_set = 0;
-        const size_t sm = fx_smem<NQ>(epb);
-        if (sm > sm_set) {   // before any capture (prepare_bax)
-            const int rc = cuda_check(cudaFuncSetAttribute(batch_fx_kernel<NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                           int(sm)), "batch: shared-memory attribute");
-            if (rc != SEM_OK) return rc;
-            sm_set = sm;
-        }
-        if (!launch) return SEM_OK;
-        FxBatchArgs A{};
-        A.items = B->d_fx[o];
-        A.epb = epb;
-        double xi[kMaxQ], w[kMaxQ], D[kMaxQ * kMaxQ];
-        gll_rule_and_derivative(NQ - 1, xi, w, D);
-        fx_coefficients(D, NQ, &A.d, &A.dt);
-        count_launches(1);
-        return cuda_check(launch_pdl(batch_fx_kernel<NQ>, unsigned(B->fx_grid[o]), unsigned(line_threads(NQ, epb)), sm, A),
-                          "batch_fx_kernel");
-    }
+// Shared-memory limit of a block order's operator kernel (before any capture:
+// prepare_bax).
+template <typename K>
+static int block_smem(K kern, size_t sm, size_t *set) {
+    if (sm <= *set) return SEM_OK;
+    const int rc = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm)),
+                              "batch: shared-memory attribute");
+    if (rc == SEM_OK) *set = sm;
+    return rc;
 }
 
-static int fx_launch(Batch *B, int nq, bool up, bool launch) {
+// The operator launch (or, launch false, its preparation) of a block order.
+template <int NQ>
+static int block_ax_fx(Batch *B, bool launch) {
+    const int o = NQ - 2, epb = B->blk_epb[o];
+    static size_t sm_set = 0;
+    const size_t sm = fx_smem<NQ>(epb);
+    const int rc = block_smem(batch_fx_kernel<NQ>, sm, &sm_set);
+    if (rc != SEM_OK || !launch) return rc;
+    FxBatchArgs A{};
+    A.items = B->d_op[o];
+    A.epb = epb;
+    double xi[kMaxQ], w[kMaxQ], D[kMaxQ * kMaxQ];
+    gll_rule_and_derivative(NQ - 1, xi, w, D);
+    fx_coefficients(D, NQ, &A.d, &A.dt);
+    count_launches(1);
+    return cuda_check(launch_pdl(batch_fx_kernel<NQ>, unsigned(B->blk_grid[o][0]), unsigned(line_threads(NQ, epb)), sm, A),
+                      "batch_fx_kernel");
+}
+
+template <int NQ, typename GT>
+static int block_ax_f32(Batch *B, bool launch) {
+    const int o = NQ - 2, epb = B->blk_epb[o];
+    static size_t sm_set = 0;
+    const size_t sm = f32_smem<NQ>(epb);
+    int rc = block_smem(batch_f32_kernel<NQ, GT>, sm, &sm_set);
+    if (rc != SEM_OK || !launch) return rc;
+    AxArgs<float, GT> none{};
+    double xi[kMaxQ], w[kMaxQ], D[kMaxQ * kMaxQ];
+    gll_rule_and_derivative(NQ - 1, xi, w, D);
+    const AxLineArgs<float, GT> L = line_args(none, D, NQ, epb);
+    const F32BatchArgs A{B->d_op[o], L.d, L.dt, epb};
+    count_launches(2);
+    rc = cuda_check(launch_pdl(batch_f32_kernel<NQ, GT>, unsigned(B->blk_grid[o][0]), unsigned(line_threads(NQ, epb)), sm,
+                               A), "batch_f32_kernel");
+    return rc != SEM_OK ? rc : cuda_check(launch_pdl(batch_pap_kernel, unsigned(B->blk_grid[o][1]), unsigned(kPapThreads),
+                                                     0, B->d_pap[o]), "batch_pap_kernel");
+}
+
+template <int NQ>
+static int block_ax_nq(Batch *B, bool launch) {
+    return B->mode == 0 ? block_ax_fx<NQ>(B, launch)
+                        : (B->mode == 1 ? block_ax_f32<NQ, __nv_bfloat16>(B, launch) : block_ax_f32<NQ, float>(B, launch));
+}
+
+template <int NQ>
+static int block_update_nq(Batch *B) {
+    const int o = NQ - 2;
+    auto kern = B->mode == 0 ? batch_owner_kernel<NQ, double> : batch_owner_kernel<NQ, float>;
+    count_launches(1);
+    return cuda_check(launch_pdl(kern, unsigned(B->blk_grid[o][2]), 256, 0, B->d_own[o], B->d_probs, B->ctl,
+                                 B->finished_ids), "batch_owner_kernel");
+}
+
+static int block_ax(Batch *B, int nq, bool launch) {
     switch (nq) {
-#define SEM_FX(Q) case Q: return fx_launch_nq<Q>(B, up, launch);
-        SEM_FX(2) SEM_FX(3) SEM_FX(4) SEM_FX(5) SEM_FX(6) SEM_FX(7) SEM_FX(8) SEM_FX(9) SEM_FX(10)
-#undef SEM_FX
+#define SEM_BLK(Q) case Q: return block_ax_nq<Q>(B, launch);
+        SEM_BLK(2) SEM_BLK(3) SEM_BLK(4) SEM_BLK(5) SEM_BLK(6) SEM_BLK(7) SEM_BLK(8) SEM_BLK(9) SEM_BLK(10)
+#undef SEM_BLK
+        default: return set_error(SEM_EARG, "batch: unsupported order");
+    }
+}
+static int block_update(Batch *B, int nq) {
+    switch (nq) {
+#define SEM_BLK(Q) case Q: return block_update_nq<Q>(B);
+        SEM_BLK(2) SEM_BLK(3) SEM_BLK(4) SEM_BLK(5) SEM_BLK(6) SEM_BLK(7) SEM_BLK(8) SEM_BLK(9) SEM_BLK(10)
+#undef SEM_BLK
         default: return set_error(SEM_EARG, "batch: unsupported order");
     }
 }
@@ -928,8 +1022,9 @@ static int prepare_bax(Batch *B) {
         const int body = B->ord_body[o];
         if (body == kBodyNone) continue;
         int rc;
-        if (body == kBodyFX) {
-            rc = fx_launch(B, o + 2, false, false);
+        if (body == kBodyBlocks) {
+            rc = block_ax(B, o + 2, false);
+            if (rc == SEM_OK && B->mode != 0) rc = bax<double, double, 1>(B, o + 2, queue_body(B, o), 0, false);
         } else if (B->mode == 0) {
             rc = bax<double, double, 0>(B, o + 2, body, 0, false, &B->ord_res[o]);
             if (rc == SEM_OK) rc = upd<kVecUpdate64>(B, o + 2, 0, false, &B->ord_vres[o]);
@@ -988,7 +1083,6 @@ static int batch_attrs(Batch *B) {
             for (int q = 0; q < (N + 1) * (N + 1); ++q) h32[N - 1][q] = float(h64[N - 1][q]);
         }
         static EoMat<double> e64[kMaxQ - 1][2];
-        static EoMat<float> e32[kMaxQ - 1][2];
         for (int N = 1; N <= kMaxQ - 1; ++N) {
             const int nq = N + 1;
             double Dt[kMaxQ * kMaxQ];
@@ -996,13 +1090,10 @@ static int batch_attrs(Batch *B) {
                 for (int l = 0; l < nq; ++l) Dt[i * nq + l] = h64[N - 1][l * nq + i];
             e64[N - 1][0] = eo_coefficients<double>(h64[N - 1], nq);
             e64[N - 1][1] = eo_coefficients<double>(Dt, nq);
-            e32[N - 1][0] = eo_coefficients<float>(h64[N - 1], nq);
-            e32[N - 1][1] = eo_coefficients<float>(Dt, nq);
         }
         int rc = cuda_check(cudaMemcpyToSymbol(c_D64, h64, sizeof h64), "batch: D table");
         if (rc == SEM_OK) rc = cuda_check(cudaMemcpyToSymbol(c_D32, h32, sizeof h32), "batch: D table");
         if (rc == SEM_OK) rc = cuda_check(cudaMemcpyToSymbol(c_E64, e64, sizeof e64), "batch: even-odd table");
-        if (rc == SEM_OK) rc = cuda_check(cudaMemcpyToSymbol(c_E32, e32, sizeof e32), "batch: even-odd table");
         if (rc != SEM_OK) return rc;
         done = true;
     }
@@ -1060,10 +1151,10 @@ static void order_signature(const Batch *B, int *out) {
     for (int o = 0; o < kOrders; ++o) {
         const bool on = B->ord_body[o] != kBodyNone;
         out[2 * kOrders + o] = 0;
-        if (B->ord_body[o] == kBodyFX) {
-            out[o] = kBodyFX + 1;   // the grids: keep_or_drop_graph
+        if (B->ord_body[o] == kBodyBlocks) {
+            out[o] = kBodyBlocks + 1;   // the grids: keep_or_drop_graph
             out[kOrders + o] = 0;
-            out[2 * kOrders + o] = B->fx_epb[o];
+            out[2 * kOrders + o] = B->blk_epb[o];
             continue;
         }
         out[o] = on ? 4 * items_grid(B->ord_res[o], B->ord_count[o]) + B->ord_body[o] + 1 : 0;
@@ -1075,89 +1166,106 @@ static void graph_buffers(const Batch *B, const void **out) {
     const void *bufs[7] = {B->d_probs, B->d_ax, B->d_vec, B->part, B->part_vec, B->tickets, B->finished_ids};
     std::copy(bufs, bufs + 7, out);
     for (int o = 0; o < kOrders; ++o) {
-        out[7 + o] = B->d_fx[o];
-        out[7 + kOrders + o] = B->d_own[o];
+        out[7 + 3 * o] = B->d_op[o];
+        out[8 + 3 * o] = B->d_pap[o];
+        out[9 + 3 * o] = B->d_own[o];
     }
 }
 
 template <typename X>
 static int grow(X **buf, int *cap, int need);
 
-// The lists of the fixed-point orders, members in order, finished ones left
-// out, written on the device.  A member's items and their reduction tree
-// depend on the member only.
-static int build_fx_lists(Batch *B) {
+// The lists of the block orders, members in order, finished ones left out,
+// written on the device.  A member's items and their reduction tree depend on
+// the member only.
+static int build_block_lists(Batch *B) {
     const int n = int(B->probs.size());
-    std::vector<FxMember> ms;
+    std::vector<BlockMember> ms;
     int rc = SEM_OK;
     for (int o = 0; o < kOrders && rc == SEM_OK; ++o) {
-        if (B->ord_body[o] != kBodyFX) continue;
+        if (B->ord_body[o] != kBodyBlocks) continue;
         const size_t m0 = ms.size();
-        int nf = 0, nu = 0;
+        int nf = 0, np = 0, nu = 0;
         for (int k = 0; k < n; ++k) {
             const Problem *P = B->probs[k];
             if (P->nq - 2 != o || B->gone[k]) continue;
-            FxMember M{};
-            M.op = FxItem{P->r, P->w, P->p, P->x, P->Gfx, P->kgfx, P->st, P->partials, 0, 0, 0,
-                          int((P->E + B->fx_epb[o] - 1) / B->fx_epb[o]), P->partials_cap};
-            M.up = OwnerItem{P->r, P->w, P->st, P->partials, box_dims(P->nx, P->ny, P->nz), int(P->E), 0,
-                             owner_blocks_of(P), k, P->partials_cap};
+            const int blocks = int((P->E + B->blk_epb[o] - 1) / B->blk_epb[o]);
+            const BoxDims bd = box_dims(P->nx, P->ny, P->nz);
+            BlockMember M{};
+            if (B->mode == 0) {
+                M.op = AxItem{P->r, P->w, P->p, P->x, P->Gfx, P->kgfx, P->st, P->partials, 0, 0, 0, blocks, P->partials_cap};
+                M.up = OwnerItem{P->r, P->w, P->st, P->partials, bd, int(P->E), 0, owner_blocks_of<double>(P), k,
+                                 P->partials_cap};
+            } else {
+                M.op = AxItem{P->r32, P->w32, P->p32, P->d32, B->mode == 1 ? P->G16 : P->G32, nullptr, P->st_in,
+                              P->partials, 0, 0, 0, blocks, P->partials_cap};
+                M.pap = PapItem{P->st_in, P->partials, P->partials_cap, blocks, 0, pap_blocks(blocks), 0};
+                M.up = OwnerItem{P->r32, P->w32, P->st_in, P->partials, bd, int(P->E), 0, owner_blocks_of<float>(P), k,
+                                 P->partials_cap};
+            }
             if (M.op.nb > P->partials_cap || M.up.nb > P->partials_cap)
                 return set_error(SEM_ERANGE, "batch: more blocks than reduction slots");
             M.first = nf;
+            M.pap_first = np;
             M.up_first = nu;
-            M.epb = B->fx_epb[o];
+            M.epb = B->blk_epb[o];
             M.E = P->E;
             nf += M.op.nb;
+            np += M.pap.nb;
             nu += M.up.nb;
             ms.push_back(M);
         }
-        B->fx_grid[o] = std::max(nf, 1);
-        B->own_grid[o] = std::max(nu, 1);
-        rc = grow(&B->d_fx[o], &B->cap_fx[o], B->fx_grid[o]);
-        if (rc == SEM_OK) rc = grow(&B->d_own[o], &B->cap_own[o], B->own_grid[o]);
+        B->blk_grid[o][0] = std::max(nf, 1);
+        B->blk_grid[o][1] = std::max(np, 1);
+        B->blk_grid[o][2] = std::max(nu, 1);
+        rc = grow(&B->d_op[o], &B->cap_op[o], B->blk_grid[o][0]);
+        if (rc == SEM_OK) rc = grow(&B->d_pap[o], &B->cap_pap[o], B->blk_grid[o][1]);
+        if (rc == SEM_OK) rc = grow(&B->d_own[o], &B->cap_own[o], B->blk_grid[o][2]);
         for (size_t m = m0; m < ms.size(); ++m) {
-            ms[m].items = B->d_fx[o];
+            ms[m].items = B->d_op[o];
+            ms[m].paps = B->d_pap[o];
             ms[m].owners = B->d_own[o];
         }
         // a captured round may have more blocks than there are items now: theirs are empty
         if (rc == SEM_OK)
-            rc = cuda_check(cudaMemsetAsync(B->d_fx[o], 0, sizeof(FxItem) * size_t(B->cap_fx[o]), stream()), "batch");
+            rc = cuda_check(cudaMemsetAsync(B->d_op[o], 0, sizeof(AxItem) * size_t(B->cap_op[o]), stream()), "batch");
+        if (rc == SEM_OK)
+            rc = cuda_check(cudaMemsetAsync(B->d_pap[o], 0, sizeof(PapItem) * size_t(B->cap_pap[o]), stream()), "batch");
         if (rc == SEM_OK)
             rc = cuda_check(cudaMemsetAsync(B->d_own[o], 0, sizeof(OwnerItem) * size_t(B->cap_own[o]), stream()), "batch");
     }
     if (rc != SEM_OK || ms.empty()) return rc;
     rc = grow(&B->d_members, &B->cap_members, int(ms.size()));
     if (rc == SEM_OK)
-        rc = cuda_check(cudaMemcpyAsync(B->d_members, ms.data(), sizeof(FxMember) * ms.size(), cudaMemcpyHostToDevice,
+        rc = cuda_check(cudaMemcpyAsync(B->d_members, ms.data(), sizeof(BlockMember) * ms.size(), cudaMemcpyHostToDevice,
                                         stream()), "batch: members");
     if (rc != SEM_OK) return rc;
-    batch_fx_items_kernel<<<unsigned(ms.size()), 256, 0, stream()>>>(B->d_members);
+    batch_items_kernel<<<unsigned(ms.size()), 256, 0, stream()>>>(B->d_members);
     count_launches(1);
-    rc = cuda_check(cudaGetLastError(), "batch_fx_items_kernel");
+    rc = cuda_check(cudaGetLastError(), "batch_items_kernel");
     // the members come from pageable memory
     return rc != SEM_OK ? rc : cuda_check(cudaStreamSynchronize(stream()), "batch: sync");
 }
 
 // Drops the captured round unless its buffers stayed in place and its
-// launches' grids still fit: equal ones, or, for the fixed-point orders, a
+// launches' grids still fit: equal ones, or, for the block orders, a
 // grid of at least the current blocks and at most twice as many (or 64 more:
 // the blocks beyond the lists find an empty item).
 static void keep_or_drop_graph(Batch *B) {
-    const void *bufs[7 + 2 * kOrders];
+    const void *bufs[kGraphBufs];
     graph_buffers(B, bufs);
     int ord_now[3 * kOrders];
     order_signature(B, ord_now);
     bool fits = true;
     for (int o = 0; o < kOrders; ++o) {
-        if (B->ord_body[o] != kBodyFX) continue;
-        for (int u = 0; u < 2; ++u) {
-            const int now = u ? B->own_grid[o] : B->fx_grid[o], had = B->graph_fx[2 * o + u];
+        if (B->ord_body[o] != kBodyBlocks) continue;
+        for (int u = 0; u < 3; ++u) {
+            const int now = B->blk_grid[o][u], had = B->graph_blk[o][u];
             if (now > had || had > std::max(2 * now, now + 64)) fits = false;
         }
     }
     if (B->graph && !(fits && std::equal(ord_now, ord_now + 3 * kOrders, B->graph_ord) &&
-                      std::equal(bufs, bufs + 7 + 2 * kOrders, B->graph_bufs))) {
+                      std::equal(bufs, bufs + kGraphBufs, B->graph_bufs))) {
         cudaGraphExecDestroy(B->graph);
         B->graph = nullptr;
     }
@@ -1227,7 +1335,7 @@ static int compact(Batch *B) {
     if (rc == SEM_OK) {
         B->n_ax = counts[0];
         B->n_vec = counts[1];
-        rc = build_fx_lists(B);
+        rc = build_block_lists(B);
     }
     if (rc == SEM_OK) keep_or_drop_graph(B);
     return rc;
@@ -1274,8 +1382,15 @@ int batch_set(Batch *B, Problem **probs, const double *const *b, const uint8_t *
     std::vector<BatchItem> by_ord_v[kOrders]; // vector items likewise
     int ord_body[kOrders];
     std::fill(ord_body, ord_body + kOrders, int(kBodyNone));
-    int fx_epb[kOrders] = {};
+    int blk_epb[kOrders] = {};
     bool any_init = false;
+    // An order with members in mid-solve keeps its operator choice: a block
+    // order leaves the last step of x (or d) to its next operator launch, so
+    // its body does not change under them.
+    bool keep[kOrders] = {};
+    for (int k = 0; k < n; ++k)
+        for (size_t j = 0; j < B->probs.size(); ++j)
+            if (B->probs[j] == probs[k] && !start[k] && !old[j].finished) keep[probs[k]->nq - 2] = true;
     for (int k = 0; k < n && rc == SEM_OK; ++k) {
         Problem *P = probs[k];
         if (B->mode != 0) rc = mixed_prepare(P, B->mode == 1 ? kGBF16 : kGF32);
@@ -1304,27 +1419,26 @@ int batch_set(Batch *B, Problem **probs, const double *const *b, const uint8_t *
         // size stand-alone blocks, whose count per SM varies with it); an
         // item holds several passes (item_nodes)
         const int full = kBatchThreads / (P->nq * P->nq);
-        const TuneChoice c = tune_get(B->mode == 0 ? kTuneF64 : (B->mode == 1 ? kTuneF32G16 : kTuneF32G32), P->nq);
-        // the fixed-point variant: its line body in FP64 batches (factors
-        // made here, before any capture); mixed batches (whose FP64 operator
-        // runs only for the refinement residual) keep the FP64 line body
-        const bool fx = B->mode == 0 && c.variant == kAxLinesFX;
-        if (fx) {
-            rc = fx_prepare(P);
-            if (rc != SEM_OK) break;
-            if (fx_epb[P->nq - 2] && fx_epb[P->nq - 2] != c.epb) {
-                rc = set_error(SEM_EARG, "batch: members of one order with different operator bodies");
-                break;
-            }
-            fx_epb[P->nq - 2] = c.epb;
-        }
+        TuneChoice &c = B->ord_choice[P->nq - 2];
+        if (!keep[P->nq - 2])
+            c = tune_get(B->mode == 0 ? kTuneF64 : (B->mode == 1 ? kTuneF32G16 : kTuneF32G32), P->nq);
+        // block orders: the fixed-point variant in FP64 batches (factors made
+        // here, before any capture), the line variants in mixed ones (whose
+        // FP64 operator, for the refinement residual, runs the line body)
         const bool lines = c.variant == kAxLines || c.variant == kAxLinesPrefetch || c.variant == kAxLinesStaged ||
                            c.variant == kAxLinesFX;
+        const bool blocks = B->mode == 0 ? c.variant == kAxLinesFX : lines;
+        if (blocks) {
+            if (B->mode == 0) rc = fx_prepare(P);
+            if (rc != SEM_OK) break;
+            blk_epb[P->nq - 2] = c.epb;
+        }
+        q.deferred = B->mode != 0 && blocks;
         const int group = full;
         const int np = P->nq * P->nq * P->nq;
         const int per_item = group * std::max(1, item_nodes(P->nL) / (np * group));
         const int o = P->nq - 2;
-        const int body = fx ? kBodyFX : (lines ? kBodyLines : kBodyColumns);
+        const int body = blocks ? kBodyBlocks : (lines ? kBodyLines : kBodyColumns);
         if (ord_body[o] != kBodyNone && ord_body[o] != body) {
             rc = set_error(SEM_EARG, "batch: members of one order with different operator bodies");
             break;
@@ -1356,7 +1470,7 @@ int batch_set(Batch *B, Problem **probs, const double *const *b, const uint8_t *
         hp[k].vec_first += ord_first[kOrders + probs[k]->nq - 2];
     }
     std::copy(ord_body, ord_body + kOrders, B->ord_body);
-    std::copy(fx_epb, fx_epb + kOrders, B->fx_epb);
+    std::copy(blk_epb, blk_epb + kOrders, B->blk_epb);
     for (int o = 0; o < kOrders; ++o) {
         B->ord_count[o] = int(by_ord[o].size());
         B->ord_vcount[o] = int(by_ord_v[o].size());
@@ -1416,7 +1530,7 @@ int batch_set(Batch *B, Problem **probs, const double *const *b, const uint8_t *
     if (rc == SEM_OK) rc = upload_order_ranges(B, ord_first);
     if (rc == SEM_OK) rc = cuda_check(cudaStreamSynchronize(stream()), "batch: sync");
     B->seen_finished = 0;
-    if (rc == SEM_OK) rc = build_fx_lists(B);
+    if (rc == SEM_OK) rc = build_block_lists(B);
     // the captured round reads the lists and counts from device memory: it
     // is captured again only if a buffer moved (grew) or a grid changed
     if (rc == SEM_OK) keep_or_drop_graph(B);
@@ -1435,7 +1549,8 @@ void batch_destroy(Batch *B) {
     for (void *q : ptrs)
         if (q) dev_free(q);
     for (int o = 0; o < kOrders; ++o) {
-        if (B->d_fx[o]) dev_free(B->d_fx[o]);
+        if (B->d_op[o]) dev_free(B->d_op[o]);
+        if (B->d_pap[o]) dev_free(B->d_pap[o]);
         if (B->d_own[o]) dev_free(B->d_own[o]);
     }
     if (B->d_members) dev_free(B->d_members);
@@ -1461,8 +1576,9 @@ static int capture(Batch *B) {
     cudaGraph_t g = nullptr;
     int rc = cuda_check(cudaStreamBeginCapture(stream(), cudaStreamCaptureModeThreadLocal), "batch: capture");
     if (rc != SEM_OK) return rc;
-    int orders = 0;
-    for (int o = 0; o < kOrders; ++o) orders += B->ord_body[o] != kBodyNone;
+    int per_iter = 0;
+    for (int o = 0; o < kOrders; ++o)
+        if (B->ord_body[o] != kBodyNone) per_iter += B->mode != 0 && B->ord_body[o] == kBodyBlocks ? 3 : 2;
     // each order's problems are independent of the others': its K
     // iterations form one chain of (operator, update) launches, the orders'
     // chains parallel branches of the round
@@ -1470,9 +1586,9 @@ static int capture(Batch *B) {
         const int nq = o + 2, body = B->ord_body[o], na = B->ord_count[o], nv = B->ord_vcount[o];
         int r = SEM_OK;
         for (int k = 0; k < B->K && r == SEM_OK; ++k) {
-            if (body == kBodyFX) {
-                r = fx_launch(B, nq, false, true);
-                if (r == SEM_OK) r = fx_launch(B, nq, true, true);
+            if (body == kBodyBlocks) {
+                r = block_ax(B, nq, true);
+                if (r == SEM_OK) r = block_update(B, nq);
             } else if (B->mode == 0) {
                 r = bax<double, double, 0>(B, nq, body, na, true);
                 if (r == SEM_OK) r = upd<kVecUpdate64>(B, nq, nv, true);
@@ -1484,7 +1600,7 @@ static int capture(Batch *B) {
         }
         return r;
     });
-    B->graph_launches = int64_t(B->K) * 2 * orders;
+    B->graph_launches = int64_t(B->K) * per_iter;
     count_launches(-B->graph_launches);
     const int rc_end = cuda_check(cudaStreamEndCapture(stream(), &g), "batch: end capture");
     if (rc == SEM_OK) rc = rc_end;
@@ -1496,10 +1612,7 @@ static int capture(Batch *B) {
         B->graph_items[0] = items_grid(1 << 30, B->n_ax);
         B->graph_items[1] = items_grid(1 << 30, B->n_vec);
         order_signature(B, B->graph_ord);
-        for (int o = 0; o < kOrders; ++o) {
-            B->graph_fx[2 * o] = B->fx_grid[o];
-            B->graph_fx[2 * o + 1] = B->own_grid[o];
-        }
+        std::copy(&B->blk_grid[0][0], &B->blk_grid[0][0] + 3 * kOrders, &B->graph_blk[0][0]);
     }
     return rc;
 }
@@ -1619,11 +1732,11 @@ int batch_results_of(Batch *B, const std::vector<int> &which, int64_t *iters, do
     return SEM_OK;
 }
 
-// A finished member's solution: the fixed-point orders defer x += alpha p to
-// the next operator launch, so the last one is applied here.
+// A finished member's solution: FP64 block orders defer x += alpha p to the
+// next operator launch, so the last one is applied here.
 int batch_emit_x(const Batch *B, int k, double *out) {
     const Problem *P = B->probs[k];
-    if (B->ord_body[P->nq - 2] == kBodyFX) return launch_x_finish(P, out);
+    if (B->mode == 0 && B->ord_body[P->nq - 2] == kBodyBlocks) return launch_x_finish(P, out);
     return cuda_check(cudaMemcpyAsync(out, P->x, sizeof(double) * P->nL, cudaMemcpyDeviceToDevice, stream()),
                       "batch: copy x");
 }

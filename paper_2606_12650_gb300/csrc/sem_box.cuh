@@ -99,9 +99,6 @@ __device__ __forceinline__ void acc_weighted_square(double &a, double d, double 
 __device__ __forceinline__ void acc_weighted_square(DwAcc &a, double d, double r) {
     a.v = dw_add_weighted_square(a.v, d, r);
 }
-__device__ __forceinline__ void acc_merge(double &a, double b) { a += b; }
-__device__ __forceinline__ void acc_merge(float &a, float b) { a += b; }
-__device__ __forceinline__ void acc_merge(DwAcc &a, const DwAcc &b) { a.v = dw_add(a.v, b.v); }
 __device__ __forceinline__ double acc_value(double a) { return a; }
 __device__ __forceinline__ double acc_value(float a) { return double(a); }
 __device__ __forceinline__ double acc_value(const DwAcc &a) { return dw_to_double(a.v); }
@@ -171,16 +168,13 @@ __device__ __forceinline__ void vstore(T *p, const T (&v)[V]) {
 // element) before the own value and that of node N (upper element) after it,
 // lists the copies in ascending local index -- the order of the sorted-
 // segment gather-scatter, so every copy of a node gets the same bits.  The
-// nodes then update themselves: r -= alpha (QQ^T w), and x += alpha p unless
-// DX (the x update is deferred to the next operator kernel, which holds p in
-// shared memory anyway).  Masked nodes are left as they are (zero).  <r, r>
-// (PRE: <r, M^-1 r> and <r, r> into *acc_rr) is accumulated into acc at each
-// node's first copy.
-template <int NQ, int V, typename T, typename Acc, bool PRE = false, bool DX = false>
+// nodes then update themselves: r -= alpha (QQ^T w), x += alpha p.  Masked nodes
+// are left as they are (zero).  <r, r> is accumulated into acc at each node's
+// first copy.
+template <int NQ, int V, typename T, typename Acc>
 __device__ __forceinline__ void update_vec(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ p,
                                           const T *__restrict__ w, int l0, const BoxDims &bd, T alpha,
-                                          Acc &acc, const T *__restrict__ dinv = nullptr,
-                                          Acc *acc_rr = nullptr) {
+                                          Acc &acc) {
     constexpr int N = NQ - 1, NQ2 = NQ * NQ, NP = NQ2 * NQ;
     const int nx = bd.nx, ny = bd.ny, nz = bd.nz;
     const unsigned e = unsigned(l0) / unsigned(NP);
@@ -202,13 +196,10 @@ __device__ __forceinline__ void update_vec(T *__restrict__ x, T *__restrict__ r,
     const bool mask_hi = i0 + V - 1 == N && ex == nx - 1;
     // the node's own values first: their loads then overlap those of w and
     // its neighbour copies below instead of waiting for the sum
-    T xv[V], pv[V], rv[V], dv[V];
-    if (!DX) {
-        vload<T, V>(x + l0, xv);
-        vload<T, V>(p + l0, pv);
-    }
+    T xv[V], pv[V], rv[V];
+    vload<T, V>(x + l0, xv);
+    vload<T, V>(p + l0, pv);
     vload<T, V>(r + l0, rv);
-    if (PRE) vload<T, V>(dinv + l0, dv);
     T sv[V];
     if (sy == 0 && sz == 0) {
         // Row inside the element in s and t: copies only across the r faces.
@@ -313,30 +304,20 @@ __device__ __forceinline__ void update_vec(T *__restrict__ x, T *__restrict__ r,
         }
     }
     const bool owner_row = sy >= 0 && sz >= 0;
-    Acc rr = acc_zero<Acc>();
 #pragma unroll
     for (int v = 0; v < V; ++v) {
         const bool masked = (v == 0 && mask_lo) || (v == V - 1 && mask_hi);
         if (!masked) {
-            if (!DX) xv[v] = fma(alpha, pv[v], xv[v]);
+            xv[v] = fma(alpha, pv[v], xv[v]);
             rv[v] = fma(-alpha, sv[v], rv[v]);
-            if (owner_row && !((v == 0) && has_lo)) {
-                if constexpr (PRE) {
-                    // <r, M^-1 r> for beta and <r, r> for the stop test
-                    acc_weighted_square(acc, dv[v], rv[v]);
-                    acc_square(rr, rv[v]);
-                } else {
-                    acc_square(acc, rv[v]);
-                }
-            }
+            if (owner_row && !((v == 0) && has_lo)) acc_square(acc, rv[v]);
         }
     }
-    if (!DX) vstore<T, V>(x + l0, xv);
+    vstore<T, V>(x + l0, xv);
     vstore<T, V>(r + l0, rv);
-    if constexpr (PRE) acc_merge(*acc_rr, rr);
 }
 
-// FP64 update by owner rows.  Only the first copy of a global node (i, j, k >=
+// The update by owner rows.  Only the first copy of a global node (i, j, k >=
 // 1 in its element) is summed and updated: r -= alpha (QQ^T w), and the result
 // is written to the node's other copies (the values are equal there, so they
 // are not read).  A warp takes the same row (j, k) of EG consecutive elements,
@@ -351,7 +332,10 @@ __device__ __forceinline__ void update_vec(T *__restrict__ x, T *__restrict__ r,
 // and lane, costs 6 FP64 operations per local node instead of 1.4.  E = 32^3,
 // N = 7: 133 us for every copy updating itself with the classes' additions in
 // one chain, 164 us for owner rows in one body, 78 us like this (HBM time of
-// the 22 B per node: 55 us); N = 8 187 -> 102 us, N = 9 102 -> 74 us.
+// the 22 B per node: 55 us); N = 8 187 -> 102 us, N = 9 102 -> 74 us.  In FP32,
+// where the memory traffic counts (11 B per node instead of the 24 of a step
+// that reads every copy and carries d along): N = 7 75 -> 39 us, N = 6 124 ->
+// 60 us, N = 9 74 -> 40 us, at 1.7e7 nodes.
 template <int NQ, typename T>
 struct OwnerRows {
     static constexpr int V = UpdVec<NQ, T>::value;
@@ -361,10 +345,10 @@ struct OwnerRows {
     static __host__ __device__ int64_t tasks(int64_t E) { return (E + EG - 1) / EG * (N * N); }
 };
 
-template <int NQ, int CY, int CZ, bool PRE, typename Acc>
-__device__ __forceinline__ void owner_rows(double *r, const double *w, const double *__restrict__ dinv, int j, int k, int eg, int lane, int E,
-                                           const BoxDims &bd, double alpha, Acc &acc, Acc &acc_rr) {
-    using R = OwnerRows<NQ, double>;
+template <int NQ, int CY, int CZ, bool PRE, typename T, typename Acc>
+__device__ __forceinline__ void owner_rows(T *r, const T *w, const T *__restrict__ dinv, int j, int k, int eg, int lane,
+                                           int E, const BoxDims &bd, T alpha, Acc &acc, Acc &acc_rr) {
+    using R = OwnerRows<NQ, T>;
     constexpr int V = R::V, N = R::N, NP = R::NP, LR = R::LR, EG = R::EG, C = CY * CZ;
     const int g = lane / LR, v = lane - g * LR;
     const int e = eg * EG + g;
@@ -382,22 +366,22 @@ __device__ __forceinline__ void owner_rows(double *r, const double *w, const dou
     const bool first = v == 0, last = v == LR - 1;
     const bool hi = last && ex < bd.nx - 1;        // node N has a copy in element e + 1,
     const bool here = g + 1 < EG && e + 1 < E;     // held by the next lane
-    double s[V], rv[V], dv[V], wv[C][V], xn[C];
+    T s[V], rv[V], dv[V], wv[C][V], xn[C];
 #pragma unroll
-    for (int q = 0; q < V; ++q) rv[q] = dv[q] = 0.0;
+    for (int q = 0; q < V; ++q) rv[q] = dv[q] = T(0);
 #pragma unroll
     for (int c = 0; c < C; ++c) {
-        xn[c] = 0.0;
+        xn[c] = T(0);
 #pragma unroll
-        for (int q = 0; q < V; ++q) wv[c][q] = 0.0;
+        for (int q = 0; q < V; ++q) wv[c][q] = T(0);
     }
     auto offset = [&](int c) { return (CY > 1 && (c & 1) ? oy : 0) + (CZ > 1 && (CY > 1 ? c >> 1 : c) ? oz : 0); };
     if (live) {
-        vload_cg<double, V>(r + l0, rv);
-        if (PRE) vload_nc<double, V>(dinv + l0, dv);
+        vload_cg<T, V>(r + l0, rv);
+        if (PRE) vload_nc<T, V>(dinv + l0, dv);
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-            vload_cg<double, V>(w + l0 + offset(c), wv[c]);
+            vload_cg<T, V>(w + l0 + offset(c), wv[c]);
             if (hi && !here) xn[c] = __ldcg(w + l0 + offset(c) + V - 1 + ox);
         }
     }
@@ -407,12 +391,12 @@ __device__ __forceinline__ void owner_rows(double *r, const double *w, const dou
 #pragma unroll
         for (int c = 1; c < C; ++c) s[q] += wv[c][q];
     }
-    double up = xn[0];
+    T up = xn[0];
     if (C > 1 && hi && !here) {
 #pragma unroll
         for (int c = 1; c < C; ++c) up += xn[c];
     }
-    const double next = __shfl_down_sync(0xffffffffu, s[0], 1);
+    const T next = __shfl_down_sync(0xffffffffu, s[0], 1);
     if (hi && here) up = next;
     if (last) s[V - 1] += up;
     // masked nodes (r faces of the cube) are left as they are
@@ -420,7 +404,7 @@ __device__ __forceinline__ void owner_rows(double *r, const double *w, const dou
 #pragma unroll
     for (int q = 0; q < V; ++q) {
         const bool masked = (q == 0 && mask_lo) || (q == V - 1 && mask_hi);
-        rv[q] = fma(masked ? 0.0 : -alpha, s[q], rv[q]);
+        rv[q] = fma(masked ? T(0) : -alpha, s[q], rv[q]);
         if (live && !masked && !(q == 0 && first)) {
             if constexpr (PRE) {
                 acc_weighted_square(acc, dv[q], rv[q]);
@@ -432,18 +416,18 @@ __device__ __forceinline__ void owner_rows(double *r, const double *w, const dou
     }
     // node 0 has its first copy in element e - 1: the previous lane, or (first
     // element of the warp) the previous warp, whose last lane writes it
-    const double prev = __shfl_up_sync(0xffffffffu, rv[V - 1], 1);
+    const T prev = __shfl_up_sync(0xffffffffu, rv[V - 1], 1);
     const bool skip = first && ex > 0 && g == 0;
     if (first && ex > 0) rv[0] = prev;
     if (live) {
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-            double *q = r + l0 + offset(c);
+            T *q = r + l0 + offset(c);
             if (skip) {
 #pragma unroll
                 for (int z = 1; z < V; ++z) q[z] = rv[z];
             } else {
-                vstore<double, V>(q, rv);
+                vstore<T, V>(q, rv);
             }
             if (hi && !here) q[V - 1 + ox] = rv[V - 1];
         }
@@ -451,9 +435,9 @@ __device__ __forceinline__ void owner_rows(double *r, const double *w, const dou
 }
 
 // One task: row (j, k) of element group eg, tasks numbered row fastest.
-template <int NQ, bool PRE, typename Acc>
-__device__ __forceinline__ void owner_task(double *r, const double *w, const double *dinv, int task, int lane, int E,
-                                           const BoxDims &bd, double alpha, Acc &acc, Acc &acc_rr) {
+template <int NQ, bool PRE, typename T, typename Acc>
+__device__ __forceinline__ void owner_task(T *r, const T *w, const T *dinv, int task, int lane, int E,
+                                           const BoxDims &bd, T alpha, Acc &acc, Acc &acc_rr) {
     constexpr int N = NQ - 1;
     const int eg = task / (N * N), row = task - eg * (N * N);
     const int k = 1 + row / N, j = 1 + row - (k - 1) * N;
@@ -470,21 +454,30 @@ __device__ __forceinline__ void owner_task(double *r, const double *w, const dou
 // The tasks of warp `wid` of `nw`: a contiguous run, so that every warp gets
 // rows of every class (with a stride of nw, a multiple of N^2 gives a warp
 // the same row each time: 133 -> 106 us at N = 7 for the former kernel).
-template <int NQ, bool PRE, typename Acc>
-__device__ __forceinline__ void owner_tasks(double *r, const double *w, const double *dinv, int wid, int nw, int E,
-                                            const BoxDims &bd, double alpha, Acc &acc, Acc &acc_rr) {
-    const int ntask = int(OwnerRows<NQ, double>::tasks(E));
+template <int NQ, bool PRE, typename T, typename Acc>
+__device__ __forceinline__ void owner_tasks(T *r, const T *w, const T *dinv, int wid, int nw, int E,
+                                            const BoxDims &bd, T alpha, Acc &acc, Acc &acc_rr) {
+    const int ntask = int(OwnerRows<NQ, T>::tasks(E));
     const int per = (ntask + nw - 1) / nw;
     const int end = min(ntask, (wid + 1) * per);
     for (int task = wid * per; task < end; ++task)
         owner_task<NQ, PRE>(r, w, dinv, task, int(threadIdx.x & 31), E, bd, alpha, acc, acc_rr);
 }
 
+// The block's sum of an owner-row accumulator (thread 0): FP32 values in FP32,
+// else one warp's FP64 sum (13 instead of 40 warp-wide FP64 additions).
+__device__ __forceinline__ double owner_block_sum(float acc, double *scratch) {
+    return double(block_sum_f32(acc, reinterpret_cast<float *>(scratch)));
+}
+__device__ __forceinline__ double owner_block_sum(const DwAcc &acc, double *scratch) {
+    return block_sum_wide(acc_value(acc), scratch);
+}
+
 // Blocks of 256 threads (6 resident per SM) of an owner-row launch.
 constexpr int kOwnerBlocks = 6;
-template <int NQ>
+template <int NQ, typename T = double>
 static unsigned owner_grid(const Problem *P) {
-    const int64_t blocks = (OwnerRows<NQ, double>::tasks(P->E) * 32 + 255) / 256;
+    const int64_t blocks = (OwnerRows<NQ, T>::tasks(P->E) * 32 + 255) / 256;
     return unsigned(std::min<int64_t>(blocks, int64_t(sm_count()) * kOwnerBlocks));
 }
 
@@ -515,100 +508,47 @@ __global__ void assemble_box_kernel(const double *__restrict__ f, double *__rest
     b[l] = s;
 }
 
-// One CG update step over all local nodes (grid-stride), with the <r, r>
-// reduction: per-thread partials and block sums in Acc, the grid sum in FP64
-// over groups of blocks, and the block that completes it closes the
-// iteration (beta, counter, stop flag).  Bounded to 48
-// registers so that 5 blocks of 256 threads stay resident per SM: the FP32
-// step is latency-bound (E = 32^3, N = 7: inner iteration -3 %).
-template <int NQ, typename T, typename Acc>
-__global__ void __launch_bounds__(256, 5) cg_update_nodes_kernel(T *__restrict__ x, T *__restrict__ r,
-                                                              const T *__restrict__ p, const T *__restrict__ w,
-                                                              int nL, BoxDims bd, double *partials, int64_t cap,
-                                                              CgState *st) {
-    __shared__ double scratch[256];
-    if (st->done) return;
-    const T alpha = T(st->alpha);
-    Acc acc = acc_zero<Acc>();
-    constexpr int V = UpdVec<NQ, T>::value;
-    const int nv = nL / V;   // nL is a multiple of (N+1), hence of V
-    for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < nv; u += gridDim.x * blockDim.x)
-        update_vec<NQ, V, T, Acc>(x, r, p, w, u * V, bd, alpha, acc);
-    // all blocks of the resident wave reach this point together: block sums
-    // in Acc when it is FP32, one warp's FP64 sum otherwise, grid sum in groups
-    double bs;
-    if constexpr (std::is_same<Acc, float>::value)
-        bs = double(block_sum_f32(acc, reinterpret_cast<float *>(scratch)));
-    else
-        bs = block_sum_wide(acc_value(acc), scratch);
-    double rho_new;
-    if (grid_sum(bs, partials, cap, &st->ticket_up, int(blockIdx.x), int(gridDim.x), &rho_new) && threadIdx.x == 0)
-        cg_close_iteration(st, rho_new);
-}
-
-// The FP64 step by owner rows (x += alpha p is deferred to the next operator
-// kernel, which holds p anyway).
-template <int NQ>
+// One CG update step, with the <r, r> reduction: per-thread partials and block
+// sums in FP32 for FP32 vectors (double-word and FP64 for FP64), the grid sum in
+// FP64, and the block that completes it closes the iteration (beta, counter,
+// stop flag).  The step of the solution (x or d += alpha p) is deferred to the
+// next operator kernel, which holds p anyway.
+template <int NQ, typename T>
 __global__ void __launch_bounds__(256, kOwnerBlocks)
-    cg_update_owner_kernel(double *r, const double *w, int E, BoxDims bd, double *partials,
-                           int64_t cap, CgState *st) {
+    cg_update_owner_kernel(T *r, const T *w, int E, BoxDims bd, double *partials, int64_t cap, CgState *st) {
+    using Acc = typename std::conditional<sizeof(T) == 8, DwAcc, float>::type;
     __shared__ double scratch[256];
     pdl_wait();
     if (st->done) return;
-    DwAcc acc = acc_zero<DwAcc>(), unused = acc_zero<DwAcc>();
-    owner_tasks<NQ, false>(r, w, nullptr, int(blockIdx.x * blockDim.x + threadIdx.x) >> 5,
-                           int(gridDim.x * blockDim.x) >> 5, E, bd, st->alpha, acc, unused);
-    // one warp's FP64 sum per block (13 instead of 40 warp-wide FP64 adds),
-    // grid sum in groups
-    const double bs = block_sum_wide(acc_value(acc), scratch);
+    Acc acc = acc_zero<Acc>(), unused = acc_zero<Acc>();
+    owner_tasks<NQ, false, T>(r, w, nullptr, int(blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                              int(gridDim.x * blockDim.x) >> 5, E, bd, T(st->alpha), acc, unused);
+    const double bs = owner_block_sum(acc, scratch);
     double rho_new;
     if (grid_sum(bs, partials, cap, &st->ticket_up, int(blockIdx.x), int(gridDim.x), &rho_new) && threadIdx.x == 0)
         cg_close_iteration(st, rho_new);
 }
 
-// Blocks of an FP32 update launch, grid-stride beyond: one resident wave (E =
-// 32^3, N = 7: inner CG iteration 216 -> 190 us).
-template <typename K>
-static int64_t resident_blocks(K kern, int threads) {
-    static int per_sm = 0;
-    if (!per_sm) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, 0) != cudaSuccess || per_sm < 1) {
-            cudaGetLastError();
-            per_sm = 4;
-        }
-    }
-    return int64_t(per_sm) * sm_count();
-}
-
-template <int NQ, typename T, typename Acc>
-static int launch_update_rows_nq(const Problem *P, T *x, T *r, const T *p, const T *w, CgState *st) {
-    constexpr int V = UpdVec<NQ, T>::value;
-    if constexpr (sizeof(T) == 8) {
-        count_launches(1);
-        return cuda_check(launch_pdl(cg_update_owner_kernel<NQ>, owner_grid<NQ>(P), 256, 0, r, w, int(P->E),
-                                     box_dims(P->nx, P->ny, P->nz), P->partials, P->partials_cap, st),
-                          "cg_update_owner_kernel");
-    }
-    int64_t blocks = (P->nL / V + 255) / 256;
-    blocks = std::min(blocks, resident_blocks(cg_update_nodes_kernel<NQ, T, Acc>, 256));
-    cg_update_nodes_kernel<NQ, T, Acc><<<unsigned(blocks), 256, 0, stream()>>>(
-        x, r, p, w, int(P->nL), box_dims(P->nx, P->ny, P->nz), P->partials, P->partials_cap, st);
+template <int NQ, typename T>
+static int launch_update_rows_nq(const Problem *P, T *r, const T *w, CgState *st) {
     count_launches(1);
-    return cuda_check(cudaGetLastError(), "cg_update_nodes_kernel");
+    return cuda_check(launch_pdl(cg_update_owner_kernel<NQ, T>, owner_grid<NQ, T>(P), 256, 0, r, w, int(P->E),
+                                 box_dims(P->nx, P->ny, P->nz), P->partials, P->partials_cap, st),
+                      "cg_update_owner_kernel");
 }
 
-template <typename T, typename Acc>
-static int launch_update_rows(const Problem *P, T *x, T *r, const T *p, const T *w, CgState *st) {
+template <typename T>
+static int launch_update_rows(const Problem *P, T *r, const T *w, CgState *st) {
     switch (P->nq) {
-        case 2: return launch_update_rows_nq<2, T, Acc>(P, x, r, p, w, st);
-        case 3: return launch_update_rows_nq<3, T, Acc>(P, x, r, p, w, st);
-        case 4: return launch_update_rows_nq<4, T, Acc>(P, x, r, p, w, st);
-        case 5: return launch_update_rows_nq<5, T, Acc>(P, x, r, p, w, st);
-        case 6: return launch_update_rows_nq<6, T, Acc>(P, x, r, p, w, st);
-        case 7: return launch_update_rows_nq<7, T, Acc>(P, x, r, p, w, st);
-        case 8: return launch_update_rows_nq<8, T, Acc>(P, x, r, p, w, st);
-        case 9: return launch_update_rows_nq<9, T, Acc>(P, x, r, p, w, st);
-        case 10: return launch_update_rows_nq<10, T, Acc>(P, x, r, p, w, st);
+        case 2: return launch_update_rows_nq<2, T>(P, r, w, st);
+        case 3: return launch_update_rows_nq<3, T>(P, r, w, st);
+        case 4: return launch_update_rows_nq<4, T>(P, r, w, st);
+        case 5: return launch_update_rows_nq<5, T>(P, r, w, st);
+        case 6: return launch_update_rows_nq<6, T>(P, r, w, st);
+        case 7: return launch_update_rows_nq<7, T>(P, r, w, st);
+        case 8: return launch_update_rows_nq<8, T>(P, r, w, st);
+        case 9: return launch_update_rows_nq<9, T>(P, r, w, st);
+        case 10: return launch_update_rows_nq<10, T>(P, r, w, st);
         default: return set_error(SEM_EARG, "cg: unsupported order");
     }
 }

@@ -134,10 +134,11 @@ enum GPrecision : int { kGF32 = 0, kGBF16 = 1 };
 // (one thread per (i, j) column, fixed elements per block), the line kernel
 // of sem_ax_lines.cuh (whole lines per thread, even-odd split, elements per
 // block chosen at launch), and the persistent TMA-pipelined column kernel of
-// sem_ax32p.cuh (FP32 only), and the line kernel with the geometric factors
-// loaded into registers before the slab wait (FP32 with BF16 factors only) or
-// staged in shared memory with the slab (FP32), and the line kernel of the
-// FP64 operator in 64-bit fixed-point arithmetic (sem_ax_fx.cuh, FP64 only).
+// sem_ax32p.cuh (FP32 only), and the line kernel of the FP64 operator in
+// 64-bit fixed-point arithmetic (sem_ax_fx.cuh, FP64 only).  In FP32, kAxLines
+// is the direct-load kernel of sem_ax_f32.cuh; kAxLinesPrefetch (BF16 factors
+// only) names the same kernel in saved tables, and kAxLinesStaged is the line
+// kernel with slab and factors in shared memory.
 enum AxVariant : int {
     kAxColumns = 0,
     kAxLines = 1,
@@ -174,8 +175,8 @@ int launch_lines_fx(const Problem *P, const double *x, double *y, int mode, int 
 int fx_prepare(Problem *P);                   // allocate + fill P->Gfx, P->kgfx (once)
 void fx_release(Problem *P);
 int prepare_f64_variant(Problem *P);          // whatever the tuned FP64 variant needs (before a capture)
-// gm: where phase 2 reads the factors (0 global, 1 registers, 2 staged in shared memory)
-int launch_lines32(const Problem *P, const float *x, float *y, int gprec, bool cg, int epb, int gm);
+// FP32: the direct-load kernel, or (staged) slab and factors in shared memory
+int launch_lines32(const Problem *P, const float *x, float *y, int gprec, bool cg, int epb, bool staged);
 bool lines_epb_ok(int nq, int epb, size_t elem_bytes, int g_stage_bytes = 0);
 void problem_drop_graphs(Problem *P);                     // sem_setup.cu
 
@@ -245,7 +246,8 @@ int launch_ax_cg(const Problem *P);          // p = r + beta p; w = A_local p; <
 int prepare_ax32(const Problem *P);
 int convert_geometry(const Problem *P, int gprec, void *out);
 int launch_ax32(const Problem *P, const float *x, float *y, int gprec);
-int launch_ax32_cg(const Problem *P, int gprec);   // inner CG on r32/p32/w32 with st_in
+int launch_ax32_cg(const Problem *P, int gprec);   // inner CG on r32/p32/d32/w32 with st_in
+int ax32_cg_launches(const Problem *P, int gprec); // kernels of one launch_ax32_cg
 int mixed_prepare(Problem *P, int gprec);          // allocate + convert on first use
 int mixed_solve(Problem *P, const double *b, double *x, double tol, int max_outer, double inner_tol,
                 int inner_maxit, int gprec, int64_t *inner_iters, int64_t *outer_iters, double *rel_res,

@@ -60,14 +60,16 @@ __global__ void mixed_inner_init_kernel(const double *__restrict__ r64, const do
     }
 }
 
-// x64 += double(d32)
-__global__ void mixed_correct_kernel(double *__restrict__ x, const float *__restrict__ d, int64_t n) {
+// x64 += double(d32 + alpha p32): the inner solve's last step of d is still to
+// be applied (each one is left to the next operator kernel)
+__global__ void mixed_correct_kernel(double *__restrict__ x, const float *__restrict__ d, const float *__restrict__ p,
+                                     const CgState *__restrict__ st, int64_t n) {
     const int64_t l = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (l < n) x[l] += double(d[l]);
+    if (l < n) x[l] += double(fmaf(float(st->alpha), p[l], d[l]));
 }
 
 static int launch_update32(const Problem *P) {
-    return launch_update_rows<float, float>(P, P->d32, P->r32, P->p32, P->w32, P->st_in);
+    return launch_update_rows<float>(P, P->r32, P->w32, P->st_in);
 }
 
 int mixed_prepare(Problem *P, int gprec) {
@@ -127,7 +129,7 @@ static int capture_inner(Problem *P, int gprec) {
         rc = launch_ax32_cg(P, gprec);
         if (rc == SEM_OK) rc = launch_update32(P);
     }
-    count_launches(-2 * int64_t(K));
+    count_launches(-ax32_cg_launches(P, gprec) * int64_t(K) - int64_t(K));
     const int rc_end = cuda_check(cudaStreamEndCapture(stream(), &g), "mixed: end capture");
     if (rc == SEM_OK) rc = rc_end;
     if (rc == SEM_OK) rc = cuda_check(cudaGraphInstantiate(&P->graph32[gprec], g, 0), "mixed: instantiate");
@@ -187,13 +189,14 @@ int mixed_solve(Problem *P, const double *b, double *x, double tol, int max_oute
         for (int64_t rep = 0; rep < max_replays; ++rep) {
             rc = cuda_check(cudaGraphLaunch(P->graph32[gprec], stream()), "mixed: graph launch");
             if (rc != SEM_OK) return rc;
-            count_launches(2 * int64_t(P->graph32_iters));
+            count_launches((ax32_cg_launches(P, gprec) + 1) * int64_t(P->graph32_iters));
             rc = read_state(P->st_in_host, P->st_in);
             if (rc != SEM_OK) return rc;
             if (P->st_in_host->done) break;
         }
         inner_total += P->st_in_host->iter;
-        mixed_correct_kernel<<<unsigned((P->nL + 255) / 256), 256, 0, stream()>>>(P->x, P->d32, P->nL);
+        mixed_correct_kernel<<<unsigned((P->nL + 255) / 256), 256, 0, stream()>>>(P->x, P->d32, P->p32, P->st_in,
+                                                                                       P->nL);
         count_launches(1);
         rc = cuda_check(cudaGetLastError(), "mixed_correct_kernel");
         // true residual in FP64: r = b - mask(QQ^T(A_local x))
