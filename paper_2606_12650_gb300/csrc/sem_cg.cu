@@ -27,7 +27,8 @@
 // group's partials in index order and the last group sums the group sums
 // (grid_sum), so results are reproducible run to run.  Scalars
 // never leave the device inside the loop: the host replays a CUDA graph of K
-// iterations and polls the stop flag once per replay.
+// iterations and polls the stop flag once per replay.  Problems of up to three
+// elements per SM run in one kernel instead (sem_cg_small.cu).
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -345,14 +346,21 @@ int cg_solve(Problem *P, const double *b, double *x, double tol, int maxit, doub
         P->graph = nullptr;
     }
     rc = prepare_f64_variant(P);
-    if (rc == SEM_OK) rc = capture_graph(P);
+    const bool small = rc == SEM_OK && small_fits(P, false);
+    if (rc == SEM_OK && !small) rc = capture_graph(P);
     if (rc != SEM_OK) return rc;
-    // at most ceil(maxit / K) replays; the flag stops earlier replays short
-    const int64_t max_replays = (int64_t(maxit) + P->graph_iters - 1) / P->graph_iters;
+    // at most ceil(maxit / K) replays; the flag stops earlier replays short (a
+    // small problem's launches hold many more iterations than K)
+    const int64_t K = small ? 1 : P->graph_iters;
+    const int64_t max_replays = (int64_t(maxit) + K - 1) / K;
     for (int64_t rep = 0; rep < max_replays; ++rep) {
-        rc = cuda_check(cudaGraphLaunch(P->graph, stream()), "cg: graph launch");
+        if (small) {
+            rc = launch_small(P, false);
+        } else {
+            rc = cuda_check(cudaGraphLaunch(P->graph, stream()), "cg: graph launch");
+            if (rc == SEM_OK) count_launches(2 * K);
+        }
         if (rc != SEM_OK) return rc;
-        count_launches(2 * int64_t(P->graph_iters));
         rc = cuda_check(cudaMemcpyAsync(P->st_host, P->st, sizeof(CgState), cudaMemcpyDeviceToHost, stream()),
                         "cg: state read");
         if (rc == SEM_OK)
@@ -365,7 +373,9 @@ int cg_solve(Problem *P, const double *b, double *x, double tol, int maxit, doub
         if (*status_host() != 0) break;
         if (P->st_host->done) break;
     }
-    rc = launch_x_finish(P, x);
+    rc = small ? cuda_check(cudaMemcpyAsync(x, P->x, sizeof(double) * P->nL, cudaMemcpyDeviceToDevice, stream()),
+                            "cg: copy x")
+               : launch_x_finish(P, x);
     if (rc == SEM_OK)
         rc = cuda_check(cudaMemcpyAsync(P->st_host, P->st, sizeof(CgState), cudaMemcpyDeviceToHost, stream()),
                         "cg: state read");

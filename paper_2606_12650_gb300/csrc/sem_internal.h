@@ -263,6 +263,9 @@ int launch_cg_update(const Problem *P);
 int launch_x_finish(const Problem *P, double *out);   // out = x + alpha p of the last iteration (deferred update)
 int cg_solve(Problem *P, const double *b, double *x, double tol, int maxit, double *hist,
              int64_t *iters, double *rel_res);
+// whole solves of small problems in one kernel (sem_cg_small.cu)
+bool small_fits(const Problem *P, bool pre);
+int launch_small(const Problem *P, bool pre);
 int launch_ax_pcg(const Problem *P);         // p = dinv r + beta p; w = A_local p; <p,w>
 int jacobi_prepare(Problem *P);              // dinv = 1 / (mask(QQ^T diag(A_local)))
 int pcg_solve(Problem *P, const double *b, double *x, double tol, int maxit, double *hist,

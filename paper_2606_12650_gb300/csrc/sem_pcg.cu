@@ -199,14 +199,19 @@ int pcg_solve(Problem *P, const double *b, double *x, double tol, int maxit, dou
     count_launches(1);
     rc = cuda_check(cudaGetLastError(), "pcg_init_kernel");
     if (rc == SEM_OK) rc = prepare_f64_variant(P);
-    if (rc == SEM_OK) rc = capture_pcg(P);
+    const bool small = rc == SEM_OK && small_fits(P, true);
+    if (rc == SEM_OK && !small) rc = capture_pcg(P);
     if (rc != SEM_OK) return rc;
-    const int K = P->nL < (1 << 20) ? 64 : 16;
+    const int64_t K = small ? 1 : P->graph_iters;
     const int64_t max_replays = (int64_t(maxit) + K - 1) / K;
     for (int64_t rep = 0; rep < max_replays; ++rep) {
-        rc = cuda_check(cudaGraphLaunch(P->graph_pcg, stream()), "pcg: graph launch");
+        if (small) {
+            rc = launch_small(P, true);
+        } else {
+            rc = cuda_check(cudaGraphLaunch(P->graph_pcg, stream()), "pcg: graph launch");
+            if (rc == SEM_OK) count_launches(2 * K);
+        }
         if (rc != SEM_OK) return rc;
-        count_launches(2 * int64_t(K));
         rc = cuda_check(cudaMemcpyAsync(P->st_host, P->st, sizeof(CgState), cudaMemcpyDeviceToHost, stream()),
                         "pcg: state read");
         if (rc == SEM_OK)
@@ -216,7 +221,10 @@ int pcg_solve(Problem *P, const double *b, double *x, double tol, int maxit, dou
         if (rc != SEM_OK) return rc;
         if (*status_host() != 0 || P->st_host->done) break;
     }
-    rc = launch_x_finish(P, x);   // the last iteration's deferred x += alpha p
+    // the last iteration's deferred x += alpha p
+    rc = small ? cuda_check(cudaMemcpyAsync(x, P->x, sizeof(double) * P->nL, cudaMemcpyDeviceToDevice, stream()),
+                            "pcg: copy x")
+               : launch_x_finish(P, x);
     if (rc == SEM_OK)
         rc = cuda_check(cudaMemcpyAsync(P->st_host, P->st, sizeof(CgState), cudaMemcpyDeviceToHost, stream()),
                         "pcg: state read");
