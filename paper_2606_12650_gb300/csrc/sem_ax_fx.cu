@@ -65,14 +65,18 @@ int fx_prepare(Problem *P) {
     }
     P->Gfx = g;
     P->kgfx = kg;
+    P->fxc = new FxConsts();
+    fx_coefficients(P->oc.D, P->nq, &P->fxc->d, &P->fxc->dt);
     return SEM_OK;
 }
 
 void fx_release(Problem *P) {
     if (P->Gfx) dev_free(P->Gfx);
     if (P->kgfx) dev_free(P->kgfx);
+    delete P->fxc;
     P->Gfx = nullptr;
     P->kgfx = nullptr;
+    P->fxc = nullptr;
 }
 
 // Elements per block: the tuned number, or fewer for problems that would not
@@ -125,7 +129,8 @@ int launch_lines_fx(const Problem *P, const double *x, double *y, int mode, int 
     L.a = ax_args<double, double>(P, P->G, P->partials, P->st);
     L.G = P->Gfx;
     L.kg = P->kgfx;
-    fx_coefficients(P->oc.D, P->nq, &L.d, &L.dt);
+    L.d = P->fxc->d;
+    L.dt = P->fxc->dt;
     L.epb = fx_epb(P, epb);
     if (mode == 0) {
         L.a.x = x;

@@ -542,6 +542,12 @@ inline EoMatFX eo_coefficients_fx(const double *M, int nq, double ubound, double
     return c;
 }
 
+// A problem's matrices, made once beside its factors (~2 us on the host, of a
+// launch's 8).
+struct FxConsts {
+    EoMatFX d, dt;
+};
+
 // Host: both matrices of an order.  |X| < 2^kFxBits, |W| <= 3 2^kFxGBits |D X|.
 inline void fx_coefficients(const double *D, int nq, EoMatFX *d, EoMatFX *dt) {
     double Dt[kMaxQ * kMaxQ], b1, b2;

@@ -543,7 +543,8 @@ int launch_small(const Problem *P, bool pre) {
     A.dinv = P->dinv;
     A.G = P->Gfx;
     A.kg = P->kgfx;
-    fx_coefficients(P->oc.D, P->nq, &A.d, &A.dt);
+    A.d = P->fxc->d;
+    A.dt = P->fxc->dt;
     A.nx = P->nx;
     A.ny = P->ny;
     A.nz = P->nz;

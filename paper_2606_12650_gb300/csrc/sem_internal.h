@@ -118,6 +118,7 @@ struct Problem {
     // their scale per element (sem_ax_fx.cuh)
     int4 *Gfx = nullptr;
     int32_t *kgfx = nullptr;
+    struct FxConsts *fxc = nullptr;   // host: its matrices (sem_ax_fx.cuh)
     float *d32 = nullptr, *r32 = nullptr, *p32 = nullptr, *w32 = nullptr;
     CgState *st_in = nullptr;
     CgState *st_in_host = nullptr;
