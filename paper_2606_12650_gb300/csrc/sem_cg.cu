@@ -27,7 +27,7 @@
 // group's partials in index order and the last group sums the group sums
 // (grid_sum), so results are reproducible run to run.  Scalars
 // never leave the device inside the loop: the host replays a CUDA graph of K
-// iterations and polls the stop flag once per replay.  Problems of up to three
+// iterations and polls the stop flag once per replay.  Problems of up to five
 // elements per SM run in one kernel instead (sem_cg_small.cu).
 #include <cuda_runtime.h>
 

@@ -521,15 +521,18 @@ int small_call(const Problem *P, const SmallArgs *A, int *capacity) {
 }  // namespace
 
 // Problems this path takes: the fixed-point operator is the order's choice,
-// every element has a resident block, and there are at most three per SM.
-// Above, the exchanges grow and the two launches fill the GPU: N = 7, E = 512
-// 21.3 here and 21.2 us as a graph, N = 3, E = 1000 17.2 and 17.2, N = 2, E =
-// 1728 22 and 18, N = 1, E = 4096 53 and 16.
+// every element has a resident block (152 SMs: 608 at N = 7, 456 at N = 8, 304
+// at N = 9), and there are at most five per SM.  At the limit of residence this
+// kernel is still the faster one (E = 600: N = 7 22.3 us an iteration against
+// 23.1, N = 6 19.6 against 25.4, N = 4 14.9 against 19.6; E = 441, N = 8 22.2
+// against 29.0); where small elements would allow more, the exchanges grow past
+// it (E = 800, N = 3 15.7 against 16.1; E = 1728, N = 2 22 against 18; E = 4096,
+// N = 1 53 against 16).
 bool small_fits(const Problem *P, bool pre) {
     if (tune_get(kTuneF64, P->nq).variant != kAxLinesFX) return false;
     int capacity = 0;
     const int rc = pre ? small_call<true>(P, nullptr, &capacity) : small_call<false>(P, nullptr, &capacity);
-    return rc == SEM_OK && P->E <= std::min<int64_t>(capacity, 3 * int64_t(sm_count()));
+    return rc == SEM_OK && P->E <= std::min<int64_t>(capacity, 5 * int64_t(sm_count()));
 }
 
 // One launch: up to kSmallIters iterations from P's state, x complete at its

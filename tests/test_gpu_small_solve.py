@@ -1,8 +1,8 @@
-"""Whole CG and PCG solves in one kernel (problems of up to three elements per
+"""Whole CG and PCG solves in one kernel (problems of up to five elements per
 SM) against the general path, which every other operator variant takes.
 
 Block counts around the exchange's limits (32 blocks and their neighbours, whole
-and partial groups) and the rule's own limit (456 elements on 152 SMs), boxes
+and partial groups) and the rule's own limit (760 elements on 152 SMs), boxes
 one element thick, every order.  Both paths run the same recurrences, so their
 histories differ by rounding alone: the first entries, before rounding grows
 with the iterations, agree to 1e-9 relative (each iteration's operator and sums
@@ -40,7 +40,8 @@ def _both(semlib, M, b, N, solve, tol, maxit):
 @pytest.mark.parametrize("pre", [False, True], ids=["cg", "pcg"])
 @pytest.mark.parametrize("dims,N", [((1, 1, 5), 2), ((7, 1, 2), 3), ((4, 4, 2), 7), ((11, 3, 1), 5), ((4, 4, 4), 9),
                                     ((13, 5, 1), 8), ((3, 11, 3), 6), ((4, 8, 4), 4), ((19, 6, 4), 3),
-                                    ((19, 6, 4), 1), ((5, 4, 3), 1)])
+                                    ((19, 6, 4), 1), ((5, 4, 3), 1), ((19, 8, 5), 3),
+                                    ((19, 2, 8), 9), ((19, 2, 16), 7), ((20, 19, 2), 2)])
 def test_matches_the_general_path(semlib, oracle_mod, dims, N, pre):
     from paper_2606_12650_gb300 import Mesh
     verts = box_vertices(*dims, 0.05, seed=N)
