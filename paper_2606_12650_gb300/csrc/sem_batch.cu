@@ -218,13 +218,13 @@ __global__ void __maxnreg__((F32Regs<NQ, GT>::value)) batch_f32_kernel(const __g
     extern __shared__ __align__(16) float smem32[];
     const AxItem it = P.items[blockIdx.x];
     pdl_wait();
-    if (it.ne == 0 || it.st->done) return;
+    if (it.ne == 0) return;
     const GT *G = static_cast<const GT *>(it.G);
-    f32_prefetch<NQ>(G, it.e0, it.ne);
-    const float part = lines_group_f32<NQ, GT, true>(static_cast<const float *>(it.r), static_cast<float *>(it.w),
-                                                     static_cast<float *>(it.p), static_cast<float *>(it.x), G, P.d,
-                                                     P.dt, float(it.st->beta), float(it.st->alpha), it.e0, it.ne, P.epb,
-                                                     smem32);
+    float part = 0.f;
+    if (!lines_group_f32_state<NQ, GT>(static_cast<const float *>(it.r), static_cast<float *>(it.w),
+                                       static_cast<float *>(it.p), static_cast<float *>(it.x), G, P.d, P.dt, it.st,
+                                       it.e0, it.ne, P.epb, smem32, &part))
+        return;
     const float s = block_sum_f32(part, smem32);
     if (threadIdx.x == 0) it.partials[it.b] = double(s);
 }
