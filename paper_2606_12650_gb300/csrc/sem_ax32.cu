@@ -143,6 +143,17 @@ int launch_ax32(const Problem *Pb, const float *x, float *y, int gprec) {
     return launch_ax32p<__nv_bfloat16, false>(Pb, a);
 }
 
+// Which stand-alone inner solves leave d += alpha p to the next operator launch
+// and update r by owner rows (an inner iteration at 1.7e7 nodes, deferred /
+// not, FP32 and BF16 factors: N = 7 176 / 191 and 149 / 166 us, N = 6 226 / 262
+// and 208 / 246, N = 4 228 / 259 and 206 / 239, N = 9 208 / 209 and 183 / 189).
+// Not at N = 3 (232 / 197, 215 / 182) and N = 5 (218 / 209, 195 / 190): their
+// rows of 16 and 24 bytes fill half of the sectors that a warp of owner rows
+// touches, where the node-wise update reads whole runs.  Nor at N = 2 with FP32
+// factors, whose persistent operator with the node-wise update takes 292 us
+// against 321.  At 2e5 nodes deferring is 0.5 to 1.7 us faster for every order.
+bool f32_defers(int nq, int gprec) { return nq != 4 && nq != 6 && !(nq == 3 && gprec == kGF32); }
+
 int ax32_cg_launches(const Problem *Pb, int gprec) {
     const int v = tune_get(tune_kind_of_gprec(gprec), Pb->nq).variant;
     return v == kAxLines || v == kAxLinesPrefetch ? 2 : 1;
@@ -157,7 +168,7 @@ int launch_ax32_cg(const Problem *Pb, int gprec) {
         a.x = Pb->r32;
         a.y = Pb->w32;
         a.p = Pb->p32;
-        a.xs = Pb->d32;   // d += alpha p of the previous iteration
+        a.xs = f32_defers(Pb->nq, gprec) ? Pb->d32 : nullptr;   // d += alpha p of the previous iteration
         return launch_ax32p<float, true>(Pb, a);
     }
     AxArgs<float, __nv_bfloat16> a =
@@ -165,7 +176,7 @@ int launch_ax32_cg(const Problem *Pb, int gprec) {
     a.x = Pb->r32;
     a.y = Pb->w32;
     a.p = Pb->p32;
-    a.xs = Pb->d32;   // d += alpha p of the previous iteration
+    a.xs = f32_defers(Pb->nq, gprec) ? Pb->d32 : nullptr;   // d += alpha p of the previous iteration
     return launch_ax32p<__nv_bfloat16, true>(Pb, a);
 }
 

@@ -135,7 +135,7 @@ ax32p_kernel(const AxArgs<float, GT> P, int ngroups) {
                 for (int k = 0; k < NQ; ++k) {
                     const int q = eb * NP + k * NQ2 + ij;
                     const float pn = fmaf(beta, sb[q], sa[q]);
-                    P.xs[nb + k * NQ2 + ij] = fmaf(xalpha, sb[q], P.xs[nb + k * NQ2 + ij]);
+                    if (P.xs) P.xs[nb + k * NQ2 + ij] = fmaf(xalpha, sb[q], P.xs[nb + k * NQ2 + ij]);
                     sb[q] = pn;
                     xk[k] = pn;
                     P.p[nb + k * NQ2 + ij] = pn;

@@ -17,7 +17,7 @@
 // with it, 76 us without (E = 32^3, N = 7, BF16, d not yet updated here), and
 // the sum over 16384 parts takes 3 us.
 //
-// d += alpha p of the previous iteration is applied here, where the old p is
+// d += alpha p of the previous iteration is applied here (d given), where the old p is
 // in registers anyway (+17 us), which leaves the update kernel with r and w
 // alone (sem_box.cuh, 72 -> 39 us).
 #pragma once
@@ -120,7 +120,7 @@ __device__ __forceinline__ bool lines_core_f32(const float *x, float *y, float *
         for (int k = 0; k < NQ; ++k) {
             pv[CG ? k : 0] = __ldcg(p + nb + k * NQ2);
             xk[k] = __ldcg(x + nb + k * NQ2);
-            dv[CG ? k : 0] = __ldcg(d + nb + k * NQ2);
+            if (d) dv[CG ? k : 0] = __ldcg(d + nb + k * NQ2);
         }
     }
     if (STATE) {
@@ -133,7 +133,7 @@ __device__ __forceinline__ bool lines_core_f32(const float *x, float *y, float *
         if constexpr (CG) {
 #pragma unroll
             for (int k = 0; k < NQ; ++k) {
-                d[nb + k * NQ2] = fmaf(alpha, pv[k], dv[k]);
+                if (d) d[nb + k * NQ2] = fmaf(alpha, pv[k], dv[k]);
                 xk[k] = fmaf(beta, pv[k], xk[k]);
                 p[nb + k * NQ2] = xk[k];
             }

@@ -88,7 +88,7 @@ static int launch_lines32_gt(const Problem *P, const GT *G, const float *x, floa
     a.y = cg ? P->w32 : y;
     if (cg) {
         a.p = P->p32;
-        a.xs = P->d32;   // d += alpha p of the previous iteration
+        a.xs = f32_defers(P->nq, sizeof(GT) == 4 ? kGF32 : kGBF16) ? P->d32 : nullptr;   // d += alpha p of the previous iteration
     }
     const AxLineArgs<float, GT> L = line_args(a, P->oc.D, P->nq, staged ? epb : f32_epb(P, epb));
     if (staged)

@@ -248,6 +248,7 @@ int prepare_ax32(const Problem *P);
 int convert_geometry(const Problem *P, int gprec, void *out);
 int launch_ax32(const Problem *P, const float *x, float *y, int gprec);
 int launch_ax32_cg(const Problem *P, int gprec);   // inner CG on r32/p32/d32/w32 with st_in
+bool f32_defers(int nq, int gprec);                // inner CG: d += alpha p is left to the next operator launch
 int ax32_cg_launches(const Problem *P, int gprec); // kernels of one launch_ax32_cg
 int mixed_prepare(Problem *P, int gprec);          // allocate + convert on first use
 int mixed_solve(Problem *P, const double *b, double *x, double tol, int max_outer, double inner_tol,

@@ -60,15 +60,68 @@ __global__ void mixed_inner_init_kernel(const double *__restrict__ r64, const do
     }
 }
 
+// The FP32 step over all local nodes (grid-stride), d += alpha p included, for
+// orders that do not defer it.  Bounded to 48 registers so that 5 blocks of 256
+// threads stay resident per SM: the step is latency-bound (E = 32^3, N = 7:
+// inner iteration -3 %).
+template <int NQ>
+__global__ void __launch_bounds__(256, 5) cg_update_nodes_kernel(float *__restrict__ x, float *__restrict__ r,
+                                                              const float *__restrict__ p, const float *__restrict__ w,
+                                                              int nL, BoxDims bd, double *partials, int64_t cap,
+                                                              CgState *st) {
+    __shared__ float scratch[32];
+    if (st->done) return;
+    const float alpha = float(st->alpha);
+    float acc = 0.f;
+    constexpr int V = UpdVec<NQ, float>::value;
+    const int nv = nL / V;   // nL is a multiple of (N+1), hence of V
+    for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < nv; u += gridDim.x * blockDim.x)
+        update_vec<NQ, V, float, float>(x, r, p, w, u * V, bd, alpha, acc);
+    const double bs = double(block_sum_f32(acc, scratch));
+    double rho_new;
+    if (grid_sum(bs, partials, cap, &st->ticket_up, int(blockIdx.x), int(gridDim.x), &rho_new) && threadIdx.x == 0)
+        cg_close_iteration(st, rho_new);
+}
+
+// Its launch: one resident wave (E = 32^3, N = 7: 216 -> 190 us an inner
+// iteration), not a programmatic dependent one (it reads w through L1).
+template <int NQ>
+static int launch_update_nodes(const Problem *P) {
+    constexpr int V = UpdVec<NQ, float>::value;
+    static int per_sm = 0;
+    if (!per_sm && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg_update_nodes_kernel<NQ>, 256, 0) != cudaSuccess ||
+                    per_sm < 1)) {
+        cudaGetLastError();
+        per_sm = 4;
+    }
+    const int64_t blocks = std::min<int64_t>((P->nL / V + 255) / 256, int64_t(per_sm) * sm_count());
+    cg_update_nodes_kernel<NQ><<<unsigned(blocks), 256, 0, stream()>>>(P->d32, P->r32, P->p32, P->w32, int(P->nL),
+                                                                     box_dims(P->nx, P->ny, P->nz), P->partials,
+                                                                     P->partials_cap, P->st_in);
+    count_launches(1);
+    return cuda_check(cudaGetLastError(), "cg_update_nodes_kernel");
+}
+
 // x64 += double(d32 + alpha p32): the inner solve's last step of d is still to
-// be applied (each one is left to the next operator kernel)
+// be applied where each one is left to the next operator kernel (st given)
 __global__ void mixed_correct_kernel(double *__restrict__ x, const float *__restrict__ d, const float *__restrict__ p,
                                      const CgState *__restrict__ st, int64_t n) {
     const int64_t l = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (l < n) x[l] += double(fmaf(float(st->alpha), p[l], d[l]));
+    if (l < n) x[l] += double(st ? fmaf(float(st->alpha), p[l], d[l]) : d[l]);
 }
 
-static int launch_update32(const Problem *P) {
+static int launch_update32(const Problem *P, int gprec) {
+    if (!f32_defers(P->nq, gprec)) switch (P->nq) {
+            case 2: return launch_update_nodes<2>(P);
+            case 3: return launch_update_nodes<3>(P);
+            case 4: return launch_update_nodes<4>(P);
+            case 5: return launch_update_nodes<5>(P);
+            case 6: return launch_update_nodes<6>(P);
+            case 7: return launch_update_nodes<7>(P);
+            case 8: return launch_update_nodes<8>(P);
+            case 9: return launch_update_nodes<9>(P);
+            case 10: return launch_update_nodes<10>(P);
+        }
     return launch_update_rows<float>(P, P->r32, P->w32, P->st_in);
 }
 
@@ -127,7 +180,7 @@ static int capture_inner(Problem *P, int gprec) {
     if (rc != SEM_OK) return rc;
     for (int k = 0; k < K && rc == SEM_OK; ++k) {
         rc = launch_ax32_cg(P, gprec);
-        if (rc == SEM_OK) rc = launch_update32(P);
+        if (rc == SEM_OK) rc = launch_update32(P, gprec);
     }
     count_launches(-ax32_cg_launches(P, gprec) * int64_t(K) - int64_t(K));
     const int rc_end = cuda_check(cudaStreamEndCapture(stream(), &g), "mixed: end capture");
@@ -195,7 +248,8 @@ int mixed_solve(Problem *P, const double *b, double *x, double tol, int max_oute
             if (P->st_in_host->done) break;
         }
         inner_total += P->st_in_host->iter;
-        mixed_correct_kernel<<<unsigned((P->nL + 255) / 256), 256, 0, stream()>>>(P->x, P->d32, P->p32, P->st_in,
+        mixed_correct_kernel<<<unsigned((P->nL + 255) / 256), 256, 0, stream()>>>(P->x, P->d32, P->p32,
+            f32_defers(P->nq, gprec) ? P->st_in : nullptr,
                                                                                        P->nL);
         count_launches(1);
         rc = cuda_check(cudaGetLastError(), "mixed_correct_kernel");

@@ -35,7 +35,8 @@ uint64_t g_epoch = 1;
 // the problems at hand.  FP64: the fixed-point line kernel at every order
 // (e.g. N = 3: 281 us against 1203 us for the DFMA line kernel; N = 7: 371
 // against 1579; N = 9: 576 against 2117).  FP32: the direct-load kernel at
-// every order, with the elements per block that were best at that size; with
+// every order but N = 2 with FP32 factors (f32_defers), with the elements per
+// block that were best at that size; with
 // the step of d included the TMA-staged and persistent kernels take 130 (N =
 // 7), 142 (N = 3) and 215 us (N = 2) with BF16 factors, this one 93, 106, 124.
 struct DefaultEntry {
@@ -45,7 +46,7 @@ constexpr DefaultEntry kDefault[kTuneKinds][kMaxQ + 1] = {
     // FP64
     {{0, 0}, {0, 0}, {5, 32}, {5, 14}, {5, 8}, {5, 5}, {5, 3}, {5, 5}, {5, 1}, {5, 1}, {5, 1}},
     // FP32, FP32 factors
-    {{1, 0}, {1, 0}, {1, 32}, {1, 7}, {1, 4}, {1, 5}, {1, 4}, {1, 1}, {1, 1}, {1, 1}, {1, 2}},
+    {{1, 0}, {1, 0}, {1, 32}, {2, 0}, {1, 4}, {1, 5}, {1, 4}, {1, 1}, {1, 1}, {1, 1}, {1, 2}},
     // FP32, BF16 factors
     {{1, 0}, {1, 0}, {1, 32}, {1, 14}, {1, 8}, {1, 5}, {1, 5}, {1, 1}, {1, 2}, {1, 1}, {1, 2}},
 };
