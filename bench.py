@@ -25,7 +25,7 @@ Also reported on the same JSON line:
   clocks        nvidia-smi samples taken during the timed region
   autotune      the per-order operator tuner's candidates and choices
   pcg           the same solve with the Jacobi preconditioner
-  batched       256 uneven problems, each CG phase one persistent launch
+  batched       256 uneven problems, one launch per order and CG phase
   serve         Poisson arrivals at 100..5000 req/s: p50/p99 latency, solves/s
   paper_sweep   the paper's protocol: GDOF/s against E = 2^1..2^14, N = 4, 6, 8
   vs_oracle     the small workload (E = 64, N = 7, sine source) solved on the
@@ -62,7 +62,7 @@ AX_SOURCES = [os.path.join(ROOT, "paper_2606_12650_gb300", "csrc", f)
                         "sem_internal.h", "sem_ax_fx.cuh", "sem_ax_fx.cu")]
 GOLDEN_SMALL = os.path.join(ROOT, "tests", "golden", "oracle_cg_E64_N7.npz")
 AX32_SOURCES = [os.path.join(ROOT, "paper_2606_12650_gb300", "csrc", f)
-                for f in ("sem_ax_kernel.cuh", "sem_ax_lines.cuh", "sem_ax32.cu", "sem_ax_lines32.cu", "sem_ax32p.cuh",
+                for f in ("sem_ax_kernel.cuh", "sem_ax_lines.cuh", "sem_ax32.cu", "sem_ax_lines32.cu", "sem_ax32p.cuh", "sem_ax_f32.cuh",
                           "sem_device.cuh", "sem_internal.h")]
 VARIANTS = {0: "columns", 1: "lines", 2: "persistent", 3: "lines_prefetch", 4: "lines_staged", 5: "lines_fx"}
 
@@ -456,7 +456,7 @@ def run_ours(a):
     if not a.no_mixed:
         mixed = run_mixed(a, M, b, x, t_max, job, stream, sem, torch)
 
-    # ---- batched: many uneven problems, one persistent launch per CG phase
+    # ---- batched: many uneven problems, one launch per order and CG phase
     batched = None
     if not a.no_batched:
         batched = run_batched(a, job, rank, stream, sem, torch)
@@ -663,7 +663,7 @@ def run_mixed(a, M, b, x64, t64_ms, job, stream, sem, torch):
     e1.record(stream)
     torch.cuda.synchronize()
     ax_ms = e0.elapsed_time(e1) / a.ax_reps
-    alg = E * (N + 1) ** 3 * 28   # r, p in (FP32); p, w out (FP32); 6 BF16 factors
+    alg = E * (N + 1) ** 3 * 36   # r, p, d in (FP32); p, w, d out (FP32); 6 BF16 factors
     peak, how = hbm_peak()
     gbs = alg / (ax_ms * 1e-3) / 1e9
     traffic = None
@@ -705,7 +705,7 @@ def run_mixed(a, M, b, x64, t64_ms, job, stream, sem, torch):
 def run_batched(a, job, rank, stream, sem, torch):
     """256 independent problems (E log-uniform in [8, 4096] as near-cubic boxes,
     N uniform in {3, 5, 7, 9}, jitter 5 %, random right-hand sides), each CG
-    phase of all of them one persistent launch: FP64 CG and mixed refinement
+    phase of all of them one launch per order: FP64 CG and mixed refinement
     to 1e-8.  Throughput counts every problem's own iterations."""
     import numpy as np
     from paper_2606_12650_gb300 import Batch, Mesh
@@ -743,13 +743,13 @@ def run_batched(a, job, rank, stream, sem, torch):
     setup_s = time.perf_counter() - t0
     gdof_per_iter = np.array([m.E * m.N ** 3 for m in meshes], dtype=np.float64)
     nL = np.array([m.nL for m in meshes], dtype=np.float64)
-    # algorithmic bytes per local node and CG iteration: FP64 -- operator r, p
-    # in, p, w out, 48 B of factors (80), update x, r, p, w in, x, r out (48);
-    # mixed -- FP32 operator with BF16 factors (28), FP32 update (24)
-    bytes_per_node_iter = {"fp64": 128.0, "mixed_bf16": 52.0}
+    # algorithmic bytes per local node and CG iteration: FP64 -- operator r, p,
+    # x in, p, w, x out, 48 B of factors (96), update r, w in, r out (24);
+    # mixed -- FP32 operator likewise with BF16 factors (36), FP32 update (12)
+    bytes_per_node_iter = {"fp64": 120.0, "mixed_bf16": 48.0}
     hbm, hbm_how = hbm_peak()
     out = {"workload": f"{len(meshes)} problems, E log-uniform [8, 4096] (near-cubic boxes), N in {{3,5,7,9}}, "
-                       f"jitter 5%, random RHS; tol {a.tol:g}; per order one persistent launch per CG phase, the orders in parallel",
+                       f"jitter 5%, random RHS; tol {a.tol:g}; per order one launch per CG phase, the orders in parallel",
            "problems": len(meshes), "local_dofs_total": int(B.nL_total), "tuned_per_order": tuned,
            "E_total": int(sum(m.E for m in meshes)), "setup_s": setup_s}
     for mode, name in ((0, "fp64"), (1, "mixed_bf16")):
