@@ -188,7 +188,30 @@ __global__ void mask_kernel(double *__restrict__ u, const int32_t *__restrict__ 
     if (t < n) u[idx[t]] = 0.0;
 }
 
-int launch_gs(const Problem *P, double *u) { return launch_gs_any(P, u, false); }
+// u = QQ^T u from the index lists: one thread per shared global id, its copies
+// in ascending local index.
+__global__ void gs_lists_kernel(double *__restrict__ u, const int32_t *__restrict__ ptr,
+                                const int32_t *__restrict__ idx, int64_t nseg) {
+    const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (t >= nseg) return;
+    const int32_t b0 = ptr[t], b1 = ptr[t + 1];
+    double s = u[idx[b0]];
+    for (int32_t q = b0 + 1; q < b1; ++q) s += u[idx[q]];
+    for (int32_t q = b0; q < b1; ++q) u[idx[q]] = s;
+}
+
+// N = 1 and 2 alone and without the mask from the lists (where they exist): most
+// of their nodes are corners and edges, whose copies the box form enumerates
+// with more address arithmetic than the lists take to read (1.7e7 nodes, N = 1:
+// 117 us against 146, 1e6 nodes 11.3 / 13.7; N = 2 14.5 / 15.9; from N = 3 on
+// the box form is equal or faster, e.g. N = 7 66 / 52 us).
+int launch_gs(const Problem *P, double *u) {
+    if (P->nq > 3 || !P->maps_ready) return launch_gs_any(P, u, false);
+    if (P->n_sh == 0) return SEM_OK;
+    gs_lists_kernel<<<grid_for(P->n_sh, kThreads), kThreads, 0, stream()>>>(u, P->sh_ptr, P->sh_idx, P->n_sh);
+    count_launches(1);
+    return cuda_check(cudaGetLastError(), "gs_lists_kernel");
+}
 int launch_gs_mask(const Problem *P, double *u) { return launch_gs_any(P, u, true); }
 
 int launch_mask(const Problem *P, double *u) {
