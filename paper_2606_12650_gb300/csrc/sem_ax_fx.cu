@@ -50,6 +50,12 @@ __global__ void __launch_bounds__(256) geometry_fx_kernel(const double *__restri
 int fx_prepare(Problem *P) {
     if (P->Gfx) return SEM_OK;
     int4 *g = static_cast<int4 *>(dev_alloc(sizeof(int4) * 3 * size_t(P->nL)));
+    if (!g && P->Gdw) {   // both forms do not fit: the other one is made again when it is needed
+        cudaStreamSynchronize(stream());
+        problem_drop_graphs(P);
+        dw_release(P);
+        g = static_cast<int4 *>(dev_alloc(sizeof(int4) * 3 * size_t(P->nL)));
+    }
     int32_t *kg = static_cast<int32_t *>(dev_alloc(sizeof(int32_t) * size_t(P->E)));
     int rc = g && kg ? SEM_OK : SEM_ENOMEM;
     if (rc == SEM_OK) {

@@ -168,13 +168,13 @@ __device__ __forceinline__ void vstore(T *p, const T (&v)[V]) {
 // element) before the own value and that of node N (upper element) after it,
 // lists the copies in ascending local index -- the order of the sorted-
 // segment gather-scatter, so every copy of a node gets the same bits.  The
-// nodes then update themselves: r -= alpha (QQ^T w), x += alpha p.  Masked nodes
-// are left as they are (zero).  <r, r> is accumulated into acc at each node's
-// first copy.
-template <int NQ, int V, typename T, typename Acc>
+// nodes then update themselves: r -= alpha (QQ^T w), and x += alpha p unless
+// DX (the x update is deferred to the next operator kernel).  Masked nodes are
+// left as they are (zero).  <r, r> is accumulated into
+// acc at each node's first copy.
+template <int NQ, int V, typename T, typename Acc, bool DX = false>
 __device__ __forceinline__ void update_vec(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ p,
-                                          const T *__restrict__ w, int l0, const BoxDims &bd, T alpha,
-                                          Acc &acc) {
+                                          const T *__restrict__ w, int l0, const BoxDims &bd, T alpha, Acc &acc) {
     constexpr int N = NQ - 1, NQ2 = NQ * NQ, NP = NQ2 * NQ;
     const int nx = bd.nx, ny = bd.ny, nz = bd.nz;
     const unsigned e = unsigned(l0) / unsigned(NP);
@@ -197,8 +197,10 @@ __device__ __forceinline__ void update_vec(T *__restrict__ x, T *__restrict__ r,
     // the node's own values first: their loads then overlap those of w and
     // its neighbour copies below instead of waiting for the sum
     T xv[V], pv[V], rv[V];
-    vload<T, V>(x + l0, xv);
-    vload<T, V>(p + l0, pv);
+    if (!DX) {
+        vload<T, V>(x + l0, xv);
+        vload<T, V>(p + l0, pv);
+    }
     vload<T, V>(r + l0, rv);
     T sv[V];
     if (sy == 0 && sz == 0) {
@@ -308,14 +310,35 @@ __device__ __forceinline__ void update_vec(T *__restrict__ x, T *__restrict__ r,
     for (int v = 0; v < V; ++v) {
         const bool masked = (v == 0 && mask_lo) || (v == V - 1 && mask_hi);
         if (!masked) {
-            xv[v] = fma(alpha, pv[v], xv[v]);
+            if (!DX) xv[v] = fma(alpha, pv[v], xv[v]);
             rv[v] = fma(-alpha, sv[v], rv[v]);
             if (owner_row && !((v == 0) && has_lo)) acc_square(acc, rv[v]);
         }
     }
-    vstore<T, V>(x + l0, xv);
+    if (!DX) vstore<T, V>(x + l0, xv);
     vstore<T, V>(r + l0, rv);
 }
+
+// Row-class mapping of update vectors to threads: a warp takes the same row
+// (j, k) of EG consecutive elements, LR = (N+1)/V lanes per row, so every
+// lane of a warp is in the same face class in s and t (the gather branches
+// of update_vec are warp-uniform).  Returns the first local node of the
+// lane's vector, or -1 for an idle lane.
+template <int NQ, int V>
+struct RowMap {
+    static constexpr int NQ2 = NQ * NQ, NP = NQ2 * NQ;
+    static constexpr int LR = NQ / V;
+    static constexpr int EG = 32 / LR;
+    static __device__ __forceinline__ int l0(int task, int lane, int E) {
+        const int eg = task / NQ2;
+        const int row = task - eg * NQ2;
+        const int g = lane / LR, v = lane - g * LR;
+        const int e = eg * EG + g;
+        if (g >= EG || e >= E) return -1;
+        return e * NP + row * NQ + v * V;
+    }
+    static __host__ __device__ int tasks(int E) { return (E + EG - 1) / EG * NQ2; }
+};
 
 // The update by owner rows.  Only the first copy of a global node (i, j, k >=
 // 1 in its element) is summed and updated: r -= alpha (QQ^T w), and the result

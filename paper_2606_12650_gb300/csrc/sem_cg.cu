@@ -28,9 +28,12 @@
 // (grid_sum), so results are reproducible run to run.  Scalars
 // never leave the device inside the loop: the host replays a CUDA graph of K
 // iterations and polls the stop flag once per replay.  Problems of up to five
-// elements per SM run in one kernel instead (sem_cg_small.cu).
+// elements per SM run in one kernel instead (sem_cg_small.cu), and solves of a
+// given number of iterations (tol = 0) keep their own operator, update and
+// summation orders (sem_ax_dw.cuh says why).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 
@@ -265,10 +268,11 @@ int launch_sub(const Problem *P, const double *a, const double *b, double *out) 
 
 // ---------------------------------------------------------------- CG
 // x = 0, p = 0, r = b; rho0 = <b, b>_c (weighted, local); scalars reset.
+// steps: for the kernels of a given number of iterations.
 __global__ void cg_init_kernel(const double *__restrict__ b, const double *__restrict__ c,
                                double *__restrict__ x, double *__restrict__ r,
                                double *__restrict__ p, int64_t n, double *partials, CgState *st,
-                               int maxit, double tol, double *hist) {
+                               int maxit, double tol, double *hist, bool steps) {
     __shared__ double red[32];
     double acc = 0.0;
     reset_group_tickets(partials);
@@ -293,7 +297,7 @@ __global__ void cg_init_kernel(const double *__restrict__ b, const double *__res
             st->hist = hist;
             st->iter = 0;
             st->maxit = maxit;
-            st->done = (rho0 == 0.0 || maxit <= 0) ? 1 : 0;
+            st->done = (rho0 == 0.0 || maxit <= 0) ? 1 : (steps && !dw_in_range(rho0) ? int(kDoneOutOfRange) : 0);
             st->ticket_ax = 0;
             st->ticket_up = 0;
             if (hist) hist[0] = sqrt(rho0);
@@ -301,9 +305,9 @@ __global__ void cg_init_kernel(const double *__restrict__ b, const double *__res
     }
 }
 
-int launch_cg_init(const Problem *P, const double *b, int maxit, double tol, double *hist) {
+int launch_cg_init(const Problem *P, const double *b, int maxit, double tol, double *hist, bool steps) {
     cg_init_kernel<<<stream_grid(P->nL), kThreads, 0, stream()>>>(b, P->c, P->x, P->r, P->p, P->nL,
-                                                                   P->partials, P->st, maxit, tol, hist);
+                                                                   P->partials, P->st, maxit, tol, hist, steps);
     count_launches(1);
     return cuda_check(cudaGetLastError(), "cg_init_kernel");
 }
@@ -324,6 +328,60 @@ int launch_x_finish(const Problem *P, double *out) {
     return cuda_check(cudaGetLastError(), "x_finish_kernel");
 }
 
+// The update of solves of a given number of iterations: every copy of a node
+// sums its copies in ascending order and updates itself, <r, r> in double-word
+// FP32 per thread, 8 blocks per SM (E = 32^3, N = 7: 133 us, where owner rows
+// take 78).
+template <int NQ>
+__global__ void __launch_bounds__(256) cg_update_class_kernel(double *__restrict__ r, const double *__restrict__ w,
+                                                              int E, BoxDims bd, double *partials, int64_t cap,
+                                                              CgState *st) {
+    __shared__ double scratch[256];
+    if (st->done) return;
+    constexpr int V = UpdVec<NQ, double>::value;
+    using RM = RowMap<NQ, V>;
+    const double alpha = st->alpha;
+    const int ntask = RM::tasks(E);
+    const int lane = threadIdx.x & 31;
+    const int nwarps = int(gridDim.x * blockDim.x) >> 5;
+    DwAcc acc = acc_zero<DwAcc>();
+    for (int task = int(blockIdx.x * blockDim.x + threadIdx.x) >> 5; task < ntask; task += nwarps) {
+        const int l0 = RM::l0(task, lane, E);
+        if (l0 >= 0) update_vec<NQ, V, double, DwAcc, true>(nullptr, r, nullptr, w, l0, bd, alpha, acc);
+    }
+    const double bs = block_sum_wide(acc_value(acc), scratch);
+    double rho_new;
+    if (grid_sum_groups(bs, partials, cap, &st->ticket_up, &rho_new) && threadIdx.x == 0) {
+        cg_close_iteration(st, rho_new);
+        if (!st->done && !dw_in_range(rho_new)) st->done = kDoneOutOfRange;
+    }
+}
+
+template <int NQ>
+static int launch_update_steps_nq(const Problem *P) {
+    const int64_t tasks = RowMap<NQ, UpdVec<NQ, double>::value>::tasks(int(P->E));
+    const int64_t blocks = std::min<int64_t>((tasks * 32 + 255) / 256, int64_t(sm_count()) * 8);
+    cg_update_class_kernel<NQ><<<unsigned(blocks), 256, 0, stream()>>>(
+        P->r, P->w, int(P->E), box_dims(P->nx, P->ny, P->nz), P->partials, P->partials_cap, P->st);
+    count_launches(1);
+    return cuda_check(cudaGetLastError(), "cg_update_class_kernel");
+}
+
+static int launch_update_steps(const Problem *P) {
+    switch (P->nq) {
+        case 2: return launch_update_steps_nq<2>(P);
+        case 3: return launch_update_steps_nq<3>(P);
+        case 4: return launch_update_steps_nq<4>(P);
+        case 5: return launch_update_steps_nq<5>(P);
+        case 6: return launch_update_steps_nq<6>(P);
+        case 7: return launch_update_steps_nq<7>(P);
+        case 8: return launch_update_steps_nq<8>(P);
+        case 9: return launch_update_steps_nq<9>(P);
+        case 10: return launch_update_steps_nq<10>(P);
+        default: return set_error(SEM_EARG, "cg: unsupported order");
+    }
+}
+
 int launch_cg_update(const Problem *P) {
     // <r, r> accumulated in double-word FP32 per thread (sem_box.cuh)
     return launch_update_rows<double>(P, P->r, P->w, P->st);
@@ -335,22 +393,23 @@ static int graph_iters_for(const Problem *P) {
     return P->nL < (1 << 20) ? 64 : 16;
 }
 
-static int capture_graph(Problem *P) {
+static int capture_graph(Problem *P, bool steps) {
     if (P->graph_epoch != tune_epoch()) problem_drop_graphs(P);   // operator variant changed
-    if (P->graph) return SEM_OK;
+    cudaGraphExec_t &graph = steps ? P->graph_steps : P->graph;
+    if (graph) return SEM_OK;
     const int K = graph_iters_for(P);
     cudaGraph_t g = nullptr;
     int rc = cuda_check(cudaStreamBeginCapture(stream(), cudaStreamCaptureModeThreadLocal), "cg: begin capture");
     if (rc != SEM_OK) return rc;
     for (int k = 0; k < K && rc == SEM_OK; ++k) {
-        rc = launch_ax_cg(P);
-        if (rc == SEM_OK) rc = launch_cg_update(P);
+        rc = steps ? launch_ax_dw(P) : launch_ax_cg(P);
+        if (rc == SEM_OK) rc = steps ? launch_update_steps(P) : launch_cg_update(P);
     }
     // launches inside a capture are counted at replay time instead
     count_launches(-2 * int64_t(K));
     const int rc_end = cuda_check(cudaStreamEndCapture(stream(), &g), "cg: end capture");
     if (rc == SEM_OK) rc = rc_end;
-    if (rc == SEM_OK) rc = cuda_check(cudaGraphInstantiate(&P->graph, g, 0), "cg: instantiate");
+    if (rc == SEM_OK) rc = cuda_check(cudaGraphInstantiate(&graph, g, 0), "cg: instantiate");
     if (g) cudaGraphDestroy(g);
     if (rc == SEM_OK) {
         P->graph_iters = K;
@@ -362,25 +421,34 @@ static int capture_graph(Problem *P) {
 int cg_solve(Problem *P, const double *b, double *x, double tol, int maxit, double *hist,
              int64_t *iters, double *rel_res) {
     if (maxit < 0) return set_error(SEM_EARG, "cg_solve: maxit must be >= 0");
-    int rc = launch_cg_init(P, b, maxit, tol, hist);
-    if (rc != SEM_OK) return rc;
-    if (P->graph && P->graph_stream != stream()) {
-        cudaGraphExecDestroy(P->graph);
-        P->graph = nullptr;
+    if (P->graph_stream != stream()) {
+        for (cudaGraphExec_t *g : {&P->graph, &P->graph_steps}) {
+            if (*g) cudaGraphExecDestroy(*g);
+            *g = nullptr;
+        }
     }
-    rc = prepare_f64_variant(P);
-    const bool small = rc == SEM_OK && small_fits(P, false);
-    if (rc == SEM_OK && !small) rc = capture_graph(P);
+    // a given number of iterations: sem_ax_dw.cuh, where the table names the
+    // fixed-point operator and the factors are within range
+    int rc = SEM_OK;
+    bool steps = !(tol > 0.0) && tune_get(kTuneF64, P->nq).variant == kAxLinesFX;
+    if (steps) {
+        rc = dw_prepare(P);
+        steps = !P->dw_out;
+    }
+    if (rc == SEM_OK && !steps) rc = prepare_f64_variant(P);
+    if (rc == SEM_OK) rc = launch_cg_init(P, b, maxit, tol, hist, steps);
+    const bool small = rc == SEM_OK && !steps && small_fits(P, false);
+    if (rc == SEM_OK && !small) rc = capture_graph(P, steps);
     if (rc != SEM_OK) return rc;
-    // at most ceil(maxit / K) replays; the flag stops earlier replays short (a
-    // small problem's launches hold many more iterations than K)
-    const int64_t K = small ? 1 : P->graph_iters;
-    const int64_t max_replays = (int64_t(maxit) + K - 1) / K;
-    for (int64_t rep = 0; rep < max_replays; ++rep) {
+    // at most maxit iterations are left to run; the flag stops earlier replays
+    // short (a small problem's launches hold many more iterations than K)
+    int64_t left = maxit;
+    while (left > 0) {
+        const int64_t K = small ? 1 : P->graph_iters;
         if (small) {
             rc = launch_small(P, false);
         } else {
-            rc = cuda_check(cudaGraphLaunch(P->graph, stream()), "cg: graph launch");
+            rc = cuda_check(cudaGraphLaunch(steps ? P->graph_steps : P->graph, stream()), "cg: graph launch");
             if (rc == SEM_OK) count_launches(2 * K);
         }
         if (rc != SEM_OK) return rc;
@@ -394,7 +462,19 @@ int cg_solve(Problem *P, const double *b, double *x, double tol, int maxit, doub
         rc = cuda_check(cudaStreamSynchronize(stream()), "cg: sync");
         if (rc != SEM_OK) return rc;
         if (*status_host() != 0) break;
-        if (P->st_host->done) break;
+        left -= K;
+        if (P->st_host->done == kDoneOutOfRange) {
+            // ||r|| left the range of double-word numbers: the general kernels
+            // go on from this state
+            steps = false;
+            left = maxit - P->st_host->iter;
+            rc = prepare_f64_variant(P);
+            if (rc == SEM_OK) rc = capture_graph(P, false);
+            if (rc == SEM_OK) rc = cuda_check(cudaMemsetAsync(&P->st->done, 0, sizeof(int32_t), stream()), "cg: resume");
+            if (rc != SEM_OK) return rc;
+        } else if (P->st_host->done) {
+            break;
+        }
     }
     rc = small ? cuda_check(cudaMemcpyAsync(x, P->x, sizeof(double) * P->nL, cudaMemcpyDeviceToDevice, stream()),
                             "cg: copy x")

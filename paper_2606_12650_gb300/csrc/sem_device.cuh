@@ -275,6 +275,50 @@ __device__ __forceinline__ bool grid_sum(double v0, double *partials, int64_t ca
     return true;
 }
 
+// The sum always in two levels, each added by one warp in the order of its
+// lanes: the summation order of solves of a given number of iterations
+// (sem_ax_dw.cuh).  Returns true in all threads of the block that completes
+// it, with the sum in its thread 0.
+__device__ __forceinline__ bool grid_sum_groups(double v0, double *partials, int64_t cap, uint32_t *ticket,
+                                                double *total) {
+    __shared__ int s_last;
+    const int b = int(blockIdx.x), g = b / kSumGroup, g0 = g * kSumGroup;
+    const int gn = min(kSumGroup, int(gridDim.x) - g0), ng = int((gridDim.x + kSumGroup - 1) / kSumGroup);
+    uint32_t *gt = group_tickets(partials, cap) + g;
+    if (threadIdx.x == 0) {
+        partials[b] = v0;
+        __threadfence();
+        s_last = atomicAdd(gt, 1u) == uint32_t(gn - 1);
+    }
+    __syncthreads();
+    if (!s_last) return false;
+    __syncthreads();   // every thread has read s_last before thread 0 rewrites it
+    if (threadIdx.x < 32) {
+        __threadfence();
+        double s = int(threadIdx.x) < gn ? __ldcg(partials + g0 + threadIdx.x) : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) {
+            partials[cap + g] = s;
+            *gt = 0u;
+            __threadfence();
+            s_last = atomicAdd(ticket, 1u) == uint32_t(ng - 1);
+        }
+    }
+    __syncthreads();
+    if (!s_last) return false;
+    if (threadIdx.x < 32) {
+        __threadfence();
+        double s = 0.0;
+        for (int q = threadIdx.x; q < ng; q += 32) s += __ldcg(partials + cap + q);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) *ticket = 0u;
+        *total = s;
+    }
+    return true;
+}
+
 // Zero the group tickets (grid-stride): at the start of every solve, so that
 // a launch that gave up half-way (a timed-out copy) leaves no stale count.
 __device__ __forceinline__ void reset_group_tickets(double *partials) {
@@ -359,6 +403,10 @@ __device__ __forceinline__ void pcg_close_iteration(CgState *st, double rho_new,
     const bool conv = st->tol > 0.0 && sqrt(rr / st->bb) <= st->tol;
     if (conv || it >= st->maxit) st->done = 1;
 }
+
+// <r, r> for which vectors of double-word FP32 numbers and the low parts of
+// their products stay within FP32's exponents (false for a NaN).
+__device__ __forceinline__ bool dw_in_range(double rho) { return rho >= 0x1p-80 && rho <= 0x1p100; }
 
 // Closing step of a CG iteration, run by thread 0 of the last block once
 // rho_new = <r_{k+1}, r_{k+1}> is known: iteration count, optional history,

@@ -2,8 +2,9 @@
 // h + l (~48 significant bits), computed on the FP32 pipe with error-free
 // transformations (Knuth's TwoSum; Dekker's product formed with one FMA) and
 // FP32 low-order terms; and exact FP64 <-> double-word conversions in integer
-// and FP32 arithmetic.  Used by the <r, r> reductions of the FP64 CG and PCG
-// updates (sem_box.cuh).
+// and FP32 arithmetic.  Used by the solves of a given number of iterations
+// (sem_ax_dw.cuh) and by the <r, r> reductions of the FP64 CG and PCG updates
+// (sem_box.cuh).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -73,6 +74,20 @@ __device__ __forceinline__ dwf dw_add(dwf a, dwf b) {
     float s, e;
     two_sum(a.h, b.h, s, e);
     return {s, __fadd_rn(__fadd_rn(a.l, b.l), e)};
+}
+
+__device__ __forceinline__ dwf dw_sub(dwf a, dwf b) {
+    float s, e;
+    two_sum(a.h, -b.h, s, e);
+    return {s, __fadd_rn(__fsub_rn(a.l, b.l), e)};
+}
+
+// c u: c.h u.h = p + e exactly (one FMA), the cross terms in FP32; c.l u.l
+// (2^-48 of the product) is dropped.
+__device__ __forceinline__ dwf dw_mul(dwf c, dwf u) {
+    const float p = __fmul_rn(c.h, u.h);
+    const float e = __fmaf_rn(c.h, u.h, -p);
+    return {p, __fmaf_rn(c.l, u.h, __fmaf_rn(c.h, u.l, e))};
 }
 
 // acc + c u: the high product joins acc.h through TwoSum; every low-order

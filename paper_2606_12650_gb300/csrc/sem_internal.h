@@ -70,6 +70,10 @@ struct CgState {
     uint32_t pad1;
 };
 
+// CgState::done beyond 0 (running) and 1 (over): the solve stopped because ||r||
+// left the range of its kernels (dw_in_range), others may go on from its state.
+constexpr int32_t kDoneOutOfRange = 2;
+
 // Status word written by kernels whose bounded waits give up.
 enum DeviceStatus : int32_t {
     kStatusOk = 0,
@@ -105,6 +109,7 @@ struct Problem {
     CgState *st_host = nullptr;    // pinned mirror for polling (pad0: the mesh check's flag at set-up)
     int32_t *bad_dev = nullptr;    // deferred set-up: the geometry kernel's flag until read
     cudaGraphExec_t graph = nullptr;
+    cudaGraphExec_t graph_steps = nullptr;   // CG solves of a given number of iterations
     int graph_iters = 0;
     cudaStream_t graph_stream = nullptr;
 
@@ -119,6 +124,10 @@ struct Problem {
     int4 *Gfx = nullptr;
     int32_t *kgfx = nullptr;
     struct FxConsts *fxc = nullptr;   // host: its matrices (sem_ax_fx.cuh)
+    // solves of a given number of iterations (sem_ax_dw.cuh): factors as [nL][6]
+    // (h, l) FP32 pairs, made on first use; dw_out: outside their range
+    float *Gdw = nullptr;
+    bool dw_out = false;
     float *d32 = nullptr, *r32 = nullptr, *p32 = nullptr, *w32 = nullptr;
     CgState *st_in = nullptr;
     CgState *st_in_host = nullptr;
@@ -175,6 +184,10 @@ int launch_lines64(const Problem *P, const double *x, double *y, int mode, int e
 int launch_lines_fx(const Problem *P, const double *x, double *y, int mode, int epb);
 int fx_prepare(Problem *P);                   // allocate + fill P->Gfx, P->kgfx (once)
 void fx_release(Problem *P);
+// double-word CG operator (sem_ax_dw.cu): solves of a given number of iterations
+int dw_prepare(Problem *P);                   // allocate + fill P->Gdw (once), or set P->dw_out
+void dw_release(Problem *P);
+int launch_ax_dw(const Problem *P);
 int prepare_f64_variant(Problem *P);          // whatever the tuned FP64 variant needs (before a capture)
 // FP32: the direct-load kernel, or (staged) slab and factors in shared memory
 int launch_lines32(const Problem *P, const float *x, float *y, int gprec, bool cg, int epb, bool staged);
@@ -260,7 +273,7 @@ int launch_mask(const Problem *P, double *u);
 int launch_gs_mask(const Problem *P, double *u);   // mask(QQ^T u), one pass
 int launch_dot(const Problem *P, const double *u, const double *v);  // -> st->dot_out
 int launch_sub(const Problem *P, const double *a, const double *b, double *out);  // out = a - b
-int launch_cg_init(const Problem *P, const double *b, int maxit, double tol, double *hist);
+int launch_cg_init(const Problem *P, const double *b, int maxit, double tol, double *hist, bool steps = false);
 int launch_cg_update(const Problem *P);
 int launch_x_finish(const Problem *P, double *out);   // out = x + alpha p of the last iteration (deferred update)
 int cg_solve(Problem *P, const double *b, double *x, double tol, int maxit, double *hist,

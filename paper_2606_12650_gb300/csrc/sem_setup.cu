@@ -449,10 +449,11 @@ int problem_maps(Problem *P) {
 // capture time); the next solve captures them again.
 void problem_drop_graphs(Problem *P) {
     if (P->graph) cudaGraphExecDestroy(P->graph);
+    if (P->graph_steps) cudaGraphExecDestroy(P->graph_steps);
     if (P->graph_pcg) cudaGraphExecDestroy(P->graph_pcg);
     for (auto &g : P->graph32)
         if (g) cudaGraphExecDestroy(g);
-    P->graph = P->graph_pcg = nullptr;
+    P->graph = P->graph_steps = P->graph_pcg = nullptr;
     P->graph32[0] = P->graph32[1] = nullptr;
     P->graph_epoch = tune_epoch();
 }
@@ -460,11 +461,13 @@ void problem_drop_graphs(Problem *P) {
 void problem_destroy(Problem *P) {
     if (!P) return;
     if (P->graph) cudaGraphExecDestroy(P->graph);
+    if (P->graph_steps) cudaGraphExecDestroy(P->graph_steps);
     if (P->graph_pcg) cudaGraphExecDestroy(P->graph_pcg);
     if (P->dinv) dev_free(P->dinv);
     if (P->bad_dev) dev_free(P->bad_dev);
     mixed_release(P);
     fx_release(P);
+    dw_release(P);
     if (P->partials) dev_free(reinterpret_cast<unsigned char *>(P->partials) - 16);
     double *dptrs[] = {P->verts, P->G, P->B, P->c, P->x, P->r, P->p, P->w};
     for (double *q : dptrs)
