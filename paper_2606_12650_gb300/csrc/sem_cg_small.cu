@@ -135,6 +135,9 @@ __device__ __forceinline__ bool exchange(uint64_t *slots, int nb, int e, uint32_
         double v[NV];
         ok = get_share<NV, FENCE>(slots + size_t(2 * NV) * e, min(32, nb - e), epoch, v);
         ok = __all_sync(0xffffffffu, ok);
+        // orders every lane's reads (and fence) before lane 0's store below: votes
+        // and shuffles do not order memory between lanes
+        __syncwarp();
 #pragma unroll
         for (int c = 0; c < NV; ++c) {
 #pragma unroll
