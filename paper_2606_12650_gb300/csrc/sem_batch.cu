@@ -726,18 +726,17 @@ __global__ void __launch_bounds__(kBatchThreads, MODE == kVecUpdate32 ? kUpd32Bl
     leave_queue(q);
 }
 
-// The owner-row update of a block order.
+// The owner-row update of a block order, <r, r> in the vectors' precision.
 template <int NQ, typename T>
 __global__ void __launch_bounds__(256, kOwnerBlocks)
     batch_owner_kernel(const OwnerItem *items, BatchProb *probs, BatchCtl *ctl, int32_t *finished_ids) {
-    using Acc = typename std::conditional<sizeof(T) == 8, DwAcc, float>::type;
     __shared__ double scratch[256];
     const OwnerItem it = items[blockIdx.x];
     pdl_wait();
     if (it.nb == 0 || it.st->done) return;
-    Acc acc = acc_zero<Acc>(), unused = acc_zero<Acc>();
+    T acc = T(0), unused = T(0);
     owner_tasks<NQ, false, T>(static_cast<T *>(it.r), static_cast<const T *>(it.w), nullptr,
-                              8 * it.b + int(threadIdx.x >> 5), 8 * it.nb, it.E, it.bd, T(it.st->alpha), acc, unused);
+                              8 * it.b + int(threadIdx.x >> 5), 8 * it.nb, it.E, it.bd, T(it.st->alpha), 0, acc, unused);
     const double bs = owner_block_sum(acc, scratch);
     double rho_new;
     if (grid_sum(bs, it.partials, it.cap, &it.st->ticket_up, it.b, it.nb, &rho_new) && threadIdx.x == 0) {

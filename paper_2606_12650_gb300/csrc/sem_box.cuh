@@ -85,19 +85,19 @@ __device__ __forceinline__ BoxNode box_node(int l, int nx, int ny, int nz) {
 
 namespace sem {
 
-// Accumulators of <r, r>: FP64 or FP32 fma, or (FP64 CG update) double-word
+// Accumulators of <r, r>: FP64 or FP32 fma, or (FP64 CG and PCG updates) double-word
 // FP32, which takes the reduction off GB300's 1/64-rate FP64 pipe; the
-// recurrences (copy sums, r -= alpha w) stay FP64.
+// recurrences (copy sums, r -= alpha w) stay FP64.  bias: of the conversion to
+// double-word, see dw_shift.
 struct DwAcc {
     dwf v;
 };
-__device__ __forceinline__ void acc_square(double &a, double r) { a = fma(r, r, a); }
-__device__ __forceinline__ void acc_square(float &a, float r) { a = fmaf(r, r, a); }
-__device__ __forceinline__ void acc_square(DwAcc &a, double r) { a.v = dw_add_square(a.v, r); }
-// Jacobi PCG: acc + d r^2 (= r . (d r) with z = d r), FP64 or double-word
-__device__ __forceinline__ void acc_weighted_square(double &a, double d, double r) { a = fma(r, d * r, a); }
-__device__ __forceinline__ void acc_weighted_square(DwAcc &a, double d, double r) {
-    a.v = dw_add_weighted_square(a.v, d, r);
+__device__ __forceinline__ void acc_square(double &a, double r, int) { a = fma(r, r, a); }
+__device__ __forceinline__ void acc_square(float &a, float r, int) { a = fmaf(r, r, a); }
+__device__ __forceinline__ void acc_square(DwAcc &a, double r, int bias) { a.v = dw_add_square(a.v, r, bias); }
+// Jacobi PCG: acc + d r^2 (= r . (d r) with z = d r)
+__device__ __forceinline__ void acc_weighted_square(DwAcc &a, double d, double r, int bias) {
+    a.v = dw_add_weighted_square(a.v, d, r, bias);
 }
 __device__ __forceinline__ double acc_value(double a) { return a; }
 __device__ __forceinline__ double acc_value(float a) { return double(a); }
@@ -312,7 +312,7 @@ __device__ __forceinline__ void update_vec(T *__restrict__ x, T *__restrict__ r,
         if (!masked) {
             if (!DX) xv[v] = fma(alpha, pv[v], xv[v]);
             rv[v] = fma(-alpha, sv[v], rv[v]);
-            if (owner_row && !((v == 0) && has_lo)) acc_square(acc, rv[v]);
+            if (owner_row && !((v == 0) && has_lo)) acc_square(acc, rv[v], kDwBias);
         }
     }
     if (!DX) vstore<T, V>(x + l0, xv);
@@ -370,7 +370,7 @@ struct OwnerRows {
 
 template <int NQ, int CY, int CZ, bool PRE, typename T, typename Acc>
 __device__ __forceinline__ void owner_rows(T *r, const T *w, const T *__restrict__ dinv, int j, int k, int eg, int lane,
-                                           int E, const BoxDims &bd, T alpha, Acc &acc, Acc &acc_rr) {
+                                           int E, const BoxDims &bd, T alpha, int bias, Acc &acc, Acc &acc_rr) {
     using R = OwnerRows<NQ, T>;
     constexpr int V = R::V, N = R::N, NP = R::NP, LR = R::LR, EG = R::EG, C = CY * CZ;
     const int g = lane / LR, v = lane - g * LR;
@@ -430,10 +430,10 @@ __device__ __forceinline__ void owner_rows(T *r, const T *w, const T *__restrict
         rv[q] = fma(masked ? T(0) : -alpha, s[q], rv[q]);
         if (live && !masked && !(q == 0 && first)) {
             if constexpr (PRE) {
-                acc_weighted_square(acc, dv[q], rv[q]);
-                acc_square(acc_rr, rv[q]);
+                acc_weighted_square(acc, dv[q], rv[q], bias);
+                acc_square(acc_rr, rv[q], bias);
             } else {
-                acc_square(acc, rv[q]);
+                acc_square(acc, rv[q], bias);
             }
         }
     }
@@ -460,18 +460,18 @@ __device__ __forceinline__ void owner_rows(T *r, const T *w, const T *__restrict
 // One task: row (j, k) of element group eg, tasks numbered row fastest.
 template <int NQ, bool PRE, typename T, typename Acc>
 __device__ __forceinline__ void owner_task(T *r, const T *w, const T *dinv, int task, int lane, int E,
-                                           const BoxDims &bd, T alpha, Acc &acc, Acc &acc_rr) {
+                                           const BoxDims &bd, T alpha, int bias, Acc &acc, Acc &acc_rr) {
     constexpr int N = NQ - 1;
     const int eg = task / (N * N), row = task - eg * (N * N);
     const int k = 1 + row / N, j = 1 + row - (k - 1) * N;
     if (j < N && k < N)
-        owner_rows<NQ, 1, 1, PRE>(r, w, dinv, j, k, eg, lane, E, bd, alpha, acc, acc_rr);
+        owner_rows<NQ, 1, 1, PRE>(r, w, dinv, j, k, eg, lane, E, bd, alpha, bias, acc, acc_rr);
     else if (k < N)
-        owner_rows<NQ, 2, 1, PRE>(r, w, dinv, j, k, eg, lane, E, bd, alpha, acc, acc_rr);
+        owner_rows<NQ, 2, 1, PRE>(r, w, dinv, j, k, eg, lane, E, bd, alpha, bias, acc, acc_rr);
     else if (j < N)
-        owner_rows<NQ, 1, 2, PRE>(r, w, dinv, j, k, eg, lane, E, bd, alpha, acc, acc_rr);
+        owner_rows<NQ, 1, 2, PRE>(r, w, dinv, j, k, eg, lane, E, bd, alpha, bias, acc, acc_rr);
     else
-        owner_rows<NQ, 2, 2, PRE>(r, w, dinv, j, k, eg, lane, E, bd, alpha, acc, acc_rr);
+        owner_rows<NQ, 2, 2, PRE>(r, w, dinv, j, k, eg, lane, E, bd, alpha, bias, acc, acc_rr);
 }
 
 // The tasks of warp `wid` of `nw`: a contiguous run, so that every warp gets
@@ -479,12 +479,12 @@ __device__ __forceinline__ void owner_task(T *r, const T *w, const T *dinv, int 
 // the same row each time: 133 -> 106 us at N = 7 for the former kernel).
 template <int NQ, bool PRE, typename T, typename Acc>
 __device__ __forceinline__ void owner_tasks(T *r, const T *w, const T *dinv, int wid, int nw, int E,
-                                            const BoxDims &bd, T alpha, Acc &acc, Acc &acc_rr) {
+                                            const BoxDims &bd, T alpha, int bias, Acc &acc, Acc &acc_rr) {
     const int ntask = int(OwnerRows<NQ, T>::tasks(E));
     const int per = (ntask + nw - 1) / nw;
     const int end = min(ntask, (wid + 1) * per);
     for (int task = wid * per; task < end; ++task)
-        owner_task<NQ, PRE>(r, w, dinv, task, int(threadIdx.x & 31), E, bd, alpha, acc, acc_rr);
+        owner_task<NQ, PRE>(r, w, dinv, task, int(threadIdx.x & 31), E, bd, alpha, bias, acc, acc_rr);
 }
 
 // The block's sum of an owner-row accumulator (thread 0): FP32 values in FP32,
@@ -492,7 +492,8 @@ __device__ __forceinline__ void owner_tasks(T *r, const T *w, const T *dinv, int
 __device__ __forceinline__ double owner_block_sum(float acc, double *scratch) {
     return double(block_sum_f32(acc, reinterpret_cast<float *>(scratch)));
 }
-__device__ __forceinline__ double owner_block_sum(const DwAcc &acc, double *scratch) {
+template <typename Acc>
+__device__ __forceinline__ double owner_block_sum(const Acc &acc, double *scratch) {
     return block_sum_wide(acc_value(acc), scratch);
 }
 
@@ -543,13 +544,14 @@ __global__ void __launch_bounds__(256, kOwnerBlocks)
     __shared__ double scratch[256];
     pdl_wait();
     if (st->done) return;
+    const int k = sizeof(T) == 8 ? dw_shift(st->rho) : 0;
     Acc acc = acc_zero<Acc>(), unused = acc_zero<Acc>();
     owner_tasks<NQ, false, T>(r, w, nullptr, int(blockIdx.x * blockDim.x + threadIdx.x) >> 5,
-                              int(gridDim.x * blockDim.x) >> 5, E, bd, T(st->alpha), acc, unused);
+                              int(gridDim.x * blockDim.x) >> 5, E, bd, T(st->alpha), kDwBias - k, acc, unused);
     const double bs = owner_block_sum(acc, scratch);
     double rho_new;
     if (grid_sum(bs, partials, cap, &st->ticket_up, int(blockIdx.x), int(gridDim.x), &rho_new) && threadIdx.x == 0)
-        cg_close_iteration(st, rho_new);
+        cg_close_iteration(st, dw_unscale(rho_new, k));
 }
 
 template <int NQ, typename T>

@@ -32,19 +32,21 @@ struct alignas(8) dwf {
 // |k| < 2^22) joined by one FMA (so l = rn(m) 2^(e-1075)), scaled by two
 // powers of two (each representable for 2^-126 <= |d|), and given d's sign.
 // |d| < 2^-126 (and zero) gives (+-0, 0); |d| >= 2^128 is outside the range.
-__device__ __forceinline__ dwf dw_from_double(double d) {
+// bias = kDwBias - k converts d 2^k instead: the same bits, another exponent.
+constexpr int kDwBias = 896;
+__device__ __forceinline__ dwf dw_from_double(double d, int bias = kDwBias) {
     const uint64_t bits = uint64_t(__double_as_longlong(d));
     const uint32_t hi = uint32_t(bits >> 32);
     const uint32_t sign = hi & 0x80000000u;
     const uint32_t e = (hi >> 20) & 0x7ffu;
     const uint64_t rb = bits + (uint64_t(1) << 28);
-    const uint32_t hb = ((uint32_t(rb >> 29) - (384u << 23)) & 0x7fffffffu) | sign;
+    const uint32_t hb = ((uint32_t(rb >> 29) - (uint32_t(bias) << 23)) & 0x7fffffffu) | sign;
     const int32_t m = int32_t(uint32_t(rb) & 0x1fffffffu) - 0x10000000;
     const float fmh = __fsub_rn(__uint_as_float(0x4b400000u + uint32_t(m >> 14)), 12582912.0f);
     const float fml = __fsub_rn(__uint_as_float(0x4b000000u | (uint32_t(m) & 0x3fffu)), 8388608.0f);
     const float fm = __fmaf_rn(fmh, 16384.0f, fml);
-    const float l = __fmul_rn(__fmul_rn(fm, 0x1p-52f), __uint_as_float((e - 896u) << 23));
-    if (e < 897u) return {__uint_as_float(sign), 0.0f};
+    const float l = __fmul_rn(__fmul_rn(fm, 0x1p-52f), __uint_as_float((e - uint32_t(bias)) << 23));
+    if (int(e) <= bias) return {__uint_as_float(sign), 0.0f};
     return {__uint_as_float(hb), __uint_as_float(__float_as_uint(l) ^ sign)};
 }
 
@@ -61,6 +63,20 @@ __device__ __forceinline__ double widen_f32(float f) {
 
 // h + l rounded once to FP64 (one FP64 addition).
 __device__ __forceinline__ double dw_to_double(dwf v) { return widen_f32(v.h) + widen_f32(v.l); }
+
+// The power of two by which vectors of squared norm rho are multiplied on
+// conversion, so that their squares and the low parts of those stay within
+// FP32's exponents at any FP64 magnitude: 0 for 2^-64 <= rho <= 2^100, else k
+// with rho 4^k near 1 (|k| <= 480: kDwBias - k stays positive).  Sums of such
+// squares are multiplied by 4^-k once (dw_unscale).
+__device__ __forceinline__ int dw_shift(double rho) {
+    const int e = int(uint32_t(__double2hiint(rho)) >> 20 & 0x7ffu) - 1023;
+    return e >= -64 && e <= 100 ? 0 : max(-480, min(480, -(e >> 1)));
+}
+__device__ __forceinline__ double dw_unscale(double s, int k) {
+    const double f = __hiloint2double((1023 - k) << 20, 0);
+    return s * f * f;
+}
 
 // s + e = a + b exactly (Knuth's TwoSum: no ordering of |a|, |b| needed).
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
@@ -101,10 +117,10 @@ __device__ __forceinline__ dwf dw_fma(dwf c, dwf u, dwf acc) {
     return {s, __fadd_rn(t, __fadd_rn(e, f))};
 }
 
-// acc + r^2 for an FP64 r: r = h + l exactly to ~2^-49, r^2 = h^2 + 2hl +
+// acc + r^2 for an FP64 r (converted times 2^k): r = h + l exactly to ~2^-49, r^2 = h^2 + 2hl +
 // l^2 with h^2 = p + e exactly (one FMA) and l^2 (2^-48 of r^2) dropped.
-__device__ __forceinline__ dwf dw_add_square(dwf acc, double r) {
-    const dwf v = dw_from_double(r);
+__device__ __forceinline__ dwf dw_add_square(dwf acc, double r, int bias) {
+    const dwf v = dw_from_double(r, bias);
     const float p = __fmul_rn(v.h, v.h);
     const float e = __fmaf_rn(v.h, v.h, -p);
     const float t = __fmaf_rn(__fmul_rn(2.0f, v.h), v.l, acc.l);
@@ -115,8 +131,8 @@ __device__ __forceinline__ dwf dw_add_square(dwf acc, double r) {
 
 // acc + d r^2 for FP64 d, r (the Jacobi-weighted <r, M^-1 r> term):
 // r^2 = p + (e + 2hl) as in dw_add_square, then times d's double-word form.
-__device__ __forceinline__ dwf dw_add_weighted_square(dwf acc, double d, double r) {
-    const dwf v = dw_from_double(r);
+__device__ __forceinline__ dwf dw_add_weighted_square(dwf acc, double d, double r, int bias) {
+    const dwf v = dw_from_double(r, bias);
     const dwf w = dw_from_double(d);
     const float p = __fmul_rn(v.h, v.h);
     const float e = __fmaf_rn(v.h, v.h, -p);

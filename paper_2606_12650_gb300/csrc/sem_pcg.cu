@@ -127,15 +127,16 @@ __global__ void __launch_bounds__(256, kOwnerBlocks)
     __shared__ double red[32];
     pdl_wait();
     if (st->done) return;
+    const int k = dw_shift(st->rr);
     DwAcc rz = acc_zero<DwAcc>(), rr = acc_zero<DwAcc>();
     owner_tasks<NQ, true>(r, w, dinv, int(blockIdx.x * blockDim.x + threadIdx.x) >> 5,
-                          int(gridDim.x * blockDim.x) >> 5, E, bd, st->alpha, rz, rr);
+                          int(gridDim.x * blockDim.x) >> 5, E, bd, st->alpha, kDwBias - k, rz, rr);
     const double s0 = block_sum(acc_value(rz), red);
     const double s1 = block_sum(acc_value(rr), red);
     if (publish_partial2(s0, s1, partials, &st->ticket_up)) {
         double rho_new, rr_new;
         finish_partials2(partials, int(gridDim.x), &st->ticket_up, red, &rho_new, &rr_new);
-        if (threadIdx.x == 0) pcg_close_iteration(st, rho_new, rr_new);
+        if (threadIdx.x == 0) pcg_close_iteration(st, dw_unscale(rho_new, k), dw_unscale(rr_new, k));
     }
 }
 
