@@ -2,7 +2,8 @@
 // mixed-precision iterative refinement: the choice of the kernel, and the
 // persistent, double-buffered one (sem_ax32p.cuh).  FP32 vectors and arithmetic, geometric factors stored in
 // FP32 (24 B/node) or BF16 (12 B/node) and widened exactly to FP32; the CG
-// variant's <p, A p> is reduced across threads and blocks in FP64.  Also the
+// variant's <p, A p> is reduced across blocks in FP64, and across threads in
+// FP64 by the persistent kernel, in batches and at N <= 3, else in FP32.  Also the
 // one-time conversion of the FP64 geometric factors (round to nearest even).
 #include <cuda_bf16.h>
 

@@ -77,7 +77,8 @@ struct F32Pad {
 template <int NQ>
 __host__ __device__ constexpr size_t f32_smem(int epb) {
     const size_t b = 3 * size_t(epb) * F32Pad<NQ>::NPP * sizeof(float);
-    return b < 128 ? 128 : b;   // 32 floats of the block sum
+    const size_t sum = size_t((epb * NQ * NQ + 31) / 32 * 32) * sizeof(double);   // block_sum_wide's, a double per thread
+    return b < sum ? sum : b;
 }
 
 // The block's factors towards L2, before its other loads.

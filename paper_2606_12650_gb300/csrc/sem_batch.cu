@@ -225,8 +225,8 @@ __global__ void __maxnreg__((F32Regs<NQ, GT>::value)) batch_f32_kernel(const __g
                                        static_cast<float *>(it.p), static_cast<float *>(it.x), G, P.d, P.dt, it.st,
                                        it.e0, it.ne, P.epb, smem32, &part))
         return;
-    const float s = block_sum_f32(part, smem32);
-    if (threadIdx.x == 0) it.partials[it.b] = double(s);
+    const double s = block_sum_wide(double(part), reinterpret_cast<double *>(smem32));
+    if (threadIdx.x == 0) it.partials[it.b] = s;
 }
 
 __global__ void __launch_bounds__(kPapThreads) batch_pap_kernel(const PapItem *items) {
@@ -726,7 +726,8 @@ __global__ void __launch_bounds__(kBatchThreads, MODE == kVecUpdate32 ? kUpd32Bl
     leave_queue(q);
 }
 
-// The owner-row update of a block order, <r, r> in the vectors' precision.
+// The owner-row update of a block order, <r, r> in the vectors' precision per
+// thread and in FP64 across threads.
 template <int NQ, typename T>
 __global__ void __launch_bounds__(256, kOwnerBlocks)
     batch_owner_kernel(const OwnerItem *items, BatchProb *probs, BatchCtl *ctl, int32_t *finished_ids) {
@@ -737,7 +738,7 @@ __global__ void __launch_bounds__(256, kOwnerBlocks)
     T acc = T(0), unused = T(0);
     owner_tasks<NQ, false, T>(static_cast<T *>(it.r), static_cast<const T *>(it.w), nullptr,
                               8 * it.b + int(threadIdx.x >> 5), 8 * it.nb, it.E, it.bd, T(it.st->alpha), 0, acc, unused);
-    const double bs = owner_block_sum(acc, scratch);
+    const double bs = block_sum_wide(double(acc), scratch);
     double rho_new;
     if (grid_sum(bs, it.partials, it.cap, &it.st->ticket_up, it.b, it.nb, &rho_new) && threadIdx.x == 0) {
         cg_close_iteration(it.st, rho_new);
