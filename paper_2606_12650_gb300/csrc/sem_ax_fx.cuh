@@ -63,10 +63,24 @@ __device__ __forceinline__ int64_t fx_mad(int32_t a, int32_t b, int64_t c) {
     return int64_t((uint64_t(uint32_t(hi)) << 32) | uint32_t(lo));
 }
 
-constexpr int64_t kFxHalf = int64_t(1) << 31;   // rounds the cut of the cross terms
+constexpr int64_t kFxHalf = int64_t(1) << 31;
+// A sum of cross terms is cut at 2^32, rounded.  Halves go upwards, but away from
+// zero at N+1 <= 3, where the coefficients of D are sums of a few powers of two
+// and halves frequent: an error of one sign everywhere comes back from a solve
+// as A^-1 of it.  At other orders full significands meet a half once in 2^32,
+// and away from zero would cost 27 instructions a node (N+1 <= 3: 1 to 3 %).
+template <int NQ>
+struct FxCut {
+    static constexpr int64_t start = NQ <= 3 ? 0 : kFxHalf;   // of the sum
+};
 
 __device__ __forceinline__ int64_t fx_cross(fxl c, fxl u, int64_t x) { return fx_mad(c.l, u.h, fx_mad(c.h, u.l, x)); }
 __device__ __forceinline__ int64_t fx_upper(int64_t x) { return int64_t(int32_t(uint64_t(x) >> 32)); }
+
+template <int NQ>
+__device__ __forceinline__ int64_t fx_cut(int64_t x) {
+    return fx_upper(NQ <= 3 ? x + kFxHalf + (x >> 63) : x);
+}
 
 // y = M u by the even-odd split (the same sums as eo_apply), st(i, y_i).
 template <int NQ, typename Store>
@@ -82,15 +96,15 @@ __device__ __forceinline__ void eo_apply_fx(const int64_t (&u)[NQ], const EoMatF
     if (ODD) um = fx_limbs(u[H]);
 #pragma unroll
     for (int i = 0; i < H; ++i) {
-        int64_t a = kFxHalf, b = kFxHalf;
+        int64_t a = FxCut<NQ>::start, b = a;
 #pragma unroll
         for (int l = 0; l < H; ++l) {
             a = fx_cross(c.e[i * H + l], ue[l], a);
             b = fx_cross(c.o[i * H + l], uo[l], b);
         }
         if (ODD) a = fx_cross(c.m[i], um, a);
-        a = fx_upper(a);
-        b = fx_upper(b);
+        a = fx_cut<NQ>(a);
+        b = fx_cut<NQ>(b);
 #pragma unroll
         for (int l = 0; l < H; ++l) {
             a = fx_mad(c.e[i * H + l].h, ue[l].h, a);
@@ -101,10 +115,10 @@ __device__ __forceinline__ void eo_apply_fx(const int64_t (&u)[NQ], const EoMatF
         st(NQ - 1 - i, b - a);
     }
     if (ODD) {
-        int64_t b = kFxHalf;
+        int64_t b = FxCut<NQ>::start;
 #pragma unroll
         for (int l = 0; l < H; ++l) b = fx_cross(c.o[H * H + l], uo[l], b);
-        b = fx_upper(b);
+        b = fx_cut<NQ>(b);
 #pragma unroll
         for (int l = 0; l < H; ++l) b = fx_mad(c.o[H * H + l].h, uo[l].h, b);
         st(H, b);
@@ -112,8 +126,9 @@ __device__ __forceinline__ void eo_apply_fx(const int64_t (&u)[NQ], const EoMatF
 }
 
 // (a . b) / 2^64 of three terms.
+template <int NQ>
 __device__ __forceinline__ int64_t fx_dot3(fxl a0, fxl a1, fxl a2, fxl b0, fxl b1, fxl b2) {
-    int64_t s = fx_upper(fx_cross(a2, b2, fx_cross(a1, b1, fx_cross(a0, b0, kFxHalf))));
+    int64_t s = fx_cut<NQ>(fx_cross(a2, b2, fx_cross(a1, b1, fx_cross(a0, b0, FxCut<NQ>::start))));
     return fx_mad(a2.h, b2.h, fx_mad(a1.h, b1.h, fx_mad(a0.h, b0.h, s)));
 }
 
@@ -135,6 +150,14 @@ constexpr int kFxEmin = 64;
 __device__ __forceinline__ double fx_pow2(int e) {
     const int f = min(max(e + 1023, 0), 2047);
     return __hiloint2double(f << 20, 0);
+}
+
+// 1.5 2^52 + v 2^(up - 11) rounded, halves away from zero (|v 2^up| < 2^62):
+// A(-x) = -A(x).  Cut instead, or with halves upwards, the error has one sign
+// everywhere, and a solve returns A^-1 of it.
+__device__ __forceinline__ double fx_top(int64_t v, int up) {
+    const int64_t w = int64_t(uint64_t(v) << up);
+    return __longlong_as_double(0x4338000000000000ll + ((w + 1024 + (w >> 63)) >> 11));
 }
 
 // Shared-memory layout of U, V and X: node (i, j, k) of an element at
@@ -360,9 +383,9 @@ __device__ __forceinline__ void lines_group_fx(const double *x, double *y, doubl
             const fxl ur = fx_limbs(SU[pq]), us = fx_limbs(SV[pq]), uv = fx_limbs(ut[k]);
             const fxl rr{g[0].x, g[0].y}, rs{g[0].z, g[0].w}, rt{g[1].x, g[1].y}, ss{g[1].z, g[1].w},
                 s_t{g[2].x, g[2].y}, tt{g[2].z, g[2].w};
-            SU[pq] = fx_dot3(rr, rs, rt, ur, us, uv);
-            SV[pq] = fx_dot3(rs, ss, s_t, ur, us, uv);
-            wt[k] = fx_dot3(rt, s_t, tt, ur, us, uv);
+            SU[pq] = fx_dot3<NQ>(rr, rs, rt, ur, us, uv);
+            SV[pq] = fx_dot3<NQ>(rs, ss, s_t, ur, us, uv);
+            wt[k] = fx_dot3<NQ>(rt, s_t, tt, ur, us, uv);
         }
     }
     __syncthreads();
@@ -384,7 +407,7 @@ __device__ __forceinline__ void lines_group_fx(const double *x, double *y, doubl
     __syncthreads();
 
     // ---- (4) sum of the three directions and <p, y>; y = Y 2^q, shifted up by
-    // the thread's common headroom and cut to 51 bits for FP64 (one FMA)
+    // the thread's common headroom and rounded to 51 bits for FP64 (one FMA)
     const int q = emax - (kFxBits - 53 + 1075) - cd.k - ct.k + 192 - kge;
     int64_t dot = 0;
     if (act) {
@@ -409,7 +432,7 @@ __device__ __forceinline__ void lines_group_fx(const double *x, double *y, doubl
         const double f0 = -0x1.8p52 * f;
 #pragma unroll
         for (int k = 0; k < NQ; ++k)
-            y[nb + k * NQ2] = fma(__longlong_as_double(0x4338000000000000ll + ((yt[k] << up) >> 11)), f, f0);
+            y[nb + k * NQ2] = fma(fx_top(yt[k], up), f, f0);
     }
     if (CG) {
         // the element's sum of X Y / 2^64: per warp by shuffles or as three

@@ -282,9 +282,9 @@ __global__ void __maxnreg__(SmallShape<NQ>::regs) cg_small_kernel(const __grid_c
                     const fxl ur = fx_limbs(q[0]), us = fx_limbs(q[RG]), ut = fx_limbs(q[2 * RG]);
                     const fxl grr{g[0].x, g[0].y}, grs{g[0].z, g[0].w}, grt{g[1].x, g[1].y}, gss{g[1].z, g[1].w},
                         gst{g[2].x, g[2].y}, gtt{g[2].z, g[2].w};
-                    q[0] = fx_dot3(grr, grs, grt, ur, us, ut);
-                    q[RG] = fx_dot3(grs, gss, gst, ur, us, ut);
-                    q[2 * RG] = fx_dot3(grt, gst, gtt, ur, us, ut);
+                    q[0] = fx_dot3<NQ>(grr, grs, grt, ur, us, ut);
+                    q[RG] = fx_dot3<NQ>(grs, gss, gst, ur, us, ut);
+                    q[2 * RG] = fx_dot3<NQ>(grt, gst, gtt, ur, us, ut);
                 }
         }
         __syncthreads();
@@ -320,7 +320,7 @@ __global__ void __maxnreg__(SmallShape<NQ>::regs) cg_small_kernel(const __grid_c
 #pragma unroll
             for (int s = 0; s < KS; ++s)
                 if (d + 3 * s < NQ) {
-                    wv[s] = fma(__longlong_as_double(0x4338000000000000ll + ((Y[s] << up) >> 11)), f, f0);
+                    wv[s] = fma(fx_top(Y[s], up), f, f0);
                     if (sx || sy || sz_of(s)) __stcg(w + l0 + s * NT, wv[s]);
                 }
         }
