@@ -4,16 +4,22 @@
 #include <algorithm>
 
 #include "sem_ax_fx.cuh"
+#include "sem_device.cuh"
 
 namespace sem {
 
 // One block per element: the largest exponent of the element's factors, then
 // g 2^kg rounded to integers, |G| < 2^kFxGBits, in integer arithmetic (FP64
-// conversions run at 1/64 rate).  Bound by HBM: 48 B read and written per
-// node; the second read hits L1 or L2.
+// conversions run at 1/64 rate), with fewer bits where the element's sum of
+// <x, y> could pass 63 (FxBound; elements with vertices moved by up to 0.6 of a
+// side reach 0.39 of the limit, at N = 9).  Bound by HBM: 48 B read and written
+// per node; the later reads hit L1 or L2.
 __global__ void __launch_bounds__(256) geometry_fx_kernel(const double *__restrict__ G, int4 *__restrict__ out,
-                                                          int32_t *__restrict__ kg, int np, int64_t E) {
+                                                          int32_t *__restrict__ kg, int nq, int64_t E, FxBound B) {
     __shared__ uint32_t s_max;
+    __shared__ float s_sum[32];
+    __shared__ int s_less;
+    const int np = nq * nq * nq;
     for (int64_t e = blockIdx.x; e < E; e += gridDim.x) {
         __syncthreads();
         if (threadIdx.x == 0) s_max = uint32_t(kFxEmin) << 20;
@@ -27,7 +33,30 @@ __global__ void __launch_bounds__(256) geometry_fx_kernel(const double *__restri
         mx = __reduce_max_sync(0xffffffffu, mx);
         if ((threadIdx.x & 31) == 0) atomicMax(&s_max, mx);
         __syncthreads();
-        const int emax = int(s_max >> 20);
+        int emax = int(s_max >> 20);
+        // |g| of the largest exponent in [1, 2), to 20 bits
+        auto rel = [emax](double d) {
+            const int h = __double2hiint(d) & 0x7fffffff;
+            return (h >> 20) - emax + 127 > 0 ? __int_as_float((h - ((emax - 127) << 20)) << 3) : 0.f;
+        };
+        float sum = 0.f;
+        for (int node = threadIdx.x; node < np; node += blockDim.x) {
+            const double2 a = __ldg(g + 3 * node), b = __ldg(g + 3 * node + 1), c = __ldg(g + 3 * node + 2);
+            const float r = B.rows[node % nq], s = B.rows[node / nq % nq], t = B.rows[node / nq / nq];
+            sum += r * r * rel(a.x) + s * s * rel(b.y) + t * t * rel(c.y) +
+                   2.f * (r * s * rel(a.y) + r * t * rel(b.x) + s * t * rel(c.x));
+        }
+        sum = block_sum_f32(sum, s_sum);
+        if (threadIdx.x == 0) {
+            int less = 0;
+            while (sum > B.limit && less < 8) {
+                sum *= 0.5f;
+                ++less;
+            }
+            s_less = less;
+        }
+        __syncthreads();
+        emax += s_less;
         if (threadIdx.x == 0) kg[e] = kFxGBits - 53 + 1075 - emax;
         auto fix = [emax](double d) {
             const int64_t bits = __double_as_longlong(d);
@@ -60,7 +89,10 @@ int fx_prepare(Problem *P) {
     int rc = g && kg ? SEM_OK : SEM_ENOMEM;
     if (rc == SEM_OK) {
         const unsigned blocks = unsigned(std::min<int64_t>(P->E, int64_t(sm_count()) * 32));
-        geometry_fx_kernel<<<blocks, 256, 0, stream()>>>(P->G, g, kg, int(P->np), P->E);
+        FxConsts c;
+        fx_coefficients(P->oc.D, P->nq, &c.d, &c.dt);
+        geometry_fx_kernel<<<blocks, 256, 0, stream()>>>(P->G, g, kg, P->nq, P->E,
+                                                         fx_bound(P->oc.D, P->nq, c.d.k, c.dt.k));
         count_launches(1);
         rc = cuda_check(cudaGetLastError(), "geometry_fx_kernel");
     }

@@ -423,6 +423,10 @@ __device__ __forceinline__ void lines_group_fx(const double *x, double *y, doubl
                 const fxl yl = fx_limbs(yt[k]), xl = fx_limbs(SX[pq]);
                 acc = fx_cross(xl, yl, acc);
                 dot = fx_mad(xl.h, yl.h, dot);
+                if (NQ == 10 && k == 4) {   // ten nodes' cross terms could pass 2^63
+                    dot += fx_upper(acc);
+                    acc = kFxHalf;
+                }
             }
         }
         dot += fx_upper(acc);
@@ -570,6 +574,25 @@ inline EoMatFX eo_coefficients_fx(const double *M, int nq, double ubound, double
 struct FxConsts {
     EoMatFX d, dt;
 };
+
+// What bounds an element's sum of |X Y| / 2^64: with |X| < 2^60, the row sums
+// rows[i] of |D| and G = g 2^61 (|g| < 2),
+//   2^(k + kt - 75) S,  S = sum over nodes and a, b of rows_a |g_ab| rows_b.
+struct FxBound {
+    float rows[kMaxQ];
+    float limit;      // of S, for a sum below 2^62
+};
+
+inline FxBound fx_bound(const double *D, int nq, int k, int kt) {
+    FxBound b{};
+    for (int i = 0; i < nq; ++i) {
+        double s = 0.0;
+        for (int l = 0; l < nq; ++l) s += std::fabs(D[i * nq + l]);
+        b.rows[i] = float(s);
+    }
+    b.limit = float(std::ldexp(0.99, 62 + 75 - k - kt));
+    return b;
+}
 
 // Host: both matrices of an order.  |X| < 2^kFxBits, |W| <= 3 2^kFxGBits |D X|.
 inline void fx_coefficients(const double *D, int nq, EoMatFX *d, EoMatFX *dt) {
