@@ -14,8 +14,20 @@
 // the sum of ch uh; cl ul (2^-64 of full scale) is dropped.  Sums of values
 // are exact.  The scales of D, of the factors (one exponent per element, kept
 // beside them) and of D^T keep every sum below 2^63 for any input
-// (fx_coefficients); the typical |y| is ~2^51, where the dropped parts are
-// ~1e-15 of max|y| (the FP64 direct evaluation: ~2e-16).
+// (fx_coefficients, FxBound).
+//
+// Every rounding is absolute on the element's scale: together they are below
+// 2^-50 of the largest |y| that the element's max |x| and max |G| allow.
+// Relative to max |y| itself that depends on how much of those sums cancels.
+// Largest error of an element over its max |y|, boxes with sides 1:1:1 to
+// 1:30:1000 (the direct FP64 evaluation / pairs of FP32 numbers):
+//   random x                  4e-16 at N = 1 .. 4e-15 at N = 9 (2e-16 .. 3e-15 / 1e-14 .. 5e-14)
+//   sines over 8 and 32
+//   elements a side           N = 3 1e-14, N = 5 1e-13, N = 7 3e-13, N = 9 6e-13
+//                             (1e-14, 1e-14, 4e-14, 2e-13 / 4e-13, 2e-12, 4e-12, 7e-12)
+//   1 + 1e-6 random           N = 3 3e-10, N = 9 1e-9 (1e-10, 6e-10 / 2e-8, 2e-8)
+//   random times 2^-40 .. 1
+//   within an element         N = 3 4e-15, N = 9 7e-15 (6e-16, 3e-15 / 2e-14, 2e-14)
 //
 // Why integers: GB300 runs FP64 at 1/64 of its FP32 rate (DFMA line kernel:
 // 1580 us at E = 32^3, N = 7), but a 32 x 32 + 64-bit multiply-add
