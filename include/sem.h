@@ -202,6 +202,10 @@ int sem_update(void *host, size_t start, size_t end, size_t elem_size, int op);
  *               the wait ran out (-1 otherwise).  The next sem_sync or solve
  *               returns SEM_ETIMEDOUT (the message names the wait) and clears
  *               the word; nothing is left in flight and later calls work.
+ *   "exchange_probe" limit_ns (1e3 .. 1e8)
+ *               The same for the exchange between the blocks of a one-kernel
+ *               solve: 40 blocks wait for a 41st that does not exist, each for
+ *               ~limit_ns (group leaders twice that).
  *   "peak_fma"  dtype (0 f64, 1 f32), iters, OUT flops_per_s
  *               measured FMA issue rate of the FP64 or FP32 pipe (device fact
  *               for the ALU roofline; not part of the method)

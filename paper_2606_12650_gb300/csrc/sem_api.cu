@@ -224,7 +224,8 @@ int poll_status() {
         snprintf(buf, sizeof buf,
                  "a bounded device wait gave up (status %d: %s)", code,
                  code == kStatusMbarTimeout ? "an mbarrier wait for a TMA copy into shared memory ran past its limit"
-                                            : "unknown wait");
+                 : code == kStatusExchangeTimeout ? "an exchange between the blocks of a solve ran past its limit"
+                                                  : "unknown wait");
         return set_error(SEM_ETIMEDOUT, buf);
     }
     return SEM_OK;
@@ -985,6 +986,14 @@ int run_wait_probe(ArgReader &R) {
     return probe_wait_timeout(uint64_t(limit), out);
 }
 
+int run_exchange_probe(ArgReader &R) {
+    if (!R.need(1)) return R.err;
+    const int64_t limit = R.i(0, "limit_ns");
+    if (R.err) return R.err;
+    if (limit < 0) return R.fail(SEM_EARG, "limit_ns must be positive");
+    return probe_exchange_timeout(uint64_t(limit));
+}
+
 int run_peak_fma(ArgReader &R) {
     if (!R.need(3)) return R.err;
     const int64_t dtype = R.i(0, "dtype"), iters = R.i(1, "iters");
@@ -1205,6 +1214,7 @@ int sem_run(const char *kernel, int nargs, const sem_arg *args) {
     else if (k == "serve_close") rc = run_serve_close(R);
     else if (k == "peak_fma") rc = run_peak_fma(R);
     else if (k == "wait_probe") rc = run_wait_probe(R);
+    else if (k == "exchange_probe") rc = run_exchange_probe(R);
     else if (k == "dist_mesh") rc = run_dist_mesh(R);
     else if (k == "dist_info") rc = run_dist_info(R);
     else if (k == "dist_ax") rc = run_dist_ax(R);

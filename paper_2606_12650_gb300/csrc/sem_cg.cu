@@ -437,7 +437,7 @@ int cg_solve(Problem *P, const double *b, double *x, double tol, int maxit, doub
     }
     if (rc == SEM_OK && !steps) rc = prepare_f64_variant(P);
     if (rc == SEM_OK) rc = launch_cg_init(P, b, maxit, tol, hist, steps);
-    const bool small = rc == SEM_OK && !steps && small_fits(P, false);
+    bool small = rc == SEM_OK && !steps && small_fits(P, false);
     if (rc == SEM_OK && !small) rc = capture_graph(P, steps);
     if (rc != SEM_OK) return rc;
     // at most maxit iterations are left to run; the flag stops earlier replays
@@ -446,7 +446,13 @@ int cg_solve(Problem *P, const double *b, double *x, double tol, int maxit, doub
     while (left > 0) {
         const int64_t K = small ? 1 : P->graph_iters;
         if (small) {
-            rc = launch_small(P, false);
+            bool refused = false;
+            rc = launch_small(P, false, &refused);
+            if (rc == SEM_OK && refused) {   // by the first launch, nothing has run
+                small = false;
+                rc = capture_graph(P, false);
+                if (rc == SEM_OK) continue;
+            }
         } else {
             rc = cuda_check(cudaGraphLaunch(steps ? P->graph_steps : P->graph, stream()), "cg: graph launch");
             if (rc == SEM_OK) count_launches(2 * K);

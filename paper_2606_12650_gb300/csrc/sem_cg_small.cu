@@ -55,6 +55,7 @@ struct SmallArgs {
     CgState *st;
     uint64_t *slots;        // zero at the launch: 2 words per block and group, then 2 or 4
     int32_t *status;
+    uint64_t limit_ns;      // of a wait
 };
 
 template <int NQ>
@@ -84,7 +85,8 @@ constexpr uint64_t kExchangeLimitNs = 4000000000ull;
 // before is then visible after the block's next barrier.  false: the wait ran
 // out.
 template <int NV, bool FENCE>
-__device__ __forceinline__ bool get_share(const uint64_t *slots, int n, uint32_t epoch, double (&sum)[NV]) {
+__device__ __forceinline__ bool get_share(const uint64_t *slots, int n, uint32_t epoch, double (&sum)[NV],
+                                          uint64_t limit_ns) {
 #pragma unroll
     for (int c = 0; c < NV; ++c) sum[c] = 0.0;
     for (int q = threadIdx.x; q < n; q += blockDim.x) {
@@ -100,7 +102,7 @@ __device__ __forceinline__ bool get_share(const uint64_t *slots, int n, uint32_t
             if (all) break;
             if (it == 0) {
                 t0 = global_ns();
-            } else if ((it & 63u) == 0 && global_ns() - t0 > kExchangeLimitNs) {
+            } else if ((it & 63u) == 0 && global_ns() - t0 > limit_ns) {
                 return false;
             }
         }
@@ -120,20 +122,20 @@ __device__ __forceinline__ bool get_share(const uint64_t *slots, int n, uint32_t
 constexpr int kDirect = 32;
 template <int NV, bool FENCE>
 __device__ __forceinline__ bool exchange(uint64_t *slots, int nb, int e, uint32_t epoch, const double (&mine)[NV],
-                                         double (&share)[NV], int *n) {
+                                         double (&share)[NV], int *n, uint64_t limit_ns) {
     if (threadIdx.x == 0) {
         if (FENCE) __threadfence();   // the block's writes and reads of w before its slot
 #pragma unroll
         for (int c = 0; c < NV; ++c) put_value(slots + 2 * (size_t(NV) * e + c), mine[c], epoch);
     }
     *n = nb;
-    if (nb <= kDirect) return get_share<NV, FENCE>(slots, nb, epoch, share);
+    if (nb <= kDirect) return get_share<NV, FENCE>(slots, nb, epoch, share, limit_ns);
     uint64_t *groups = slots + size_t(2 * NV) * nb;
     *n = (nb + 31) / 32;
     bool ok = true;
     if (e % 32 == 0 && threadIdx.x < 32) {
         double v[NV];
-        ok = get_share<NV, FENCE>(slots + size_t(2 * NV) * e, min(32, nb - e), epoch, v);
+        ok = get_share<NV, FENCE>(slots + size_t(2 * NV) * e, min(32, nb - e), epoch, v, limit_ns);
         ok = __all_sync(0xffffffffu, ok);
         // orders every lane's reads (and fence) before lane 0's store below: votes
         // and shuffles do not order memory between lanes
@@ -149,7 +151,7 @@ __device__ __forceinline__ bool exchange(uint64_t *slots, int nb, int e, uint32_
             for (int c = 0; c < NV; ++c) put_value(groups + 2 * (size_t(NV) * (e / 32) + c), v[c], epoch);
         }
     }
-    return get_share<NV, FENCE>(groups, *n, epoch, share) && ok;
+    return get_share<NV, FENCE>(groups, *n, epoch, share, limit_ns) && ok;
 }
 
 // Sum of v over the first n threads, in warp 0 (all lanes take part, the
@@ -342,10 +344,10 @@ __global__ void __maxnreg__(SmallShape<NQ>::regs) cg_small_kernel(const __grid_c
         // ---- first exchange: every block's part, and its w
         double share1[1];
         int ns;
-        const bool ok1 = exchange<1, true>(slots1, nb, e, uint32_t(n), part, share1, &ns);
+        const bool ok1 = exchange<1, true>(slots1, nb, e, uint32_t(n), part, share1, &ns, A.limit_ns);
         s_red[0][tid] = share1[0];
         if (__syncthreads_or(!ok1)) {
-            if (tid == 0) atomicExch(A.status, int32_t(kStatusMbarTimeout));
+            if (tid == 0) atomicExch(A.status, int32_t(kStatusExchangeTimeout));
             return;
         }
         double c[KS];
@@ -414,12 +416,12 @@ __global__ void __maxnreg__(SmallShape<NQ>::regs) cg_small_kernel(const __grid_c
             for (int s = 0; s < KS; ++s) x[s] = fma(alpha, p[s], x[s]);
         }
         double share2[NV2];
-        const bool ok2 = exchange<NV2, false>(slots2, nb, e, uint32_t(n), mine, share2, &ns);
+        const bool ok2 = exchange<NV2, false>(slots2, nb, e, uint32_t(n), mine, share2, &ns, A.limit_ns);
         __syncthreads();       // warp 0 has read s_red
 #pragma unroll
         for (int v = 0; v < NV2; ++v) s_red[v][tid] = share2[v];
         if (__syncthreads_or(!ok2)) {
-            if (tid == 0) atomicExch(A.status, int32_t(kStatusMbarTimeout));
+            if (tid == 0) atomicExch(A.status, int32_t(kStatusExchangeTimeout));
             return;
         }
         if (warp == 0) {
@@ -447,8 +449,8 @@ __global__ void __maxnreg__(SmallShape<NQ>::regs) cg_small_kernel(const __grid_c
     const double none[1] = {0.0};
     double share[1];
     int ns;
-    if (__syncthreads_or(!exchange<1, true>(slots1, nb, e, uint32_t(n + 1), none, share, &ns))) {
-        if (tid == 0) atomicExch(A.status, int32_t(kStatusMbarTimeout));
+    if (__syncthreads_or(!exchange<1, true>(slots1, nb, e, uint32_t(n + 1), none, share, &ns, A.limit_ns))) {
+        if (tid == 0) atomicExch(A.status, int32_t(kStatusExchangeTimeout));
         return;
     }
     if (act) {
@@ -494,7 +496,7 @@ int small_capacity_nq(int *out) {
 }
 
 template <int NQ, bool PRE>
-int launch_small_nq(const Problem *P, const SmallArgs &A) {
+int launch_small_nq(const Problem *P, const SmallArgs &A, bool *refused) {
     using S = SmallShape<NQ>;
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeCooperative;
@@ -506,19 +508,35 @@ int launch_small_nq(const Problem *P, const SmallArgs &A) {
     cfg.stream = stream();
     cfg.attrs = &at;
     cfg.numAttrs = 1;
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, cg_small_kernel<NQ, PRE>, A);
+    if (err == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        *refused = true;
+        return SEM_OK;
+    }
     count_launches(1);
-    return cuda_check(cudaLaunchKernelEx(&cfg, cg_small_kernel<NQ, PRE>, A), "cg_small_kernel");
+    return cuda_check(err, "cg_small_kernel");
 }
 
 template <bool PRE>
-int small_call(const Problem *P, const SmallArgs *A, int *capacity) {
+int small_call(const Problem *P, const SmallArgs *A, bool *refused, int *capacity = nullptr) {
     switch (P->nq) {
 #define SEM_SMALL(Q) \
-    case Q: return A ? launch_small_nq<Q, PRE>(P, *A) : small_capacity_nq<Q, PRE>(capacity);
+    case Q: return A ? launch_small_nq<Q, PRE>(P, *A, refused) : small_capacity_nq<Q, PRE>(capacity);
         SEM_SMALL(2) SEM_SMALL(3) SEM_SMALL(4) SEM_SMALL(5) SEM_SMALL(6) SEM_SMALL(7) SEM_SMALL(8) SEM_SMALL(9) SEM_SMALL(10)
 #undef SEM_SMALL
         default: return set_error(SEM_EARG, "cg: unsupported order");
     }
+}
+
+// Self-test of the exchange's bounded wait: gridDim.x blocks take part in an
+// exchange of one more, whose slot nobody fills.
+__global__ void exchange_probe_kernel(uint64_t *slots, int32_t *status, uint64_t limit_ns) {
+    const double mine[1] = {1.0};
+    double share[1];
+    int n;
+    const bool ok = exchange<1, true>(slots, int(gridDim.x) + 1, int(blockIdx.x), 1u, mine, share, &n, limit_ns);
+    if (__syncthreads_or(!ok) && threadIdx.x == 0) atomicExch(status, int32_t(kStatusExchangeTimeout));
 }
 
 }  // namespace
@@ -534,13 +552,14 @@ int small_call(const Problem *P, const SmallArgs *A, int *capacity) {
 bool small_fits(const Problem *P, bool pre) {
     if (tune_get(kTuneF64, P->nq).variant != kAxLinesFX) return false;
     int capacity = 0;
-    const int rc = pre ? small_call<true>(P, nullptr, &capacity) : small_call<false>(P, nullptr, &capacity);
+    const int rc = pre ? small_call<true>(P, nullptr, nullptr, &capacity) : small_call<false>(P, nullptr, nullptr, &capacity);
     return rc == SEM_OK && P->E <= std::min<int64_t>(capacity, 5 * int64_t(sm_count()));
 }
 
 // One launch: up to kSmallIters iterations from P's state, x complete at its
-// end (nothing deferred).
-int launch_small(const Problem *P, bool pre) {
+// end (nothing deferred).  *refused: the launch's blocks cannot all be resident
+// (fewer SMs than the device has, say), nothing ran.
+int launch_small(const Problem *P, bool pre, bool *refused) {
     SmallArgs A{};
     A.x = P->x;
     A.r = P->r;
@@ -558,11 +577,42 @@ int launch_small(const Problem *P, bool pre) {
     A.st = P->st;
     A.slots = reinterpret_cast<uint64_t *>(P->partials);
     A.status = status_word();
+    A.limit_ns = kExchangeLimitNs;
     const int64_t words = 6 * (P->E + (P->E + 31) / 32);
     if (words > P->partials_cap) return set_error(SEM_ERANGE, "cg: more blocks than reduction slots");
     const int rc = cuda_check(cudaMemsetAsync(A.slots, 0, sizeof(uint64_t) * size_t(words), stream()), "cg: slots");
     if (rc != SEM_OK) return rc;
-    return pre ? small_call<true>(P, &A, nullptr) : small_call<false>(P, &A, nullptr);
+    *refused = false;
+    return pre ? small_call<true>(P, &A, refused) : small_call<false>(P, &A, refused);
+}
+
+// Runs the exchange of 41 blocks with 40 of them (two groups, so that the
+// leader's wait and the others' both run out, each after ~limit_ns).
+int probe_exchange_timeout(uint64_t limit_ns) {
+    if (limit_ns < 1000 || limit_ns > 100000000ull)
+        return set_error(SEM_EARG, "exchange_probe: limit_ns must be in [1e3, 1e8]");
+    constexpr unsigned kBlocks = 40;
+    constexpr size_t kBytes = sizeof(uint64_t) * 2 * (kBlocks + 1 + 2);   // slots of the blocks and of two groups
+    uint64_t *slots = static_cast<uint64_t *>(dev_alloc(kBytes));
+    if (!slots) return SEM_ENOMEM;
+    int rc = cuda_check(cudaMemsetAsync(slots, 0, kBytes, stream()), "exchange_probe: slots");
+    if (rc == SEM_OK) {
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeCooperative;
+        at.val.cooperative = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(kBlocks);
+        cfg.blockDim = dim3(64);
+        cfg.stream = stream();
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        count_launches(1);
+        rc = cuda_check(cudaLaunchKernelEx(&cfg, exchange_probe_kernel, slots, status_word(), limit_ns),
+                        "exchange_probe_kernel");
+    }
+    if (rc == SEM_OK) rc = cuda_check(cudaStreamSynchronize(stream()), "exchange_probe: sync");
+    dev_free(slots);
+    return rc;
 }
 
 }  // namespace sem

@@ -78,6 +78,7 @@ constexpr int32_t kDoneOutOfRange = 2;
 enum DeviceStatus : int32_t {
     kStatusOk = 0,
     kStatusMbarTimeout = 1,
+    kStatusExchangeTimeout = 2,
 };
 
 struct Problem {
@@ -280,7 +281,7 @@ int cg_solve(Problem *P, const double *b, double *x, double tol, int maxit, doub
              int64_t *iters, double *rel_res);
 // whole solves of small problems in one kernel (sem_cg_small.cu)
 bool small_fits(const Problem *P, bool pre);
-int launch_small(const Problem *P, bool pre);
+int launch_small(const Problem *P, bool pre, bool *refused);
 int launch_ax_pcg(const Problem *P);         // p = dinv r + beta p; w = A_local p; <p,w>
 int jacobi_prepare(Problem *P);              // dinv = 1 / (mask(QQ^T diag(A_local)))
 int pcg_solve(Problem *P, const double *b, double *x, double tol, int maxit, double *hist,
@@ -331,5 +332,6 @@ int dist_cg_solve(DistProblem *D, const double *b, double *x, double tol, int ma
 int probe_fma_rate(int dtype, int iters, double *flops_per_s);   // dtype 0: f64, 1: f32
 // failure-detection self-test: a bounded mbarrier wait that runs out (status word set)
 int probe_wait_timeout(uint64_t limit_ns, double *copied_value);
+int probe_exchange_timeout(uint64_t limit_ns);   // sem_cg_small.cu
 
 }  // namespace sem

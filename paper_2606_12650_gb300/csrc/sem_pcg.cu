@@ -200,14 +200,19 @@ int pcg_solve(Problem *P, const double *b, double *x, double tol, int maxit, dou
     count_launches(1);
     rc = cuda_check(cudaGetLastError(), "pcg_init_kernel");
     if (rc == SEM_OK) rc = prepare_f64_variant(P);
-    const bool small = rc == SEM_OK && small_fits(P, true);
+    bool small = rc == SEM_OK && small_fits(P, true);
     if (rc == SEM_OK && !small) rc = capture_pcg(P);
     if (rc != SEM_OK) return rc;
-    const int64_t K = small ? 1 : P->graph_iters;
-    const int64_t max_replays = (int64_t(maxit) + K - 1) / K;
-    for (int64_t rep = 0; rep < max_replays; ++rep) {
+    for (int64_t left = maxit; left > 0;) {
+        const int64_t K = small ? 1 : P->graph_iters;
         if (small) {
-            rc = launch_small(P, true);
+            bool refused = false;
+            rc = launch_small(P, true, &refused);
+            if (rc == SEM_OK && refused) {   // by the first launch, nothing has run
+                small = false;
+                rc = capture_pcg(P);
+                if (rc == SEM_OK) continue;
+            }
         } else {
             rc = cuda_check(cudaGraphLaunch(P->graph_pcg, stream()), "pcg: graph launch");
             if (rc == SEM_OK) count_launches(2 * K);
@@ -221,6 +226,7 @@ int pcg_solve(Problem *P, const double *b, double *x, double tol, int maxit, dou
         if (rc == SEM_OK) rc = cuda_check(cudaStreamSynchronize(stream()), "pcg: sync");
         if (rc != SEM_OK) return rc;
         if (*status_host() != 0 || P->st_host->done) break;
+        left -= K;
     }
     // the last iteration's deferred x += alpha p
     rc = small ? cuda_check(cudaMemcpyAsync(x, P->x, sizeof(double) * P->nL, cudaMemcpyDeviceToDevice, stream()),
