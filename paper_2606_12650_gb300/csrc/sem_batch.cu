@@ -300,7 +300,6 @@ struct Batch {
     // valid while the buffers stay in place and the grids stay the same
     // (membership changes only rewrite the lists' contents and counts)
     const void *graph_bufs[kGraphBufs] = {};
-    int graph_items[2] = {0, 0};    // power-of-two ceilings of the item counts at capture
     int ord_ranges[4 * kOrders];    // host copy of the device per-order ranges (operator, vector)
     int graph_blk[kOrders][3] = {};   // the block orders' grids at capture
     int graph_ord[3 * kOrders] = {};  // per order: the captured launches' grid ceilings and body (0: none)
@@ -1609,8 +1608,6 @@ static int capture(Batch *B) {
     if (rc == SEM_OK) {
         B->graph_stream = stream();
         graph_buffers(B, B->graph_bufs);
-        B->graph_items[0] = items_grid(1 << 30, B->n_ax);
-        B->graph_items[1] = items_grid(1 << 30, B->n_vec);
         order_signature(B, B->graph_ord);
         std::copy(&B->blk_grid[0][0], &B->blk_grid[0][0] + 3 * kOrders, &B->graph_blk[0][0]);
     }

@@ -111,16 +111,11 @@ __global__ void mixed_correct_kernel(double *__restrict__ x, const float *__rest
 }
 
 static int launch_update32(const Problem *P, int gprec) {
-    if (!f32_defers(P->nq, gprec)) switch (P->nq) {
-            case 2: return launch_update_nodes<2>(P);
+    if (!f32_defers(P->nq, gprec)) switch (P->nq) {   // the orders that it names
             case 3: return launch_update_nodes<3>(P);
             case 4: return launch_update_nodes<4>(P);
-            case 5: return launch_update_nodes<5>(P);
             case 6: return launch_update_nodes<6>(P);
-            case 7: return launch_update_nodes<7>(P);
-            case 8: return launch_update_nodes<8>(P);
-            case 9: return launch_update_nodes<9>(P);
-            case 10: return launch_update_nodes<10>(P);
+            default: return set_error(SEM_EARG, "mixed: no node-wise update for this order");
         }
     return launch_update_rows<float>(P, P->r32, P->w32, P->st_in);
 }

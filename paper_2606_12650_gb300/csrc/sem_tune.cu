@@ -33,8 +33,8 @@ uint64_t g_epoch = 1;
 // 10 launches per candidate), as {variant, elements per block} indexed by
 // N + 1 (entries 0 and 1 unused); the run-time tuner replaces entries for
 // the problems at hand.  FP64: the fixed-point line kernel at every order
-// (e.g. N = 3: 281 us against 1203 us for the DFMA line kernel; N = 7: 371
-// against 1579; N = 9: 576 against 2117).  FP32: the direct-load kernel at
+// (e.g. N = 3: 252 us against 1203 us for the DFMA line kernel; N = 7: 277
+// against 1579; N = 9: 399 against 2117).  FP32: the direct-load kernel at
 // every order but N = 2 with FP32 factors (f32_defers), with the elements per
 // block that were best at that size; with
 // the step of d included the TMA-staged and persistent kernels take 130 (N =
