@@ -129,7 +129,11 @@ int prepare_ax32(const Problem *Pb) {
 
 int launch_ax32(const Problem *Pb, const float *x, float *y, int gprec) {
     const TuneChoice c = tune_get(tune_kind_of_gprec(gprec), Pb->nq);
-    if (c.variant == kAxLines || c.variant == kAxLinesPrefetch || c.variant == kAxLinesStaged)
+    // the plain product at N = 1 with FP32 factors, large: the persistent kernel
+    // (1.7e7 nodes 90 us against 94, 2e6 14.4 against 11.9; the table's choice is
+    // the CG operator's)
+    const bool persistent = Pb->nq == 2 && gprec == kGF32 && c.variant == kAxLines && Pb->nL >= (1 << 23);
+    if (!persistent && (c.variant == kAxLines || c.variant == kAxLinesPrefetch || c.variant == kAxLinesStaged))
         return launch_lines32(Pb, x, y, gprec, false, c.epb, c.variant == kAxLinesStaged);
     if (gprec == kGF32) {
         AxArgs<float, float> a = ax_args<float, float>(Pb, static_cast<const float *>(Pb->G32), Pb->partials, Pb->st_in);

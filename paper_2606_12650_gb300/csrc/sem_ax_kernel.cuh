@@ -51,8 +51,8 @@ struct AxArgs {
     T *xs;              // CG: solution, updated x += alpha p_old before p is replaced
                         // (the previous iteration's x update, deferred); nullptr: none
     int64_t E;
-    int64_t cap;        // slots of `partials`
     T D[kMaxQ * kMaxQ];
+    int64_t cap;        // slots of `partials`
 };
 
 __device__ __forceinline__ void load_g6(const double *G, int64_t node, double (&g)[6]) {

@@ -203,25 +203,35 @@ __global__ void gs_lists_kernel(double *__restrict__ u, const int32_t *__restric
     for (int32_t q = b0; q < b1; ++q) u[idx[q]] = s;
 }
 
-// N = 1 and 2 alone and without the mask from the lists (where they exist): most
-// of their nodes are corners and edges, whose copies the box form enumerates
-// with more address arithmetic than the lists take to read (1.7e7 nodes, N = 1:
-// 117 us against 146, 1e6 nodes 11.3 / 13.7; N = 2 14.5 / 15.9; from N = 3 on
-// the box form is equal or faster, e.g. N = 7 66 / 52 us).
+// N = 1 and 2 without the mask from the lists (where they exist) unless small:
+// most of their nodes are corners and edges, whose copies the box form enumerates
+// with more address arithmetic than the lists take to read (lists / box form, us:
+// N = 1 1.7e7 nodes 115 / 145, 6e5 8.3 / 9.4, 2e5 6.2 / 5.7, 2e4 6.1 / 4.2; N = 2
+// 6e5 10.6 / 13.2, 2e5 6.5 / 8.0, 2e4 6.1 / 4.7; from N = 3 on the box form is
+// equal or faster, e.g. N = 7 66 / 52).
 int launch_gs(const Problem *P, double *u) {
-    if (P->nq > 3 || !P->maps_ready) return launch_gs_any(P, u, false);
+    const bool lists = P->maps_ready && ((P->nq == 2 && P->nL >= 300000) || (P->nq == 3 && P->nL >= 100000));
+    if (!lists) return launch_gs_any(P, u, false);
     if (P->n_sh == 0) return SEM_OK;
     gs_lists_kernel<<<grid_for(P->n_sh, kThreads), kThreads, 0, stream()>>>(u, P->sh_ptr, P->sh_idx, P->n_sh);
     count_launches(1);
     return cuda_check(cudaGetLastError(), "gs_lists_kernel");
 }
-int launch_gs_mask(const Problem *P, double *u) { return launch_gs_any(P, u, true); }
 
 int launch_mask(const Problem *P, double *u) {
     if (P->n_mask == 0) return SEM_OK;
     mask_kernel<<<grid_for(P->n_mask, kThreads), kThreads, 0, stream()>>>(u, P->msk_idx, P->n_mask);
     count_launches(1);
     return cuda_check(cudaGetLastError(), "mask_kernel");
+}
+
+// mask(QQ^T u).  One pass of the box form, but at N = 1 from 6e6 nodes on the two
+// lists (right-hand side of 1.7e7 nodes 218 -> 193 us, assembled operator 346 ->
+// 320; 6e6 78.5 -> 76.6, 2e6 26 -> 29).
+int launch_gs_mask(const Problem *P, double *u) {
+    if (P->nq != 2 || !P->maps_ready || P->nL < 6000000) return launch_gs_any(P, u, true);
+    const int rc = launch_gs(P, u);
+    return rc != SEM_OK ? rc : launch_mask(P, u);
 }
 
 // ---------------------------------------------------------------- weighted dot
