@@ -162,6 +162,10 @@ int sem_update(void *host, size_t start, size_t end, size_t elem_size, int op);
  *               sqrt(rho_k/rho_0) <= tol or maxit iterations (tol <= 0: exactly
  *               maxit).  rho = <r,r>_c.  hist (maxit+1 doubles, optional)
  *               receives sqrt(rho_k).  rel_res = sqrt(rho/rho_0) at exit.
+ *               With tol <= 0 the iterate depends on rounding, so that these
+ *               solves keep one arithmetic (pairs of FP32 numbers in the
+ *               operator) where the operator table names variant 5; others
+ *               take the table's operator.
  *   "true_res"  handle, b, x, OUT d     ||b - A x||_c / ||b||_c (FP64)
  *   "pcg_solve" handle, b, x, tol, maxit, OUT iters, OUT rel_res, [hist]
  *               Jacobi-preconditioned CG (the original Nekbone method,

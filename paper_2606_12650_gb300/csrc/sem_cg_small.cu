@@ -1,6 +1,6 @@
-// sem_cg_small.cu -- FP64 CG and Jacobi-PCG of problems whose elements all fit
-// the GPU at once: one cooperative kernel runs the whole solve, a block per
-// element.  An iteration of CG, graph of two launches -> this kernel, in us: N
+// sem_cg_small.cu -- FP64 CG to a tolerance and Jacobi-PCG of problems whose
+// elements all fit the GPU at once: one cooperative kernel runs the whole solve,
+// a block per element.  An iteration of CG, graph of two launches -> this kernel, in us: N
 // = 7: E = 64 17.4 -> 13.0, 150 19.7 -> 14.1, 448 22.8 -> 19.6; N = 5: 384
 // 20.1 -> 14.3; N = 9: 64 21.5 -> 16.8; N = 3: 343 15.2 -> 11.9.
 //
@@ -23,7 +23,8 @@
 // next writes to it by the fences of the exchange in between, and only the
 // exchange after w needs fences.  The waits are bounded (status word); the
 // cooperative launch makes all blocks resident, and a launch runs a bounded
-// number of iterations.
+// number of iterations.  It starts when all its blocks fit, so such a solve waits
+// for other streams' kernels to leave room instead of running beside them.
 //
 // Threads.  Three per (a, b) of an element, one for each direction: thread (d,
 // a, b) takes the line (a, b) of direction d in the contractions, and the
