@@ -29,7 +29,8 @@ int dw_prepare(Problem *P) {
     float *g = static_cast<float *>(dev_alloc(bytes));
     if (!g && P->Gfx) {   // both forms do not fit: the other one is made again when it is needed
         cudaStreamSynchronize(stream());
-        problem_drop_graphs(P);
+        problem_drop_graph(&P->graph);
+        problem_drop_graph(&P->graph_pcg);
         fx_release(P);
         g = static_cast<float *>(dev_alloc(bytes));
     }

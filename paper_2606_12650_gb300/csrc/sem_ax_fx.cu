@@ -81,7 +81,7 @@ int fx_prepare(Problem *P) {
     int4 *g = static_cast<int4 *>(dev_alloc(sizeof(int4) * 3 * size_t(P->nL)));
     if (!g && P->Gdw) {   // both forms do not fit: the other one is made again when it is needed
         cudaStreamSynchronize(stream());
-        problem_drop_graphs(P);
+        problem_drop_graph(&P->graph_steps);
         dw_release(P);
         g = static_cast<int4 *>(dev_alloc(sizeof(int4) * 3 * size_t(P->nL)));
     }

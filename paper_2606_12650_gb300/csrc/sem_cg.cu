@@ -432,10 +432,8 @@ int cg_solve(Problem *P, const double *b, double *x, double tol, int maxit, doub
              int64_t *iters, double *rel_res) {
     if (maxit < 0) return set_error(SEM_EARG, "cg_solve: maxit must be >= 0");
     if (P->graph_stream != stream()) {
-        for (cudaGraphExec_t *g : {&P->graph, &P->graph_steps}) {
-            if (*g) cudaGraphExecDestroy(*g);
-            *g = nullptr;
-        }
+        problem_drop_graph(&P->graph);
+        problem_drop_graph(&P->graph_steps);
     }
     // a given number of iterations: sem_ax_dw.cuh, where the table names the
     // fixed-point operator and the factors are within range

@@ -194,6 +194,10 @@ int prepare_f64_variant(Problem *P);          // whatever the tuned FP64 variant
 int launch_lines32(const Problem *P, const float *x, float *y, int gprec, bool cg, int epb, bool staged);
 bool lines_epb_ok(int nq, int epb, size_t elem_bytes, int g_stage_bytes = 0);
 void problem_drop_graphs(Problem *P);                     // sem_setup.cu
+inline void problem_drop_graph(cudaGraphExec_t *g) {
+    if (*g) cudaGraphExecDestroy(*g);
+    *g = nullptr;
+}
 
 // ---- runtime services (sem_api.cu) ---------------------------------------
 void *dev_alloc(size_t bytes);               // nullptr on failure (error set)

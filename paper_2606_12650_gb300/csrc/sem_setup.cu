@@ -448,21 +448,14 @@ int problem_maps(Problem *P) {
 // Drops the captured CG graphs (they hold the operator variant chosen at
 // capture time); the next solve captures them again.
 void problem_drop_graphs(Problem *P) {
-    if (P->graph) cudaGraphExecDestroy(P->graph);
-    if (P->graph_steps) cudaGraphExecDestroy(P->graph_steps);
-    if (P->graph_pcg) cudaGraphExecDestroy(P->graph_pcg);
-    for (auto &g : P->graph32)
-        if (g) cudaGraphExecDestroy(g);
-    P->graph = P->graph_steps = P->graph_pcg = nullptr;
-    P->graph32[0] = P->graph32[1] = nullptr;
+    for (cudaGraphExec_t *g : {&P->graph, &P->graph_steps, &P->graph_pcg, &P->graph32[0], &P->graph32[1]})
+        problem_drop_graph(g);
     P->graph_epoch = tune_epoch();
 }
 
 void problem_destroy(Problem *P) {
     if (!P) return;
-    if (P->graph) cudaGraphExecDestroy(P->graph);
-    if (P->graph_steps) cudaGraphExecDestroy(P->graph_steps);
-    if (P->graph_pcg) cudaGraphExecDestroy(P->graph_pcg);
+    for (cudaGraphExec_t *g : {&P->graph, &P->graph_steps, &P->graph_pcg}) problem_drop_graph(g);
     if (P->dinv) dev_free(P->dinv);
     if (P->bad_dev) dev_free(P->bad_dev);
     mixed_release(P);
